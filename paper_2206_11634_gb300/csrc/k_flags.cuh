@@ -240,16 +240,40 @@ __global__ void k_init(Params P, S *f) {
     }
 }
 
-// Stored populations -> FP64 [Q][N] (and back).
+// FP32 to FP64, and FP64 to FP32 rounded to nearest even, without the FP64
+// pipe (a conversion there holds its sub-partition for 64 cycles a warp, as
+// any FP64 instruction): the same bits as the casts, which take the values
+// outside FP32's normal range.
+__device__ __forceinline__ double to_double(double v) { return v; }
+__device__ __forceinline__ double to_double(float v) {
+    const uint32_t b = __float_as_uint(v), e = (b >> 23) & 255u;
+    if (e == 0u || e == 255u) return (double)v;
+    const unsigned long long m = ((unsigned long long)(b & 0x7fffffffu) + (896ull << 23)) << 29;
+    return __longlong_as_double((long long)(m | ((unsigned long long)(b & 0x80000000u) << 32)));
+}
+template <typename C> __device__ __forceinline__ C from_double(double v);
+template <> __device__ __forceinline__ double from_double<double>(double v) { return v; }
+template <> __device__ __forceinline__ float from_double<float>(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const uint32_t hi = (uint32_t)(b >> 32), e = (hi >> 20) & 2047u;
+    if (e < 897u || e > 1149u) return (float)v;  // not certain to round to a normal FP32 value
+    const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+    return __uint_as_float((hi & 0x80000000u) | (((uint32_t)(r >> 29) - (896u << 23)) & 0x7fffffffu));
+}
+
+// Stored populations -> FP64 [Q][N] (and back).  Bound by HBM once the
+// conversions leave the FP64 pipe: 256^3 FP32, 3.83 GB: get 0.81 -> 0.64 ms, set
+// 0.72 -> 0.59 ms (6.0 and 6.5 TB/s).
 template <typename S, int Q>
 __global__ void k_get_pop(Params P, const S *f, double *out) {
     using L = Lat<Q>;
     using C = typename Codec<S>::C;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < P.N; n += (long long)gridDim.x * blockDim.x) {
+        C v[Q];  // every load before the stores, which might alias them
 #pragma unroll
-        for (int i = 0; i < Q; i++)
-            out[(long long)i * P.N + n] =
-                (double)Codec<S>::ldf(f + (long long)i * P.N + n, (C)L::w(i), (C)P.rho0);
+        for (int i = 0; i < Q; i++) v[i] = Codec<S>::ldf(f + (long long)i * P.N + n, (C)L::w(i), (C)P.rho0);
+#pragma unroll
+        for (int i = 0; i < Q; i++) out[(long long)i * P.N + n] = to_double(v[i]);
     }
 }
 template <typename S, int Q>
@@ -257,40 +281,178 @@ __global__ void k_set_pop(Params P, S *f, const double *in) {
     using L = Lat<Q>;
     using C = typename Codec<S>::C;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < P.N; n += (long long)gridDim.x * blockDim.x) {
+        double v[Q];
+#pragma unroll
+        for (int i = 0; i < Q; i++) v[i] = in[(long long)i * P.N + n];
 #pragma unroll
         for (int i = 0; i < Q; i++)
-            Codec<S>::stf(f + (long long)i * P.N + n, (C)in[(long long)i * P.N + n], (C)L::w(i), (C)P.rho0);
+            Codec<S>::stf(f + (long long)i * P.N + n, from_double<C>(v[i]), (C)L::w(i), (C)P.rho0);
     }
 }
 
+// ---------------------------------------------------------------------------
 // Macroscopic fields of the stored populations: rho = sum f, u = (sum f e -
-// F/2)/rho (the velocity of the collision that produced them).
+// F/2)/rho (the velocity of the collision that produced them), in FP64.
+//
+// An FP64 warp instruction, conversions to and from FP64 included, holds its
+// sub-partition for 64 cycles on this GPU (0.5 cycles per node and SM), while
+// a node's memory traffic (FP32 D3Q19: 76 B in, 34 B out) takes 5.2 of those
+// cycles.  The sums as FP64 additions of converted values (about 130 FP64
+// instructions a node) took 3.77 ms at 256^3.  So below FP64 storage the sums
+// run in FP32, exactly, and nine FP64 instructions are left: the density's sum
+// with rho0 and the division.  Measured at 256^3, FP32, the call: 3.77 ->
+// 0.56 ms (one 64-bit integer per value instead of the three FP32 parts
+// below: 0.87).
+//
+// Exact sums: with 2^(E - 126) above the node's largest magnitude, adding and
+// taking off 1.5 2^23 u rounds a value to a multiple of u, so a value splits
+// exactly into a multiple of u1 = 2^(E - 145) (at most 2^19 of them), one of
+// u2 = 2^-20 u1 (at most 2^19) and a rest of at most u2 / 2 (Rump, Ogita and
+// Oishi's extraction, SIAM J. Sci. Comput. 31, 2008).  Q <= 19 such multiples
+// add up exactly in FP32 in any order; the rests' sum is off by 2^-24 of
+// itself at most, under 2^-60 of the largest value.
+// ---------------------------------------------------------------------------
+constexpr int kFieldEmin = 56, kFieldEmax = 240;  // the exponent fields E that the units stay normal for
+__device__ __forceinline__ float exp2_field(int e) { return __uint_as_float((uint32_t)e << 23); }  // 2^(e - 127)
+
+// a 2^e2 rounded to nearest even (|a| < 2^63, the result in FP64's normal
+// range), without the FP64 pipe.
+__device__ __forceinline__ double fixed_double(long long a, int e2) {
+    if (a == 0) return 0.0;
+    const unsigned long long mag = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+    const int lz = __clzll((long long)mag);
+    const unsigned long long n = mag << lz;  // bit 63 set
+    unsigned long long m = n >> 11;          // 53 bits, the leading one included
+    const uint32_t rem = (uint32_t)n & 0x7ffu;
+    m += (rem > 0x400u || (rem == 0x400u && ((uint32_t)m & 1u))) ? 1ull : 0ull;
+    const unsigned long long bits = ((unsigned long long)(1023 + 63 - lz + e2 - 1) << 52) + m;
+    return __longlong_as_double((long long)(bits | (a < 0 ? 0x8000000000000000ull : 0ull)));
+}
+// FP64 to FP32 by truncation, for magnitudes within FP32's normal range.
+__device__ __forceinline__ float trunc_float(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const uint32_t hi = (uint32_t)(b >> 32);
+    return __uint_as_float((hi & 0x80000000u) | (((uint32_t)(b >> 29) - (896u << 23)) & 0x7fffffffu));
+}
+
+// Exponent field of an FP64 value (0 for zero): comparisons by it do not go
+// through the FP64 pipe, as FP64 ones do.
+__device__ __forceinline__ uint32_t exponent64(double v) {
+    return ((uint32_t)((unsigned long long)__double_as_longlong(v) >> 32) >> 20) & 2047u;
+}
+
+// a u1 + b u2 + c as FP64, rounded once; c to the nearest u3 = 2^-17 u2
+__device__ __forceinline__ double field_sum(float a, float b, float c, int E) {
+    const int ia = __float2int_rn(a * exp2_field(272 - E));
+    const int ib = __float2int_rn(b * exp2_field(292 - E));
+    const int ic = __float2int_rn(c * exp2_field(309 - E));
+    return fixed_double((long long)ia * (1ll << 37) + ((long long)ib * (1ll << 17) + ic), E - 182);
+}
+
+// Density and momentum (sum g e - F/2) of a node's FP32 offsets, E their
+// largest exponent field.
+template <int Q>
+__device__ __forceinline__ void field_moments(const Params &P, float (&g)[Q], int E, double &r, double m[3]) {
+    using L = Lat<Q>;
+    float s[3], x[3], y[3], z[3];
+#pragma unroll
+    for (int p = 0; p < 3; p++) {
+        // parts 0 and 1: the multiples of u1 and u2; part 2: what is left
+        const float big = 1.5f * exp2_field(E - (p == 0 ? 145 : 165) + 127 + 23);
+        s[p] = x[p] = y[p] = z[p] = 0.f;
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            float t = g[i];
+            if (p < 2) {
+                t = __fsub_rn(__fadd_rn(big, g[i]), big);
+                g[i] = __fsub_rn(g[i], t);
+            }
+            s[p] = __fadd_rn(s[p], t);
+            if (L::e(i, 0)) x[p] = __fadd_rn(x[p], L::e(i, 0) > 0 ? t : -t);
+            if (L::e(i, 1)) y[p] = __fadd_rn(y[p], L::e(i, 1) > 0 ? t : -t);
+            if (L::e(i, 2)) z[p] = __fadd_rn(z[p], L::e(i, 2) > 0 ? t : -t);
+        }
+    }
+    r = P.rho0 + field_sum(s[0], s[1], s[2], E);
+    m[0] = field_sum(x[0], x[1], x[2], E);
+    m[1] = field_sum(y[0], y[1], y[2], E);
+    m[2] = field_sum(z[0], z[1], z[2], E);
+    for (int a = 0; a < 3; a++)
+        if (exponent64(P.F[a])) m[a] -= 0.5 * P.F[a];
+}
+
+// u = m / r: an FP32 quotient, its FP64 residual, and the residual's share by
+// 1/r to 2^-43 (one Newton step from the FP32 reciprocal): within 0.51 ulp of
+// the quotient.  Two FP64 instructions a component and two for 1/r; operands
+// outside the range that the FP32 steps hold are divided.
+__device__ __forceinline__ void field_velocity(double r, const double m[3], double u[3]) {
+    // 2^-50 <= r < 2^50
+    const bool mid = exponent64(r) - 973u < 100u && (__double_as_longlong(r) >> 63) == 0;
+    const float r0 = __frcp_rn(mid ? trunc_float(r) : 1.0f);
+    const double r0d = to_double(r0);
+    const double r1 = fma(r0d, fma(-r, r0d, 1.0), r0d);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const uint32_t e = exponent64(m[a]);
+        if (e == 0u && mid) {
+            u[a] = 0.0;  // m is zero (sums and forces of normal values)
+        } else if (e - 957u < 130u && mid) {  // 2^-66 <= |m| < 2^64
+            const double q = to_double(trunc_float(m[a]) * r0);
+            u[a] = fma(fma(-q, r, m[a]), r1, q);
+        } else {
+            u[a] = m[a] / r;
+        }
+    }
+}
+
 template <typename S, int Q>
-__global__ void k_fields(Params P, const S *f, const uint16_t *flags, double *rho, double *u, uint16_t *fl_out) {
+__global__ void __launch_bounds__(256, 4) k_fields(Params P, const S *f, const uint16_t *flags, double *rho, double *u,
+                                                uint16_t *fl_out) {
     using L = Lat<Q>;
     using C = typename Codec<S>::C;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < P.N; n += (long long)gridDim.x * blockDim.x) {
         const uint16_t fl = flags[n];
-        if (fl_out) fl_out[n] = fl;
-        double r = 0, mx = 0, my = 0, mz = 0;
-        if (fl == 0) {
-            // offsets: rho = rho0 + sum g, momentum = sum g e
+        double r = 0, m[3] = {0, 0, 0}, uu[3] = {0, 0, 0};
+        if (rho || u) {
+            // the loads do not wait for the flag
+            C g[Q];
 #pragma unroll
-            for (int i = 0; i < Q; i++) {
-                const double gi = (double)Codec<S>::ld_plain(f + (long long)i * P.N + n, (C)L::w(i), (C)P.rho0);
-                r += gi;
-                mx += gi * L::e(i, 0);
-                my += gi * L::e(i, 1);
-                mz += gi * L::e(i, 2);
+            for (int i = 0; i < Q; i++) g[i] = Codec<S>::ld_plain(f + (long long)i * P.N + n, (C)L::w(i), (C)P.rho0);
+            if (fl == 0) {
+                bool done = false;
+                if constexpr (sizeof(C) == 4) {
+                    uint32_t top = 0;
+#pragma unroll
+                    for (int i = 0; i < Q; i++) top = max(top, __float_as_uint(g[i]) & 0x7fffffffu);
+                    const int E = top ? (int)(top >> 23) : kFieldEmin;
+                    if (E >= kFieldEmin && E <= kFieldEmax) {
+                        field_moments<Q>(P, g, E, r, m);
+                        field_velocity(r, m, uu);
+                        done = true;
+                    }
+                }
+                if (!done) {  // FP64 storage, or offsets outside the range above (not finite, too)
+#pragma unroll
+                    for (int i = 0; i < Q; i++) {
+                        const double gi = (double)g[i];
+                        r += gi;
+                        m[0] += gi * L::e(i, 0);
+                        m[1] += gi * L::e(i, 1);
+                        m[2] += gi * L::e(i, 2);
+                    }
+                    r += P.rho0;
+                    uu[0] = (m[0] - 0.5 * P.F[0]) / r;
+                    uu[1] = (m[1] - 0.5 * P.F[1]) / r;
+                    uu[2] = (m[2] - 0.5 * P.F[2]) / r;
+                }
             }
-            r += P.rho0;
         }
+        if (fl_out) fl_out[n] = fl;
         if (rho) rho[n] = r;
         if (u) {
-            const bool ok = fl == 0;
-            u[n] = ok ? (mx - 0.5 * P.F[0]) / r : 0.0;
-            u[P.N + n] = ok ? (my - 0.5 * P.F[1]) / r : 0.0;
-            u[2 * P.N + n] = ok ? (mz - 0.5 * P.F[2]) / r : 0.0;
+            u[n] = uu[0];
+            u[P.N + n] = uu[1];
+            u[2 * P.N + n] = uu[2];
         }
     }
 }
