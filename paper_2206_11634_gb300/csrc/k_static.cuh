@@ -164,28 +164,47 @@ __device__ __forceinline__ void static_plain_node(const Params &P, int n) {
     plain_pull<S, Q, true>(P, x, y, z, n, fin);
     if (!skip) collide_store<S, Q, kForce, true>(P, fin, (S *)P.fB, P.N, n);
 }
+// Step t's link kernel, then its plain kernel, then step t + 1's, all on one
+// stream as programmatic dependent launches: a kernel's CTAs come up while
+// the one before still runs.  The link kernel waits for the whole of step
+// t - 1 before it lets the plain kernel start, so that one reads nothing
+// unfinished and runs beside it on other nodes; it waits for the link kernel
+// only at its end, so its own completion stands for the whole step.  On two
+// streams with events between them, and a memset a step, a step of the 48^3
+// drag box took 22.6 us, most of it gaps; this way 7.6.
+//
+// The last CTA clears the step counters and force totals of the next step's
+// region (the binning, which clears it otherwise, does not run here); they
+// are those of step t - 1, whose kernels are done.
 template <typename S, int Q, bool kForce>
 __global__ void __launch_bounds__(BRICK, 4) k_static_plain(Params P) {
+    pdl_launch_dependents();
+    if (blockIdx.x == gridDim.x - 1) {
+        int *tail = static_cast<int *>(P.bin_next) + P.nbricks;
+        const int words = (int)(P.bin_next_bytes / 4) - P.nbricks;
+        for (int k = threadIdx.x; k < words; k += BRICK) tail[k] = 0;
+    }
     static_plain_node<S, Q, kForce>(P, blockIdx.x * BRICK + (int)threadIdx.x);
+    pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
-// link nodes: one warp per kStaticNodesPerWarp listed link nodes
+// link nodes: one warp per kPer listed link nodes
 // ---------------------------------------------------------------------------
-constexpr int kStaticSlots = 4;  // particles per warp with shared-memory force sums
+// A warp's links in a queue (lane order, then direction order): the lane's
+// node and direction, then the link's result.
 struct StaticScratch {
     unsigned short entry[BRICK / 32][kLinkQueue];  // (lane << 5) | direction
     int rec[BRICK / 32][kLinkQueue];               // link record, then (as float bits) its result
     int node[BRICK / 32][32];                      // node index of each lane
-    int ids[BRICK / 32][kStaticSlots];
-    unsigned long long fix[BRICK / 32][kStaticSlots][6];
 };
 
-// One link of node n (direction i, record r): the node's own populations and
-// x_ff's fetched in one round, the unknown and the momentum exchange with the
-// recorded geometry; the force/torque terms go to the warp's table.
+// One link of node n (direction i, record r): the node's own populations,
+// x_ff's and the record fetched in one round, the unknown and the momentum
+// exchange with the recorded geometry; the force/torque terms in fixed point.
+// Coherent loads: the kernel is up before the step before has written them.
 template <typename S, int Q>
-__device__ __noinline__ float static_link(const Params &P, StaticScratch &ss, int warp, int n, int i, int r) {
+__device__ __forceinline__ float static_link(const Params &P, int n, int i, int r, int &j, LinkTerms &lt) {
     using L = Lat<Q>;
     using Cd = Codec<S>;
     using C = typename Cd::C;
@@ -197,29 +216,28 @@ __device__ __noinline__ float static_link(const Params &P, StaticScratch &ss, in
     const int z = n / nxy, rr = n - z * nxy;
     const int y = rr / P.nx, x = rr - y * P.nx;
     const int io = L::opp(i);
-    const bool ok = rec.jf < 0;  // bit 31
-    // x_ff = x - d = x + e_i (inside the box when ok)
+    // x_ff = x - d = x + e_i; beyond a wall the wrapped node is read and its
+    // values are not used (the record says so), so no load waits for the record
     int fx = x + lat_e<Q>(i, 0), fy = y + lat_e<Q>(i, 1), fz = z + lat_e<Q>(i, 2);
     if (fx < 0) fx += P.nx; else if (fx >= P.nx) fx -= P.nx;
     if (fy < 0) fy += P.ny; else if (fy >= P.ny) fy -= P.ny;
     if (fz < 0) fz += P.nz; else if (fz >= P.nz) fz -= P.nz;
-    const int nff = ok ? fx + P.nx * (fy + P.ny * fz) : n;
+    const int nff = fx + P.nx * (fy + P.ny * fz);
     FFData<C> ff;
     ff.drho = 0;
     ff.m[0] = ff.m[1] = ff.m[2] = 0;
     ff.g_io = 0;
-    ff.ok = ok;
     C fown_io = 0, drho_f = 0, m_f[3] = {0, 0, 0};
 #pragma unroll
     for (int k = 0; k < Q; k++) {
-        const C fk = Cd::ld(A + (long long)k * N + n, (C)L::w(k), rho0);
+        const C fk = Cd::ld_plain(A + (long long)k * N + n, (C)L::w(k), rho0);
         drho_f += fk;
         m_f[0] += fk * L::e(k, 0);
         m_f[1] += fk * L::e(k, 1);
         m_f[2] += fk * L::e(k, 2);
         if (k == io) fown_io = fk;
-        if (P.vibb && ok) {
-            const C gk = Cd::ld(A + (long long)k * N + nff, (C)L::w(k), rho0);
+        if (P.vibb) {
+            const C gk = Cd::ld_plain(A + (long long)k * N + nff, (C)L::w(k), rho0);
             ff.drho += gk;
             ff.m[0] += gk * L::e(k, 0);
             ff.m[1] += gk * L::e(k, 1);
@@ -227,6 +245,7 @@ __device__ __noinline__ float static_link(const Params &P, StaticScratch &ss, in
             if (k == io) ff.g_io = gk;
         }
     }
+    ff.ok = rec.jf < 0;  // bit 31
     C u_f[3];
     const C inv_rho_f = rcp_w<C>(rho0 + drho_f);  // as the near sweep's link_coop
     for (int a = 0; a < 3; a++) u_f[a] = (m_f[a] - C(0.5) * Prm<C>::F(P, a)) * inv_rho_f;
@@ -240,26 +259,40 @@ __device__ __noinline__ float static_link(const Params &P, StaticScratch &ss, in
     const C fin = link_update<S, Q>(P, i, g, ff, fown_io, drho_f, u_f, dP);
     C t[6];
     force_terms<C>(dP, g.r, t);
-    const int j = rec.jf & 0xFFFF;
-    int slot = -1;
-    for (int k = 0; k < kStaticSlots && slot < 0; k++) {
-        const int id = ss.ids[warp][k];
-        if (id == j) {
-            slot = k;
-        } else if (id < 0) {
-            const int old = atomicCAS(&ss.ids[warp][k], -1, j);
-            if (old == -1 || old == j) slot = k;
-        }
-    }
-    for (int c = 0; c < 6; c++) {
-        if (t[c] == C(0)) continue;
-        if (slot >= 0) atomicAdd(&ss.fix[warp][slot][c], to_fixed<C>(t[c]));
-        else atomicAdd(&P.Ffix[j * 6 + c], to_fixed<C>(t[c]));
-    }
+    j = rec.jf & 0xFFFF;
+    lt.s = j;
+#pragma unroll
+    for (int c = 0; c < 6; c++) lt.t[c] = (long long)to_fixed<C>(t[c]);
     return (float)fin;
 }
 
-template <typename S, int Q, bool kForce>
+// The warp's link terms of one round added to the particles' totals: per
+// particle met, the exact 64-bit sums over the warp by 32-bit reductions (as
+// warp_add_terms) and one atomic each.  (Shared-memory atomics per link, 64
+// bits wide, are compare-and-swap loops: they took most of the link kernel.)
+__device__ __forceinline__ void static_add_terms(const Params &P, const LinkTerms &lt, int lane) {
+    unsigned todo = __ballot_sync(0xffffffffu, lt.s >= 0);
+    while (todo) {
+        const int j = __shfl_sync(0xffffffffu, lt.s, __ffs(todo) - 1);
+        const bool mine = lt.s == j;
+        todo &= ~__ballot_sync(0xffffffffu, mine);
+        unsigned long long out = 0;
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            const long long v = mine ? lt.t[c] : 0ll;
+            const unsigned lo = (unsigned)v & 0x1FFFFFu, mid = (unsigned)(v >> 21) & 0x1FFFFFu;
+            const int hi = (int)(v >> 42);
+            const unsigned long long sum =
+                (unsigned long long)__reduce_add_sync(0xffffffffu, lo) +
+                ((unsigned long long)__reduce_add_sync(0xffffffffu, mid) << 21) +
+                ((unsigned long long)(long long)__reduce_add_sync(0xffffffffu, hi) << 42);
+            if (lane == c) out = sum;
+        }
+        if (lane < 6 && out) atomicAdd(&P.Ffix[j * 6 + lane], out);
+    }
+}
+
+template <typename S, int Q, bool kForce, int kPer>
 __device__ __forceinline__ void static_links_warp(const Params &P, StaticScratch &ss, int wg) {
     using L = Lat<Q>;
     using Cd = Codec<S>;
@@ -269,15 +302,14 @@ __device__ __forceinline__ void static_links_warp(const Params &P, StaticScratch
     S *B = (S *)P.fB;
     const long long N = P.N;
     const C rho0 = Prm<C>::rho0(P);
-    if (lane < kStaticSlots) ss.ids[warp][lane] = -1;
-    for (int e = lane; e < kStaticSlots * 6; e += 32) ss.fix[warp][e / 6][e % 6] = 0ull;
-    const int idx = wg * kStaticNodesPerWarp + lane;
-    const bool has = lane < kStaticNodesPerWarp && idx < P.snodes_n;
+    const int idx = wg * kPer + lane;
+    const bool has = lane < kPer && idx < P.snodes_n;
     StaticNode sn;
     sn.n = 0;
     sn.mask = 0u;
     sn.base = 0;
     if (has) sn = P.snodes[idx];
+    __syncwarp();  // the previous round of the warp is done with its queue
     ss.node[warp][lane] = sn.n;
     const uint32_t links = sn.mask;
     const int mine = __popc(links);
@@ -299,10 +331,17 @@ __device__ __forceinline__ void static_links_warp(const Params &P, StaticScratch
         }
     }
     __syncwarp();
-    for (int e = lane; e < total; e += 32) {
-        const int ent = ss.entry[warp][e];
-        ss.rec[warp][e] =
-            __float_as_int(static_link<S, Q>(P, ss, warp, ss.node[warp][ent >> 5], ent & 31, ss.rec[warp][e]));
+    for (int r = 0; r < total; r += 32) {
+        const int e = r + lane;
+        LinkTerms lt;
+        lt.s = -1;
+        if (e < total) {
+            const int ent = ss.entry[warp][e];
+            int j;
+            ss.rec[warp][e] =
+                __float_as_int(static_link<S, Q>(P, ss.node[warp][ent >> 5], ent & 31, ss.rec[warp][e], j, lt));
+        }
+        static_add_terms(P, lt, lane);
     }
     __syncwarp();
     if (has) {
@@ -324,35 +363,31 @@ __device__ __forceinline__ void static_links_warp(const Params &P, StaticScratch
                 const bool wall = (sx | sy | sz) < 0;
                 const S *ptr = wall ? A + (long long)L::opp(i) * N + n
                                     : A + (long long)i * N + (sx + P.nx * (sy + P.ny * sz));
-                fin[i] = Cd::ldv(ptr, (C)L::w(i), rho0);
+                fin[i] = Cd::ldv_s(ptr, (C)L::w(i), rho0);
             }
         }
         collide_store<S, Q, kForce>(P, fin, B, N, n);  // collide-space values
     }
-    __syncwarp();
-    for (int e = lane; e < kStaticSlots * 6; e += 32) {
-        const int id = ss.ids[warp][e / 6];
-        const unsigned long long v = ss.fix[warp][e / 6][e % 6];
-        if (id >= 0 && v) atomicAdd(&P.Ffix[id * 6 + e % 6], v);
-    }
 }
 
 // The step's constant parts: the missing-force-point totals and the link
-// count (one thread).
-__device__ __forceinline__ void static_constants(const Params &P) {
-    for (int k = 0; k < P.np * 6; k++)
+// count (threads t of nt).
+__device__ __forceinline__ void static_constants(const Params &P, int t, int nt) {
+    for (int k = t; k < P.np * 6; k += nt)
         if (P.smf[k]) atomicAdd(&P.Ffix[k], P.smf[k]);
-    atomicAdd(&P.counters[CNT_NLINKS], P.scount[1]);
+    if (t == 0) atomicAdd(&P.counters[CNT_NLINKS], P.scount[1]);
 }
 
-template <typename S, int Q, bool kForce>
+template <typename S, int Q, bool kForce, int kPer>
 __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links(Params P) {
     if (sizeof(typename Codec<S>::C) == 8) return;
     __shared__ StaticScratch ss;
-    if (blockIdx.x == 0 && threadIdx.x == 0) static_constants(P);
-    const int warps = (P.snodes_n + kStaticNodesPerWarp - 1) / kStaticNodesPerWarp;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (blockIdx.x == gridDim.x - 1) static_constants(P, threadIdx.x, BRICK);
+    const int warps = (P.snodes_n + kPer - 1) / kPer;
     for (int wg = blockIdx.x * (BRICK / 32) + (threadIdx.x >> 5); wg < warps; wg += gridDim.x * (BRICK / 32))
-        static_links_warp<S, Q, kForce>(P, ss, wg);
+        static_links_warp<S, Q, kForce, kPer>(P, ss, wg);
 }
 
 // ---------------------------------------------------------------------------
@@ -417,8 +452,8 @@ __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links_batch(Ba
         }
         const Params &P = row[lo];
         const int wl = gw - B.swarp_off[lo];
-        if (wl == 0 && (threadIdx.x & 31) == 0) static_constants(P);
-        if (wl * kStaticNodesPerWarp < P.snodes_n) static_links_warp<S, Q, kForce>(P, ss, wl);
+        if (wl == 0) static_constants(P, threadIdx.x & 31, 32);
+        if (wl * kStaticNodesPerWarp < P.snodes_n) static_links_warp<S, Q, kForce, kStaticNodesPerWarp>(P, ss, wl);
     }
     advance_step_when_last(B.ctr + 2, B.ctr);
 }

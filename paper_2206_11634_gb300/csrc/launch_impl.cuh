@@ -136,27 +136,33 @@ void launch_static_plain_t(const Params &P, cudaStream_t st) {
     const bool force = P.F[0] != 0.0 || P.F[1] != 0.0 || P.F[2] != 0.0;
     const int grid = (int)((P.N + BRICK - 1) / BRICK);
     if (P.Q == 19) {
-        if (force) k_static_plain<S, 19, true><<<grid, BRICK, 0, st>>>(P);
-        else k_static_plain<S, 19, false><<<grid, BRICK, 0, st>>>(P);
+        if (force) launch_pdl(k_static_plain<S, 19, true>, grid, BRICK, st, P);
+        else launch_pdl(k_static_plain<S, 19, false>, grid, BRICK, st, P);
     } else {
-        if (force) k_static_plain<S, 15, true><<<grid, BRICK, 0, st>>>(P);
-        else k_static_plain<S, 15, false><<<grid, BRICK, 0, st>>>(P);
+        if (force) launch_pdl(k_static_plain<S, 15, true>, grid, BRICK, st, P);
+        else launch_pdl(k_static_plain<S, 15, false>, grid, BRICK, st, P);
     }
 }
-template <typename S>
-void launch_static_links_t(const Params &P, cudaStream_t st) {
+template <typename S, int kPer>
+void launch_static_links_per(const Params &P, cudaStream_t st) {
     const bool force = P.F[0] != 0.0 || P.F[1] != 0.0 || P.F[2] != 0.0;
-    const int warps = (P.snodes_n + kStaticNodesPerWarp - 1) / kStaticNodesPerWarp;
+    const int warps = (P.snodes_n + kPer - 1) / kPer;
     const int cap = kNearCtasPerSm * sm_count();
     int grid = (warps + BRICK / 32 - 1) / (BRICK / 32);
     grid = grid < 1 ? 1 : (grid > cap ? cap : grid);
     if (P.Q == 19) {
-        if (force) k_static_links<S, 19, true><<<grid, BRICK, 0, st>>>(P);
-        else k_static_links<S, 19, false><<<grid, BRICK, 0, st>>>(P);
+        if (force) launch_pdl(k_static_links<S, 19, true, kPer>, grid, BRICK, st, P);
+        else launch_pdl(k_static_links<S, 19, false, kPer>, grid, BRICK, st, P);
     } else {
-        if (force) k_static_links<S, 15, true><<<grid, BRICK, 0, st>>>(P);
-        else k_static_links<S, 15, false><<<grid, BRICK, 0, st>>>(P);
+        if (force) launch_pdl(k_static_links<S, 15, true, kPer>, grid, BRICK, st, P);
+        else launch_pdl(k_static_links<S, 15, false, kPer>, grid, BRICK, st, P);
     }
+}
+template <typename S>
+void launch_static_links_t(const Params &P, cudaStream_t st) {
+    const long long resident = (long long)kNearCtasPerSm * sm_count() * (BRICK / 32);  // warps at once
+    if (P.snodes_n <= resident * kStaticNodesPerWarpFew) launch_static_links_per<S, kStaticNodesPerWarpFew>(P, st);
+    else launch_static_links_per<S, kStaticNodesPerWarp>(P, st);
 }
 
 template <typename S>

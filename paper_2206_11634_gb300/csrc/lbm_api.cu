@@ -839,12 +839,14 @@ int lbm_step(lbm_handle *h, int nsteps) {
     if (!h) return fail(nullptr, LBM_ERR_BAD_ARG, "handle is NULL");
     if (nsteps < 0) return fail(h, LBM_ERR_BAD_ARG, "nsteps < 0");
     if (nsteps == 0) return LBM_OK;
-    // fork: both library streams start after everything issued so far
+    // fork: the library streams start after everything issued so far (aux
+    // with the first step that uses it: the fixed-geometry sweep does not)
     cudaError_t e = cudaEventRecord(h->ev_fork, h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->hi, h->ev_fork, 0);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->aux, h->ev_fork, 0);
     if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
     cudaStream_t hs = h->hi;
+    bool forked_aux = false;  // aux carries work of this call
+    bool plain_pending = false;  // ... that hs has not waited for
     for (int t = 0; t < nsteps; t++) {
         Params P = make_params(h);
         // with every particle fixed the flags cannot change: once both flag
@@ -896,18 +898,25 @@ int lbm_step(lbm_handle *h, int nsteps) {
             if (e != cudaSuccess) return cuda_check(h, e, "cudaMemsetAsync(bricks)");
         }
         if (fixed_sweep && h->static_state == 1) {
-            // the link nodes after the previous step's plain nodes (they read
-            // them, and overwrite the array that sweep read), the plain nodes
-            // after the previous step's link nodes, concurrently otherwise
-            if (t > 0) e = cudaStreamWaitEvent(hs, h->ev_plain, 0);
-            if (e == cudaSuccess && t > 0) e = cudaStreamWaitEvent(h->aux, h->ev_near, 0);
-            if (e != cudaSuccess) return cuda_check(h, e, "stream wait");
+            // the link nodes, then the plain nodes beside them, in stream
+            // order (k_static.cuh); behind the plain sweep of a brick step
+            if (plain_pending) {
+                e = cudaStreamWaitEvent(hs, h->ev_plain, 0);
+                if (e != cudaSuccess) return cuda_check(h, e, "stream wait");
+                plain_pending = false;
+            }
             { ProfScope s(h, 3, true, hs); by_storage<DoStaticLinks>(h->cfg.storage, P, hs); }
-            { ProfScope s(h, 2, true, h->aux); by_storage<DoStaticPlain>(h->cfg.storage, P, h->aux); }
-            e = cudaEventRecord(h->ev_plain, h->aux);
-            if (e == cudaSuccess) e = cudaEventRecord(h->ev_near, hs);
-            if (e != cudaSuccess) return cuda_check(h, e, "event record");
+            { ProfScope s(h, 2, true, hs); by_storage<DoStaticPlain>(h->cfg.storage, P, hs); }
+            // the plain kernel cleared the next region's counters and force
+            // totals (the brick counts are only written by brick steps, which
+            // do not follow before the particles are set again)
+            h->bin_clean[rp ^ 1] = 1;
         } else {
+            if (!forked_aux) {
+                e = cudaStreamWaitEvent(h->aux, h->ev_fork, 0);
+                if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
+                forked_aux = true;
+            }
             { ProfScope s(h, 0, true, hs); launch_bin(P, hs); }
             h->bin_clean[rp ^ 1] = 1;
             e = cudaEventRecord(h->ev_bin, hs);
@@ -948,6 +957,7 @@ int lbm_step(lbm_handle *h, int nsteps) {
                 e = cudaEventRecord(h->ev_plain, h->aux);
                 if (e != cudaSuccess) return cuda_check(h, e, "event record");
             }
+            plain_pending = true;
         }
         if (!P.force_fixed) { ProfScope s(h, 4, P.np > 0, hs); launch_force_reduce(P, hs); }
         { ProfScope s(h, 5, P.np > 0 && P.n_sub > 0, hs); launch_dem(P, hs, h->dem2, h->ev_dsplit, h->ev_dfree); }
@@ -963,7 +973,7 @@ int lbm_step(lbm_handle *h, int nsteps) {
     // plain sweep
     e = cudaEventRecord(h->ev_join, hs);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->ev_join, 0);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->ev_plain, 0);
+    if (e == cudaSuccess && forked_aux) e = cudaStreamWaitEvent(h->stream, h->ev_plain, 0);
     if (e != cudaSuccess) return cuda_check(h, e, "stream join");
     return LBM_OK;
 }

@@ -60,10 +60,13 @@ struct StaticLink {
     float q, r[3], uw[3];
     int jf;  // particle index in bits 0-15; bit 31: x_ff is a fluid node in the box
 };
-// Link nodes per warp of the fixed-geometry link kernel: few, so that a
-// warp's lanes evaluate its links in about one round (a link node has a few
-// links) and small cases spread over many warps.
-constexpr int kStaticNodesPerWarp = 8;
+// Link nodes per warp of the fixed-geometry link kernel.  Four (about 18
+// links, one round of a warp's lanes) while all link nodes' warps are resident
+// at once: the step then waits for one warp's latency (48^3 drag box 8.5 us a
+// step with eight, 7.6 with four; 96^3 30.1 and 26.8).  Eight (about 37 links,
+// fewer idle lanes) beyond that: the 64-box batch took 1.61 ms a step with
+// four, 1.58 with eight.
+constexpr int kStaticNodesPerWarp = 8, kStaticNodesPerWarpFew = 4;
 
 // Lattices stored below FP64 accumulate the per-particle force and torque
 // totals in 64-bit fixed point with integer atomics: exact and independent of
@@ -672,6 +675,28 @@ __device__ __forceinline__ void brick_coords(const Params &P, int b, int &bx, in
     bx = b % P.nbx;
     by = (b / P.nbx) % P.nby;
     bz = b / (P.nbx * P.nby);
+}
+
+// Programmatic dependent launch.  launch_dependents: the next kernel of the
+// stream may start once every CTA of this one has called it (or ended).
+// wait: until the kernels this one was launched behind are complete and their
+// writes visible.  Both do nothing in a kernel launched the ordinary way.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Launch that may start before the stream's previous kernel has ended (the
+// kernel itself waits, see above).
+template <typename... K, typename... A>
+inline void launch_pdl(void (*kernel)(K...), dim3 grid, int block, cudaStream_t st, const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, K(args)...);
 }
 
 // Launchers of the particle-side kernels (k_particles.cu).
