@@ -12,9 +12,10 @@
  * objective is the mean drag J = (1/W) sum_{t=T-W}^{T-1} F_x(t) over the last
  * W of T steps, starting from f^eq(rho0, u0).  The gradient is dJ/dK_i and
  * dJ/dx_i for every control point (weight K_i, world position x_i, Eq. (4)):
- * the adjoint runs backwards through the T steps, recomputing the states of
- * each segment of ceil(sqrt(T)) steps from a checkpoint kept by the forward
- * run, and accumulates dJ/dq per link, which the chain rule through Eq. (27)
+ * the adjoint runs backwards through the T steps from what the forward run
+ * kept of each (16 bytes per node and 36 per link; with more than 8 GiB of
+ * that, from a state kept every ceil(sqrt(T)) steps, running each segment
+ * forward again), and accumulates dJ/dq per link, which the chain rule through Eq. (27)
  * and Eq. (4) turns into the shape gradient.  The paper has no adjoint.
  *
  * Memory: the caller owns one device workspace (lbm_adj_workspace_size, 256-
@@ -44,8 +45,8 @@ int lbm_adj_init(const lbm_config *cfg, const lbm_particle *p, int T, int W, voi
 
 /* Forward run with control points at cp_world (host double[ncp][3], world
  * frame) with weights K (host double[ncp]), ncp as in the particle given to
- * lbm_adj_init; returns J (synchronises).  Keeps the checkpoints the
- * backward run needs. */
+ * lbm_adj_init; returns J (synchronises).  Keeps what the backward run
+ * needs. */
 int lbm_adj_forward(lbm_adj *a, const double *cp_world, const double *K, double *J);
 
 /* Gradient of the J of the last forward run: dJ_dcp host double[ncp][3],
@@ -53,7 +54,7 @@ int lbm_adj_forward(lbm_adj *a, const double *cp_world, const double *K, double 
 int lbm_adj_backward(lbm_adj *a, double *dJ_dcp, double *dJ_dK);
 
 /* Links (fluid node, direction) crossing the frozen surface, and the
- * checkpoint interval. */
+ * checkpoint interval (of a run that keeps checkpoints). */
 int lbm_adj_info(const lbm_adj *a, int *nlinks, int *checkpoint_every);
 
 int lbm_adj_destroy(lbm_adj *a);

@@ -11,26 +11,40 @@
 // cancels over the closed link set, as in the main sweep).
 //
 // Adjoint of one step, for lambda' = dJ/dg+(t+1):
-//   A1  per fluid node: recompute the pulled values, lambda_in = (dBGK/dg_in)^T
-//       lambda' (the equilibrium and forcing depend on g_in only through the
-//       density and momentum, so this is (1 - omega) lambda' + a + b.e_j),
-//       plus the drag's direct dependence on the pulled link values;
-//   A2  per fluid node y: dJ/dg+(t)_k(y) = lambda_in_k(y + e_k) (the pull,
-//       transposed) plus the halfway links' and the drag's dependence on the
-//       node's own populations.  A1 and A2 run as one kernel in push form:
-//       node n stores lambda_in_j(n) straight into dJ/dg+(t)_j(n - e_j) when
-//       n - e_j is a fluid node, and writes dJ/dg+(t) itself in the
-//       directions whose neighbour is solid (its links); every entry of a
-//       fluid node has exactly one writer, and lambda_in is kept only per
-//       link (for A3), so lambda is read and written once per step;
-//   A3  per VIBB link: the link value depends on the node's and x_ff's
-//       populations through their density, momentum and one population each,
-//       and on q: those 11 partial derivatives come from forward-mode dual
-//       numbers through the same VIBB code as the forward step, and are
-//       scattered (atomics) into dJ/dg+(t) and into dJ/dq of the link.
-// The states of each segment of ceil(sqrt(T)) steps are recomputed from the
-// forward run's checkpoint.  Finally dJ/dq goes through Eq. (27) and Eq. (4)
-// to the control points and weights (FP64).
+//   A1  per fluid node: lambda_in = (dBGK/dg_in)^T lambda' (the equilibrium
+//       and forcing depend on the pulled values g_in only through their
+//       density and momentum, so this is (1 - omega) lambda' + a + b.e_j with
+//       a and b from those four numbers), plus the drag's direct dependence
+//       on the pulled link values;
+//   A2  the pull, transposed: node n stores lambda_in_j(n) into
+//       dJ/dg+(t)_j(n - e_j) when n - e_j is a fluid node, and writes dJ/dg+(t)
+//       itself in the directions whose neighbour is solid (its links); every
+//       entry of a fluid node has exactly one writer;
+//   A3  per VIBB link: its value depends on the node's and x_ff's populations
+//       through their density, momentum and one population each, and on q.
+//       The two single populations' entries of dJ/dg+(t) are written by the
+//       link's own node (its link direction, and its push to x_ff), so their
+//       shares are added there; the density and momentum shares, (A, B) with
+//       A + B.e_k in every direction k, are summed per node beside dJ/dg+(t)
+//       and added when the next adjoint step reads it.
+//
+// What A1 and A3 need of the forward run is kept step by step: a node's four
+// moments of the pulled values (16 bytes, instead of a whole state of 76 and
+// a second gather with its link values) and nine partial derivatives per link
+// (by reverse differentiation of the VIBB value, where the value is formed).
+// Runs whose kept steps would exceed kKeepAllBytes keep a state every
+// ceil(sqrt(T)) steps instead and run each segment forward again from it.
+//
+// A step, forward or adjoint, is two kernels on disjoint nodes in programmatic
+// dependent launches (as the fixed-geometry sweep, k_static.cuh): one for the
+// fluid nodes with links, whose links are spread over a warp's lanes, and one
+// for the others, over 256-node spans.  96^3, T = 500, on a GB300: forward
+// 27 us a step (44 with the links of a node one after another in its thread),
+// adjoint 30 (113, with a recomputed forward step, a second gather and a
+// separate atomic scatter per link); 32^3: 5.6 and 5.7 (18 and 42).
+//
+// Finally dJ/dq goes through Eq. (27) and Eq. (4) to the control points and
+// weights (FP64).
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -40,7 +54,7 @@
 #include <vector>
 
 #include "lbm_adjoint.h"
-#include "lbm_internal.cuh"
+#include "k_plain.cuh"
 
 using namespace lbmmb;
 
@@ -52,163 +66,147 @@ constexpr size_t kAlign = 256;
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 // ---------------------------------------------------------------------------
-// forward-mode dual numbers with N tangents
-// ---------------------------------------------------------------------------
-template <int N>
-struct Dual {
-    float v;
-    float d[N];
-};
-template <int N>
-__device__ __forceinline__ Dual<N> dconst(float x) {
-    Dual<N> r;
-    r.v = x;
-#pragma unroll
-    for (int k = 0; k < N; k++) r.d[k] = 0.f;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> dvar(float x, int k) {
-    Dual<N> r = dconst<N>(x);
-    r.d[k] = 1.f;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator+(Dual<N> a, Dual<N> b) {
-    Dual<N> r;
-    r.v = a.v + b.v;
-#pragma unroll
-    for (int k = 0; k < N; k++) r.d[k] = a.d[k] + b.d[k];
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator-(Dual<N> a, Dual<N> b) {
-    Dual<N> r;
-    r.v = a.v - b.v;
-#pragma unroll
-    for (int k = 0; k < N; k++) r.d[k] = a.d[k] - b.d[k];
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator*(Dual<N> a, Dual<N> b) {
-    Dual<N> r;
-    r.v = a.v * b.v;
-#pragma unroll
-    for (int k = 0; k < N; k++) r.d[k] = a.d[k] * b.v + a.v * b.d[k];
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator/(Dual<N> a, Dual<N> b) {
-    Dual<N> r;
-    const float ib = 1.0f / b.v;
-    r.v = a.v * ib;
-#pragma unroll
-    for (int k = 0; k < N; k++) r.d[k] = (a.d[k] - r.v * b.d[k]) * ib;
-    return r;
-}
-template <int N> __device__ __forceinline__ Dual<N> operator+(Dual<N> a, float b) { return a + dconst<N>(b); }
-template <int N> __device__ __forceinline__ Dual<N> operator+(float a, Dual<N> b) { return dconst<N>(a) + b; }
-template <int N> __device__ __forceinline__ Dual<N> operator-(Dual<N> a, float b) { return a - dconst<N>(b); }
-template <int N> __device__ __forceinline__ Dual<N> operator-(float a, Dual<N> b) { return dconst<N>(a) - b; }
-template <int N>
-__device__ __forceinline__ Dual<N> operator*(Dual<N> a, float b) {
-    Dual<N> r;
-    r.v = a.v * b;
-#pragma unroll
-    for (int k = 0; k < N; k++) r.d[k] = a.d[k] * b;
-    return r;
-}
-template <int N> __device__ __forceinline__ Dual<N> operator*(float a, Dual<N> b) { return b * a; }
-template <int N> __device__ __forceinline__ Dual<N> operator/(float a, Dual<N> b) { return dconst<N>(a) / b; }
-__device__ __forceinline__ float val(float x) { return x; }
-template <int N> __device__ __forceinline__ float val(const Dual<N> &x) { return x.v; }
-
-// ---------------------------------------------------------------------------
-// the pieces of the step, generic in the scalar type
+// the pieces of the step
 // ---------------------------------------------------------------------------
 struct AdjConst {
     int nx, ny, nz;
     long long N;
+    FastDiv by_nxy, by_nx;
     float rho0, omega, gfac;
-    float F[3];
+    float F[3], Fg[3];  // body force, and gfac times it
 };
 
 // f^eq_i - w_i rho0 for density rho = rho0 + drho, velocity u (Eq. (16))
-template <typename T>
-__device__ __forceinline__ T geq_t(int ex, int ey, int ez, float w, T drho, T rho, T ux, T uy, T uz) {
-    const T eu = ux * (float)ex + uy * (float)ey + uz * (float)ez;
-    const T uu = ux * ux + uy * uy + uz * uz;
+__device__ __forceinline__ float geq_f(float ex, float ey, float ez, float w, float drho, float rho, float ux, float uy,
+                                       float uz) {
+    const float eu = ux * ex + uy * ey + uz * ez;
+    const float uu = ux * ux + uy * uy + uz * uz;
     return (drho + rho * (eu * 3.0f + eu * eu * 4.5f - uu * 1.5f)) * w;
 }
-
-// The VIBB unknown of a link whose direction into the solid is d (index io),
-// u_w = 0 (a fixed particle), from the moments and the io population of the
-// fluid node x_f (post-collision: u = (m - F/2)/rho) and of x_ff.
-template <typename T>
-__device__ __forceinline__ T vibb_t(const AdjConst &A, int io, T q, T drf, T mfx, T mfy, T mfz, T gf, T drff, T mffx,
-                                    T mffy, T mffz, T gff) {
-    // io is a run-time index: packed lattice entries, no table in local memory
-    const int dx = lat_e<19>(io, 0), dy = lat_e<19>(io, 1), dz = lat_e<19>(io, 2);
-    const float w = (float)lat_w<19>(io);
-    const T rf = drf + A.rho0, rff = drff + A.rho0;
-    const T irf = 1.0f / rf, irff = 1.0f / rff;
-    const T ufx = (mfx - 0.5f * A.F[0]) * irf, ufy = (mfy - 0.5f * A.F[1]) * irf, ufz = (mfz - 0.5f * A.F[2]) * irf;
-    const T uffx = (mffx - 0.5f * A.F[0]) * irff, uffy = (mffy - 0.5f * A.F[1]) * irff,
-            uffz = (mffz - 0.5f * A.F[2]) * irff;
-    const T geqf = geq_t<T>(dx, dy, dz, w, drf, rf, ufx, ufy, ufz);
-    const T geqff = geq_t<T>(dx, dy, dz, w, drff, rff, uffx, uffy, uffz);
-    const T q2 = q * 2.0f, one_m2q = 1.0f - q2;
-    const T fneq = q2 * (gf - geqf) + one_m2q * (gff - geqff);                 // Eq. (21)
-    T drd, usx, usy, usz;
-    if (val(q) <= 0.5f) {                                                       // Eqs. (22)-(23)
-        drd = q2 * drf + one_m2q * drff;
-        usx = q2 * ufx + one_m2q * uffx;
-        usy = q2 * ufy + one_m2q * uffy;
-        usz = q2 * ufz + one_m2q * uffz;
-    } else {
-        drd = drf;
-        const T a = (1.0f - q) / q;  // + (2q - 1)/q u_w, u_w = 0
-        usx = a * ufx;
-        usy = a * ufy;
-        usz = a * ufz;
-    }
-    const T b = (1.0f - q) / (1.0f + q);                                        // Eq. (24), u_w = 0
-    const T udx = (usx + 2.0f * (b * uffx)) * (1.0f / 3.0f);                   // Eq. (25)
-    const T udy = (usy + 2.0f * (b * uffy)) * (1.0f / 3.0f);
-    const T udz = (usz + 2.0f * (b * uffz)) * (1.0f / 3.0f);
-    return geq_t<T>(dx, dy, dz, w, drd, drd + A.rho0, udx, udy, udz) + fneq;  // Eqs. (20), (19)
+// its derivatives along d: dr with rho following drho, u[3]
+__device__ __forceinline__ void geq_grad(const float d[3], float w, float rho, const float u[3], float &g_dr,
+                                         float g_u[3]) {
+    const float eu = u[0] * d[0] + u[1] * d[1] + u[2] * d[2];
+    const float uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    g_dr = w * (1.0f + (eu * 3.0f + eu * eu * 4.5f - uu * 1.5f));
+    const float c = w * rho, ce = c * (3.0f + 9.0f * eu);
+#pragma unroll
+    for (int a = 0; a < 3; a++) g_u[a] = ce * d[a] - 3.0f * c * u[a];
 }
 
-// The part of the collided population i that depends on the pulled values
-// only through the density offset drho and the momentum m: omega g^eq_i +
-// Guo's term (Eq. (15) with Eq. (18)'s half-force shift).
-template <typename T>
-__device__ __forceinline__ T collide_h(const AdjConst &A, int i, T drho, T mx, T my, T mz) {
-    const int ex = L19::e(i, 0), ey = L19::e(i, 1), ez = L19::e(i, 2);
-    const float w = (float)L19::w(i);
-    const T rho = drho + A.rho0;
-    const T ir = 1.0f / rho;
-    const T ux = (mx + 0.5f * A.F[0]) * ir, uy = (my + 0.5f * A.F[1]) * ir, uz = (mz + 0.5f * A.F[2]) * ir;
-    const T eu = ux * (float)ex + uy * (float)ey + uz * (float)ez;
-    const T uF = ux * A.F[0] + uy * A.F[1] + uz * A.F[2];
-    const float eF = ex * A.F[0] + ey * A.F[1] + ez * A.F[2];
-    const T g = geq_t<T>(ex, ey, ez, w, drho, rho, ux, uy, uz) * A.omega;
-    return g + ((eF - uF) * 3.0f + eu * (9.0f * eF)) * (A.gfac * w);
+// What a link's value is formed from: the density offset, momentum and io
+// population (post-collision) of the fluid node x_f and of x_ff.
+struct LinkState {
+    float drf, mf[3], gf, drff, mff[3], gff;
+};
+// Derivatives of a link's value by those (gf: 2q, gff: 1 - 2q) and by q.
+struct LinkGrad {
+    float4 f, ff;  // by (drf, mf) and (drff, mff)
+    float q;
+};
+
+// The VIBB unknown of a link whose direction into the solid is d (index io),
+// u_w = 0 (a fixed particle): u = (m - F/2)/rho of the two nodes.  kGrad: its
+// derivatives too, by reverse differentiation (about three times the value's
+// arithmetic; forward-mode dual numbers took eleven tangents through it).
+template <bool kGrad>
+__device__ __forceinline__ float vibb_f(const AdjConst &A, int io, float q, const LinkState &s, LinkGrad &g) {
+    const float d[3] = {(float)lat_e<19>(io, 0), (float)lat_e<19>(io, 1), (float)lat_e<19>(io, 2)};
+    const float w = (float)lat_w<19>(io);
+    const float rf = s.drf + A.rho0, rff = s.drff + A.rho0;
+    const float irf = 1.0f / rf, irff = 1.0f / rff;
+    float uf[3], uff[3], us[3], ud[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        uf[a] = (s.mf[a] - 0.5f * A.F[a]) * irf;
+        uff[a] = (s.mff[a] - 0.5f * A.F[a]) * irff;
+    }
+    const float geqf = geq_f(d[0], d[1], d[2], w, s.drf, rf, uf[0], uf[1], uf[2]);
+    const float geqff = geq_f(d[0], d[1], d[2], w, s.drff, rff, uff[0], uff[1], uff[2]);
+    const float q2 = q * 2.0f, one_m2q = 1.0f - q2;
+    const float fneq = q2 * (s.gf - geqf) + one_m2q * (s.gff - geqff);  // Eq. (21)
+    const bool near = q <= 0.5f;                                        // Eqs. (22)-(23)
+    const float c_f = near ? q2 : (1.0f - q) / q;  // u* = c_f u_f + c_ff u_ff, u_w = 0
+    const float c_ff = near ? one_m2q : 0.0f;
+    const float drd = near ? q2 * s.drf + one_m2q * s.drff : s.drf;
+    const float b = (1.0f - q) / (1.0f + q);  // Eq. (24), u_w = 0
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        us[a] = c_f * uf[a] + c_ff * uff[a];
+        ud[a] = (us[a] + 2.0f * (b * uff[a])) * (1.0f / 3.0f);  // Eq. (25)
+    }
+    const float rd = drd + A.rho0;
+    const float val = geq_f(d[0], d[1], d[2], w, drd, rd, ud[0], ud[1], ud[2]) + fneq;  // Eqs. (20), (19)
+    if (kGrad) {
+        float gd_dr, gd_u[3], gf_dr, gf_u[3], gff_dr, gff_u[3];
+        geq_grad(d, w, rd, ud, gd_dr, gd_u);
+        geq_grad(d, w, rf, uf, gf_dr, gf_u);
+        geq_grad(d, w, rff, uff, gff_dr, gff_u);
+        const float iq = 1.0f / q, i1q = 1.0f / (1.0f + q);
+        float uf_b[3], uff_b[3], q_b = 2.0f * (s.gf - geqf) - 2.0f * (s.gff - geqff), su_f = 0.f, su_ff = 0.f;
+        float du = 0.f, bu = 0.f;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const float us_b = gd_u[a] * (1.0f / 3.0f);
+            uf_b[a] = c_f * us_b - q2 * gf_u[a];
+            uff_b[a] = (c_ff + 2.0f * b) * us_b - one_m2q * gff_u[a];
+            su_f += uf[a] * uf_b[a];
+            su_ff += uff[a] * uff_b[a];
+            // u* by q: 2 (u_f - u_ff), or -u_f / q^2
+            du += us_b * (near ? 2.0f * (uf[a] - uff[a]) : -iq * iq * uf[a]);
+            bu += us_b * uff[a];
+        }
+        q_b += du - 4.0f * i1q * i1q * bu;  // db/dq = -2 / (1 + q)^2
+        if (near) q_b += 2.0f * (s.drf - s.drff) * gd_dr;
+        g.q = q_b;
+        g.f.x = (near ? q2 : 1.0f) * gd_dr - q2 * gf_dr - su_f * irf;
+        g.f.y = uf_b[0] * irf;
+        g.f.z = uf_b[1] * irf;
+        g.f.w = uf_b[2] * irf;
+        g.ff.x = c_ff * gd_dr - one_m2q * gff_dr - su_ff * irff;
+        g.ff.y = uff_b[0] * irff;
+        g.ff.z = uff_b[1] * irff;
+        g.ff.w = uff_b[2] * irff;
+    }
+    return val;
+}
+
+// Population i of an array of 19 (its offset is the same for all threads).
+// Within it the span kernels address by 32-bit byte offsets, which the load
+// and store units add to the base themselves; boxes of 2^30 nodes and more
+// (kWide) by 64-bit ones.
+template <typename T, bool kWide>
+struct Pop {
+    T *base;
+    __device__ __forceinline__ T &operator[](unsigned n) const {
+        return kWide ? base[n] : *reinterpret_cast<T *>((uintptr_t)base + (size_t)(n * 4u));
+    }
+};
+template <bool kWide = true, typename T>
+__device__ __forceinline__ Pop<T, kWide> pop(T *p, const AdjConst &A, int i) {
+    return Pop<T, kWide>{p + (long long)i * A.N};
 }
 
 // ---------------------------------------------------------------------------
 // device data
 // ---------------------------------------------------------------------------
+// Node kinds: a fluid node with links and a solid node are left out of the
+// span kernels; kShared marks the others that are some link's x_ff (the
+// adjoint adds the link's shares there).
+enum NodeKind : uint8_t { kPlain = 0, kLeftOut = 1, kShared = 2 };
+
 struct AdjDev {
     AdjConst c;
-    const uint8_t *solid;     // [N]
-    const uint32_t *lmask;    // [N] particle-link directions of each node
-    const int *linkid;        // [19][N] link index or -1
-    const int *l_nf, *l_dir, *l_nff;  // [L] node, direction (unknown), x_ff node or -1
+    const uint8_t *kind;      // [N] NodeKind
+    // fluid nodes with links: node, link directions (the unknowns), first link
+    const int *n_node, *n_base;
+    const uint32_t *n_mask;
+    int nnodes;
+    const int *l_nf, *l_dir, *l_nff;  // [L] node, direction (unknown), x_ff node or -1; a node's links in
+                                      // direction order
     float *l_q;               // [L]
     double *l_dqdMf, *l_dqdMs;  // [L] dq/dM at x_f and x_s (0 where q was clamped)
     double *l_dJdq;           // [L]
-    float *l_lam;             // [L] lambda_in of the link's direction at its node (this step)
     int nlinks;
     const double *cp;         // [ncp][3] world
     const double *K;          // [ncp]
@@ -217,81 +215,55 @@ struct AdjDev {
     double *grad;             // [ncp][4]: dJ/dx, dJ/dy, dJ/dz, dJ/dK
     float inv_W;
 };
+// What a forward step keeps for the adjoint (mom NULL: nothing).
+struct Kept {
+    float4 *mom;              // [N] density offset and momentum of the pulled values
+    float4 *l_f, *l_ff;       // [L] LinkGrad
+    float *l_gq;              // [L]
+};
 
 __device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-// The value a particle link of direction i (the unknown, arriving from the
-// solid node x - e_i) takes at fluid node n: VIBB of Eqs. (19)-(25) from the
-// node's moments (drho_f, m_f) and x_ff's populations, or halfway
-// bounce-back when x_ff is solid.  i is a run-time index: populations are
-// read from the state by address, never from an indexed local array.
-__device__ __noinline__ float link_value(const AdjDev &D, const float *__restrict__ S, long long n, int i,
-                                         float drho_f, float mfx, float mfy, float mfz) {
-    const AdjConst &A = D.c;
-    const long long N = A.N;
-    const int io = L19::opp(i);
-    const float gown_io = S[(long long)io * N + n];
-    const int L = D.linkid[(long long)i * N + n];
-    const int nff = D.l_nff[L];
-    if (nff < 0) return gown_io;  // halfway bounce-back, u_w = 0
-    float drff = 0.f, mff[3] = {0.f, 0.f, 0.f};
+// The rows next to node (x, y, z): nx (y' + ny z') and x' for offsets -1, 0, 1.
+struct Around {
+    int xs[3], row[3][3];
+};
+__device__ __forceinline__ Around around(const AdjConst &A, int n) {
+    const int z = (int)fast_quot((uint32_t)n, A.by_nxy), r = n - z * A.nx * A.ny;
+    const int y = (int)fast_quot((uint32_t)r, A.by_nx), x = r - y * A.nx;
+    Around o;
+    int ys[3], zs[3];
 #pragma unroll
-    for (int k = 0; k < Q; k++) {
-        const float gk = S[(long long)k * N + nff];
-        drff += gk;
-        mff[0] += gk * L19::e(k, 0);
-        mff[1] += gk * L19::e(k, 1);
-        mff[2] += gk * L19::e(k, 2);
+    for (int k = 0; k < 3; k++) {
+        o.xs[k] = wrapi(x + k - 1, A.nx);
+        ys[k] = wrapi(y + k - 1, A.ny);
+        zs[k] = wrapi(z + k - 1, A.nz);
     }
-    const float gff_io = S[(long long)io * N + nff];
-    return vibb_t<float>(A, io, D.l_q[L], drho_f, mfx, mfy, mfz, gown_io, drff, mff[0], mff[1], mff[2], gff_io);
+#pragma unroll
+    for (int b = 0; b < 3; b++)
+#pragma unroll
+        for (int c = 0; c < 3; c++) o.row[b][c] = A.nx * (ys[b] + A.ny * zs[c]);
+    return o;
+}
+// node n - e_i
+__device__ __forceinline__ int upstream(const Around &o, int i) {
+    return o.xs[1 - L19::e(i, 0)] + o.row[1 - L19::e(i, 1)][1 - L19::e(i, 2)];
 }
 
-// The pulled values g_in of fluid node (x, y, z) from the state S, with the
-// link values substituted on its particle links (lm).  Every array here is
-// indexed by unrolled loop counters only, so it stays in registers.
-__device__ __forceinline__ void gather(const AdjDev &D, const float *__restrict__ S, int x, int y, int z, long long n,
-                                       uint32_t lm, float gin[Q]) {
-    const AdjConst &A = D.c;
-    const int N = (int)A.N;  // fewer than 2^31 nodes
-    // every pull is issued at once (on a link direction its value is replaced
-    // below), so the loads do not wait for the link mask
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-        const int sx = wrapi(x - L19::e(i, 0), A.nx), sy = wrapi(y - L19::e(i, 1), A.ny),
-                  sz = wrapi(z - L19::e(i, 2), A.nz);
-        gin[i] = S[(long long)i * N + (sx + A.nx * (sy + A.ny * sz))];
-    }
-    if (!lm) return;
-    float drho_f = 0.f, mf[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-    for (int k = 0; k < Q; k++) {
-        const float g = S[(long long)k * N + n];
-        drho_f += g;
-        mf[0] += g * L19::e(k, 0);
-        mf[1] += g * L19::e(k, 1);
-        mf[2] += g * L19::e(k, 2);
-    }
-#pragma unroll
-    for (int i = 0; i < Q; i++)
-        if ((lm >> i) & 1u) gin[i] = link_value(D, S, n, i, drho_f, mf[0], mf[1], mf[2]);
-}
-
-// Node of this thread: CTA = 32 x 4 x 2 nodes
-__device__ __forceinline__ bool node_of(const AdjConst &A, int &x, int &y, int &z, long long &n) {
-    x = blockIdx.x * 32 + threadIdx.x % 32;
-    y = blockIdx.y * 4 + (threadIdx.x / 32) % 4;
-    z = blockIdx.z * 2 + threadIdx.x / 128;
-    n = x + (long long)A.nx * (y + (long long)A.ny * z);
-    return x < A.nx && y < A.ny && z < A.nz;
+// The 256-node span of a block; every other launch runs through the lattice
+// from its end, so that it starts with what the launch before touched last
+// (two states and the adjoint of a 96^3 box are about the size of L2).
+__device__ __forceinline__ int span_node(bool reverse) {
+    const unsigned b = reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    return (int)(b * 256u + threadIdx.x);
 }
 
 __global__ void __launch_bounds__(256) k_adj_init(AdjDev D, float *S, float ux, float uy, float uz) {
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < D.c.N; n += (long long)gridDim.x * blockDim.x)
 #pragma unroll
         for (int i = 0; i < Q; i++)
-            S[(long long)i * D.c.N + n] = geq_t<float>(L19::e(i, 0), L19::e(i, 1), L19::e(i, 2), (float)L19::w(i), 0.f,
-                                                       D.c.rho0, ux, uy, uz);
+            S[(long long)i * D.c.N + n] = geq_f((float)L19::e(i, 0), (float)L19::e(i, 1), (float)L19::e(i, 2),
+                                                (float)L19::w(i), 0.f, D.c.rho0, ux, uy, uz);
 }
 
 // q of every link for the control points of this forward run (Eq. (27) with
@@ -329,169 +301,355 @@ __global__ void k_adj_q(AdjDev D) {
     }
 }
 
-// One forward step S -> R; accumulates the drag when in the window.
-__global__ void __launch_bounds__(256) k_adj_step(AdjDev D, const float *__restrict__ S, float *__restrict__ R,
-                                                   int window) {
-    const AdjConst &A = D.c;
-    int x, y, z;
-    long long n;
-    const bool in = node_of(A, x, y, z, n);
-    // the node's solid mark and link mask in one round
-    const bool solid = in ? D.solid[n] != 0 : true;
-    const uint32_t lm = in ? D.lmask[n] : 0u;
-    const bool act = in && !solid;
-    float Fx = 0.f;
-    if (act) {
-        float gin[Q];
-        gather(D, S, x, y, z, n, lm, gin);
-        if (window && lm) {
-#pragma unroll
-            for (int i = 1; i < Q; i++) {
-                if (!((lm >> i) & 1u)) continue;
-                const int io = L19::opp(i);
-                // Eq. (28), x component, offsets
-                Fx += (float)L19::e(io, 0) * (S[(long long)io * A.N + n] + gin[i]);
-            }
-        }
-        float drho = 0.f, mx = 0.f, my = 0.f, mz = 0.f;
-#pragma unroll
-        for (int i = 0; i < Q; i++) {
-            drho += gin[i];
-            mx += gin[i] * L19::e(i, 0);
-            my += gin[i] * L19::e(i, 1);
-            mz += gin[i] * L19::e(i, 2);
-        }
-#pragma unroll
-        for (int i = 0; i < Q; i++)
-            R[(long long)i * A.N + n] = (1.0f - A.omega) * gin[i] + collide_h<float>(A, i, drho, mx, my, mz);
-    }
-    if (window) {
-        for (int o = 16; o > 0; o >>= 1) Fx += __shfl_xor_sync(0xffffffffu, Fx, o);
-        if ((threadIdx.x & 31) == 0 && Fx != 0.f)
-            atomicAdd(D.J_fix, (unsigned long long)__float2ll_rn(Fx * (float)(1ull << kForceFixBits)));
-    }
+// The collided population along e, less (1 - omega) times the pulled one:
+// omega g^eq + Guo's term (Eqs. (15)-(16), Eq. (18)'s half-force shift).  The
+// roundings are spelled out: over hundreds of steps another order of them
+// drifts the drag by 1e-5 (sharing the even parts of opposite directions, as
+// collide_values does, would too).
+template <bool kForce>
+__device__ __forceinline__ float collide_h(const AdjConst &A, float w, float eu, float uu, float eF, float uF,
+                                           float drho, float rho) {
+    const float p = __fmaf_rn(-uu, 1.5f, __fmaf_rn(eu, 3.0f, __fmul_rn(__fmul_rn(eu, eu), 4.5f)));
+    const float g = __fmul_rn(__fmaf_rn(rho, p, drho), w);
+    if (!kForce) return __fmul_rn(g, A.omega);
+    const float t = __fmaf_rn(__fsub_rn(eF, uF), 3.0f, __fmul_rn(eu, __fmul_rn(9.0f, eF)));
+    return __fmaf_rn(t, __fmul_rn(A.gfac, w), __fmul_rn(g, A.omega));
 }
 
-// A1 + A2 in push form (see the top of the file): lambda_in of fluid node n
-// through the collision (with the drag's dependence on the pulled link
-// values), pushed along the pull it came from; on a link direction i the
-// node writes dJ/dg+(t) of its own opposite direction (no fluid neighbour
-// pushes it): the halfway link's value and the drag's dependence on the
-// node's own populations, and keeps lambda_in_i(n) for A3.  The arithmetic
-// and its order are those of the two-kernel form.
-__global__ void __launch_bounds__(256, 3) k_adj_back(AdjDev D, const float *__restrict__ S,
-                                                    const float *__restrict__ lamN, float *__restrict__ lamT,
-                                                    int window) {
-    const AdjConst &A = D.c;
-    int x, y, z;
-    long long n;
-    if (!node_of(A, x, y, z, n)) return;
-    const bool solid = D.solid[n] != 0;
-    const uint32_t lm = D.lmask[n];  // with the solid mark, in one round
-    if (solid) return;
-    float gin[Q];
-    gather(D, S, x, y, z, n, lm, gin);
+// Collision of the pulled values: the new populations of node n, and its
+// moments for the adjoint.
+template <bool kForce, bool kWide>
+__device__ __forceinline__ void adj_collide(const AdjConst &A, const float (&g)[Q], int n, float *R, float4 *mom) {
     float drho = 0.f, mx = 0.f, my = 0.f, mz = 0.f;
 #pragma unroll
     for (int i = 0; i < Q; i++) {
-        drho += gin[i];
-        mx += gin[i] * L19::e(i, 0);
-        my += gin[i] * L19::e(i, 1);
-        mz += gin[i] * L19::e(i, 2);
+        drho += g[i];
+        mx = add_e(mx, L19::e(i, 0), g[i]);
+        my = add_e(my, L19::e(i, 1), g[i]);
+        mz = add_e(mz, L19::e(i, 2), g[i]);
     }
-    // a = sum_i lambda_i dh_i/d(drho), b = sum_i lambda_i dh_i/dm for
-    // collide_h (h_i = omega g^eq_i + Guo's term, u = (m + F/2) / rho),
-    // differentiated by hand: with P_i = 3 e.u + 4.5 (e.u)^2 - 1.5 u.u,
-    //   dh_i/d(drho) at fixed u = omega w_i (1 + P_i),
-    //   dh_i/du = omega w_i rho (3 e_i + 9 (e_i.u) e_i - 3 u)
-    //             + gfac w_i (9 (e_i.F) e_i - 3 F),
-    // and du/dm = I / rho, du/d(drho) = -u / rho.
+    if (mom) __stcs(&mom[n], make_float4(drho, mx, my, mz));
     const float rho = drho + A.rho0, ir = 1.0f / rho;
-    const float ux = (mx + 0.5f * A.F[0]) * ir, uy = (my + 0.5f * A.F[1]) * ir, uz = (mz + 0.5f * A.F[2]) * ir;
-    const float uu = ux * ux + uy * uy + uz * uz;
-    float lam[Q], sp = 0.f, sl = 0.f, v3[3] = {0.f, 0.f, 0.f}, f3[3] = {0.f, 0.f, 0.f};
+    const float ux = (kForce ? __fmaf_rn(0.5f, A.F[0], mx) : mx) * ir, uy = (kForce ? __fmaf_rn(0.5f, A.F[1], my) : my) * ir,
+                uz = (kForce ? __fmaf_rn(0.5f, A.F[2], mz) : mz) * ir;
+    const float uu = __fmaf_rn(uz, uz, __fmaf_rn(ux, ux, __fmul_rn(uy, uy)));
+    const float uF = kForce ? __fmaf_rn(uz, A.F[2], __fmaf_rn(ux, A.F[0], __fmul_rn(uy, A.F[1]))) : 0.f;
+    const float om1 = 1.0f - A.omega;
+    pop<kWide>(R, A, 0)[(unsigned)n] =
+        __fmaf_rn(om1, g[0], collide_h<kForce>(A, (float)L19::w(0), 0.f, uu, 0.f, uF, drho, rho));
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        lam[i] = lamN[(long long)i * A.N + n];
+    for (int i = 1; i < Q; i += 2) {
         const int ex = L19::e(i, 0), ey = L19::e(i, 1), ez = L19::e(i, 2);
-        const float lw = lam[i] * (float)L19::w(i);
-        const float eu = ux * (float)ex + uy * (float)ey + uz * (float)ez;
-        sp += lw * (1.0f + (eu * 3.0f + eu * eu * 4.5f - uu * 1.5f));
-        sl += lw;
-        const float c = lw * (3.0f + 9.0f * eu);
-        const float cf = lw * (9.0f * (ex * A.F[0] + ey * A.F[1] + ez * A.F[2]));
-        v3[0] += c * ex; v3[1] += c * ey; v3[2] += c * ez;
-        f3[0] += cf * ex; f3[1] += cf * ey; f3[2] += cf * ez;
-    }
-    const float u3[3] = {ux, uy, uz};
-    float b[3], gu = 0.f;
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        const float g = A.omega * rho * (v3[c] - 3.0f * u3[c] * sl) + A.gfac * (f3[c] - 3.0f * A.F[c] * sl);
-        b[c] = g * ir;
-        gu += g * u3[c];
-    }
-    const float a = A.omega * sp - gu * ir;
-#pragma unroll
-    for (int j = 0; j < Q; j++) {
-        float v = (1.0f - A.omega) * lam[j] + a + b[0] * L19::e(j, 0) + b[1] * L19::e(j, 1) + b[2] * L19::e(j, 2);
-        if ((lm >> j) & 1u) {
-            // link j: x - e_j is solid; lamT_{opp j}(n) has no other writer
-            if (window) v += D.inv_W * (float)L19::e(L19::opp(j), 0);
-            const int L = D.linkid[(long long)j * A.N + n];
-            D.l_lam[L] = v;
-            const int io = L19::opp(j);
-            float acc = 0.f;
-            if (D.l_nff[L] < 0) acc += v;
-            if (window) acc += D.inv_W * (float)L19::e(io, 0);
-            lamT[(long long)io * A.N + n] = acc;
-        } else {
-            const int tx = wrapi(x - L19::e(j, 0), A.nx), ty = wrapi(y - L19::e(j, 1), A.ny),
-                      tz = wrapi(z - L19::e(j, 2), A.nz);
-            lamT[(long long)j * A.N + (tx + A.nx * (ty + (long long)A.ny * tz))] = v;
-        }
+        const float eu = dot_e(ex, ey, ez, ux, uy, uz);
+        const float eF = kForce ? dot_e(ex, ey, ez, A.F[0], A.F[1], A.F[2]) : 0.f;
+        const float w = (float)L19::w(i);
+        pop<kWide>(R, A, i)[(unsigned)n] = __fmaf_rn(om1, g[i], collide_h<kForce>(A, w, eu, uu, eF, uF, drho, rho));
+        pop<kWide>(R, A, i + 1)[(unsigned)n] = __fmaf_rn(om1, g[i + 1], collide_h<kForce>(A, w, -eu, uu, -eF, uF, drho, rho));
     }
 }
 
-// A3: the VIBB links (x_ff fluid): 11 partial derivatives by dual numbers,
-// scattered into dJ/dg+(t) at x_f and x_ff, and dJ/dq of the link.
-__global__ void __launch_bounds__(128) k_adj_vibb(AdjDev D, const float *__restrict__ S, float *__restrict__ lamT) {
+// Forward step S -> R, the nodes without links (k_static_plain's waits).
+// Six CTAs per SM (40 registers): what bounds it is how many loads are in
+// flight beside the arithmetic; 96^3 at 4 / 5 / 6: 30.5, 28.9, 27.5 us a step.
+template <bool kForce, bool kWide>
+__global__ void __launch_bounds__(256, 6) k_adj_step(AdjDev D, const float *__restrict__ S, float *__restrict__ R,
+                                                      Kept kept, int reverse) {
+    pdl_launch_dependents();
     const AdjConst &A = D.c;
-    const long long N = A.N;
-    for (int L = blockIdx.x * blockDim.x + threadIdx.x; L < D.nlinks; L += gridDim.x * blockDim.x) {
-        const int nff = D.l_nff[L];
-        if (nff < 0) continue;
-        const long long nf = D.l_nf[L];
-        const int i = D.l_dir[L], io = L19::opp(i);
-        const float lam = D.l_lam[L];
-        if (lam == 0.f) continue;
-        float drf = 0.f, mf[3] = {0.f, 0.f, 0.f}, gf = 0.f, drff = 0.f, mff[3] = {0.f, 0.f, 0.f}, gff = 0.f;
+    const int n = span_node(reverse != 0);
+    if (n < A.N) {
+        const bool take = D.kind[n] != kLeftOut;
+        const Around o = around(A, n);
+        float gin[Q];
 #pragma unroll
-        for (int k = 0; k < Q; k++) {
-            const float a = S[(long long)k * N + nf], b = S[(long long)k * N + nff];
-            drf += a;
-            drff += b;
-            for (int c = 0; c < 3; c++) {
-                mf[c] += a * L19::e(k, c);
-                mff[c] += b * L19::e(k, c);
+        for (int i = 0; i < Q; i++) gin[i] = pop<kWide>(S, A, i)[(unsigned)upstream(o, i)];
+        if (take) adj_collide<kForce, kWide>(A, gin, n, R, kept.mom);
+    }
+    pdl_wait();
+}
+
+// Forward step S -> R, the nodes with links: a warp takes kLinkNodes of them,
+// its lanes evaluate their links (both nodes' populations in one round of
+// loads), then each node takes its links' values, pulls the rest and collides.
+// The drag of a step in the window is Eq. (28)'s x component over the links,
+// in fixed point (exact in any order).
+constexpr int kLinkNodes = 4;
+template <bool kForce>
+__global__ void __launch_bounds__(256, 2) k_adj_step_links(AdjDev D, const float *S, float *R, Kept kept, int window) {
+    __shared__ unsigned short s_ent[8][kLinkNodes * 18];
+    __shared__ float s_val[8][kLinkNodes * 18];
+    pdl_wait();
+    pdl_launch_dependents();
+    const AdjConst &A = D.c;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int w0 = (blockIdx.x * 8 + warp) * kLinkNodes;
+    if (w0 >= D.nnodes) return;
+    const bool has = lane < kLinkNodes && w0 + lane < D.nnodes;
+    const int n = has ? D.n_node[w0 + lane] : 0, base = has ? D.n_base[w0 + lane] : 0;
+    const uint32_t lm = has ? D.n_mask[w0 + lane] : 0u;
+    const int first_link = __shfl_sync(0xffffffffu, base, 0);
+    const int first = base - first_link;  // the nodes' links follow one another
+    int total = __popc(lm);
+#pragma unroll
+    for (int o = 1; o < kLinkNodes; o <<= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    total = __shfl_sync(0xffffffffu, total, 0);
+    uint32_t m = lm;
+    for (int k = first; m; k++) {
+        const int i = __ffs(m) - 1;
+        m &= m - 1;
+        s_ent[warp][k] = (unsigned short)((lane << 5) | i);
+    }
+    __syncwarp();
+    long long drag = 0;
+    for (int r = 0; r < total; r += 32) {
+        const int e = r + lane;
+        const int ent = e < total ? s_ent[warp][e] : 0;
+        const int nf = __shfl_sync(0xffffffffu, n, ent >> 5);
+        if (e < total) {
+            const int L = first_link + e, i = ent & 31, io = L19::opp(i);
+            const int nff = D.l_nff[L];
+            const int at = nff < 0 ? nf : nff;
+            const float q = D.l_q[L];
+            LinkState s = {};
+#pragma unroll
+            for (int k = 0; k < Q; k++) {
+                const float a = pop(S, A, k)[(unsigned)nf], b = pop(S, A, k)[(unsigned)at];
+                s.drf += a;
+                s.drff += b;
+                s.mf[0] = add_e(s.mf[0], L19::e(k, 0), a);
+                s.mf[1] = add_e(s.mf[1], L19::e(k, 1), a);
+                s.mf[2] = add_e(s.mf[2], L19::e(k, 2), a);
+                s.mff[0] = add_e(s.mff[0], L19::e(k, 0), b);
+                s.mff[1] = add_e(s.mff[1], L19::e(k, 1), b);
+                s.mff[2] = add_e(s.mff[2], L19::e(k, 2), b);
+                if (k == io) {
+                    s.gf = a;
+                    s.gff = b;
+                }
             }
-            if (k == io) { gf = a; gff = b; }
-        }
-        const Dual<11> v = vibb_t<Dual<11>>(A, io, dvar<11>(D.l_q[L], 0), dvar<11>(drf, 1), dvar<11>(mf[0], 2),
-                                            dvar<11>(mf[1], 3), dvar<11>(mf[2], 4), dvar<11>(gf, 5),
-                                            dvar<11>(drff, 6), dvar<11>(mff[0], 7), dvar<11>(mff[1], 8),
-                                            dvar<11>(mff[2], 9), dvar<11>(gff, 10));
-        D.l_dJdq[L] += (double)lam * (double)v.d[0];
-#pragma unroll
-        for (int k = 0; k < Q; k++) {
-            const float ek[3] = {(float)L19::e(k, 0), (float)L19::e(k, 1), (float)L19::e(k, 2)};
-            float cf = v.d[1] + v.d[2] * ek[0] + v.d[3] * ek[1] + v.d[4] * ek[2];
-            float cff = v.d[6] + v.d[7] * ek[0] + v.d[8] * ek[1] + v.d[9] * ek[2];
-            if (k == io) { cf += v.d[5]; cff += v.d[10]; }
-            atomicAdd(&lamT[(long long)k * N + nf], lam * cf);
-            atomicAdd(&lamT[(long long)k * N + nff], lam * cff);
+            float v = s.gf;  // halfway bounce-back, u_w = 0
+            if (nff >= 0) {
+                LinkGrad g;
+                if (kept.mom) {
+                    v = vibb_f<true>(A, io, q, s, g);
+                    kept.l_f[L] = g.f;
+                    kept.l_ff[L] = g.ff;
+                    kept.l_gq[L] = g.q;
+                } else {
+                    v = vibb_f<false>(A, io, q, s, g);
+                }
+            }
+            s_val[warp][e] = v;
+            if (window) {
+                const float dx = (float)lat_e<19>(io, 0);
+                drag += __float2ll_rn(dx * (s.gf + v) * (float)(1ull << kForceFixBits));
+            }
         }
     }
+    __syncwarp();
+    if (has) {
+        const Around o = around(A, n);
+        float gin[Q];
+        int k = first;
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            if ((lm >> i) & 1u) gin[i] = s_val[warp][k++];
+            else gin[i] = pop(S, A, i)[(unsigned)upstream(o, i)];
+        }
+        adj_collide<kForce, true>(A, gin, n, R, kept.mom);
+    }
+    if (window) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) drag += __shfl_xor_sync(0xffffffffu, drag, o);
+        if (lane == 0 && drag) atomicAdd(D.J_fix, (unsigned long long)drag);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// adjoint step
+// ---------------------------------------------------------------------------
+// a = sum_i lambda_i dh_i/d(drho), b = sum_i lambda_i dh_i/dm for the part h_i
+// of the collided population i that depends on the pulled values through
+// their density offset and momentum (omega g^eq_i + Guo's term, u = (m + F/2)
+// / rho), differentiated by hand: with P_i = 3 e.u + 4.5 (e.u)^2 - 1.5 u.u,
+//   dh_i/d(drho) at fixed u = omega w_i (1 + P_i),
+//   dh_i/du = omega w_i rho (3 e_i + 9 (e_i.u) e_i - 3 u)
+//             + gfac w_i (9 (e_i.F) e_i - 3 F),
+// and du/dm = I / rho, du/d(drho) = -u / rho.  The sums over the directions,
+// with S = w_i (lambda_i + lambda_i') and D = w_i (lambda_i - lambda_i') of a
+// pair of opposite ones:
+//   sl = sum S, p = sum (3 e.u D + 4.5 (e.u)^2 S),
+//   V = sum e (omega rho (3 D + 9 e.u S) + 9 gfac e.F S).
+struct BackSums {
+    float sl, p, V[3];
+};
+// the terms of one pair (S, D) along e
+template <bool kForce>
+__device__ __forceinline__ void back_pair(const AdjConst &A, float S, float D, float eu, float eFg, float om_rho,
+                                          float &sl, float &p, float &t) {
+    const float seu = S * eu;
+    sl += S;
+    p += eu * (3.0f * D + 4.5f * seu);
+    t = om_rho * (3.0f * D + 9.0f * seu);
+    if (kForce) t += 9.0f * eFg * S;
+}
+__device__ __forceinline__ float4 back_ab(const AdjConst &A, const BackSums &s, float om_rho, float ir,
+                                          const float u[3]) {
+    const float uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    float b[3], gu = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const float g = s.V[c] - 3.0f * s.sl * (om_rho * u[c] + A.Fg[c]);
+        b[c] = g * ir;
+        gu += g * u[c];
+    }
+    return make_float4(A.omega * (s.sl * (1.0f - 1.5f * uu) + s.p) - gu * ir, b[0], b[1], b[2]);
+}
+
+// Adjoint step lamN -> lamT, the nodes without links: every neighbour is
+// fluid, so lambda_in goes to all of them.  share/share_next: the density and
+// momentum shares that this step's reader adds (and clears for the step after
+// the next) and that the link kernel sums for the next step.
+// Four CTAs per SM: 96^3 at 3 / 4: 33.6, 31.2 us a step.
+template <bool kForce, bool kWide>
+__global__ void __launch_bounds__(256, 4) k_adj_back(AdjDev D, const float4 *__restrict__ mom,
+                                                      const float *__restrict__ lamN, float *__restrict__ lamT,
+                                                      float4 *share, int reverse) {
+    pdl_launch_dependents();
+    const AdjConst &A = D.c;
+    const int n = span_node(reverse != 0);
+    if (n < A.N) {
+        const uint8_t kind = D.kind[n];
+        const float4 mo = __ldcs(&mom[n]);
+        float lam[Q];
+#pragma unroll
+        for (int i = 0; i < Q; i++) lam[i] = pop<kWide>(lamN, A, i)[(unsigned)n];
+        if (kind != kLeftOut) {
+            if (kind == kShared) {
+                const float4 x = share[n];
+                share[n] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < Q; i++)
+                    lam[i] = add_e(add_e(add_e(lam[i] + x.x, L19::e(i, 0), x.y), L19::e(i, 1), x.z), L19::e(i, 2), x.w);
+            }
+            const float rho = mo.x + A.rho0, ir = 1.0f / rho, om_rho = A.omega * rho;
+            const float u[3] = {(mo.y + 0.5f * A.F[0]) * ir, (mo.z + 0.5f * A.F[1]) * ir, (mo.w + 0.5f * A.F[2]) * ir};
+            BackSums s = {};
+            s.sl = (float)L19::w(0) * lam[0];
+#pragma unroll
+            for (int i = 1; i < Q; i += 2) {
+                const int ex = L19::e(i, 0), ey = L19::e(i, 1), ez = L19::e(i, 2);
+                const float w = (float)L19::w(i);
+                float t;
+                back_pair<kForce>(A, w * (lam[i] + lam[i + 1]), w * (lam[i] - lam[i + 1]),
+                                  dot_e(ex, ey, ez, u[0], u[1], u[2]), dot_e(ex, ey, ez, A.Fg[0], A.Fg[1], A.Fg[2]),
+                                  om_rho, s.sl, s.p, t);
+                s.V[0] = add_e(s.V[0], ex, t);
+                s.V[1] = add_e(s.V[1], ey, t);
+                s.V[2] = add_e(s.V[2], ez, t);
+            }
+            const float4 ab = back_ab(A, s, om_rho, ir, u);
+            const float om1 = 1.0f - A.omega;
+            const Around o = around(A, n);
+            pop<kWide>(lamT, A, 0)[(unsigned)n] = om1 * lam[0] + ab.x;
+#pragma unroll
+            for (int j = 1; j < Q; j += 2) {
+                const float eb = dot_e(L19::e(j, 0), L19::e(j, 1), L19::e(j, 2), ab.y, ab.z, ab.w);
+                pop<kWide>(lamT, A, j)[(unsigned)upstream(o, j)] = om1 * lam[j] + (ab.x + eb);
+                pop<kWide>(lamT, A, j + 1)[(unsigned)upstream(o, j + 1)] = om1 * lam[j + 1] + (ab.x - eb);
+            }
+        }
+    }
+    pdl_wait();
+}
+
+// Adjoint step, the nodes with links: one warp per node, lane i its direction
+// i, so a node's links and their kept derivatives are read in one round.
+__global__ void __launch_bounds__(256) k_adj_back_links(AdjDev D, Kept kept, const float *lamN, float *lamT,
+                                                         float4 *share, float4 *share_next, int window) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const AdjConst &A = D.c;
+    const int lane = threadIdx.x & 31;
+    const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (w >= D.nnodes) return;
+    const int n = D.n_node[w], base = D.n_base[w];
+    const uint32_t lm = D.n_mask[w];
+    const bool dir = lane < Q;
+    const bool link = dir && ((lm >> lane) & 1u);
+    const int L = base + __popc(lm & ((1u << lane) - 1u));
+    const int ei[3] = {dir ? lat_e<19>(lane, 0) : 0, dir ? lat_e<19>(lane, 1) : 0, dir ? lat_e<19>(lane, 2) : 0};
+    const float ex = (float)ei[0], ey = (float)ei[1], ez = (float)ei[2];
+    const float wi = dir ? (float)lat_w<19>(lane) : 0.f;
+    const float4 mo = kept.mom[n];
+    const float4 x = share[n];
+    float lam = dir ? lamN[(long long)lane * A.N + n] : 0.f;
+    int nff = -1;
+    float q = 0.f, gq = 0.f;
+    float4 gf = make_float4(0.f, 0.f, 0.f, 0.f), gff = gf;
+    if (link) {
+        nff = D.l_nff[L];
+        q = D.l_q[L];
+        gq = kept.l_gq[L];
+        gf = kept.l_f[L];
+        gff = kept.l_ff[L];
+    }
+    __syncwarp();
+    if (lane == 0) share[n] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (dir) lam += x.x + ex * x.y + ey * x.z + ez * x.w;
+    const float rho = mo.x + A.rho0, ir = 1.0f / rho, om_rho = A.omega * rho;
+    const float u[3] = {(mo.y + 0.5f * A.F[0]) * ir, (mo.z + 0.5f * A.F[1]) * ir, (mo.w + 0.5f * A.F[2]) * ir};
+    // a lane's direction by itself: S = D = w_i lambda_i
+    BackSums s = {};
+    float t;
+    back_pair<true>(A, wi * lam, wi * lam, u[0] * ex + u[1] * ey + u[2] * ez, A.Fg[0] * ex + A.Fg[1] * ey + A.Fg[2] * ez,
+                    om_rho, s.sl, s.p, t);
+    s.V[0] = ex * t;
+    s.V[1] = ey * t;
+    s.V[2] = ez * t;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s.sl += __shfl_xor_sync(0xffffffffu, s.sl, o);
+        s.p += __shfl_xor_sync(0xffffffffu, s.p, o);
+#pragma unroll
+        for (int c = 0; c < 3; c++) s.V[c] += __shfl_xor_sync(0xffffffffu, s.V[c], o);
+    }
+    const float4 ab = back_ab(A, s, om_rho, ir, u);
+    float v = (1.0f - A.omega) * lam + ab.x + ab.y * ex + ab.z * ey + ab.w * ez;
+    // the drag's x component of a link along its opposite direction: -e_x
+    if (link && window) v -= D.inv_W * ex;
+    const bool vibb = link && nff >= 0;
+    // the share of x_ff's single population goes with this node's push along
+    // the link's opposite direction
+    const float vff = vibb ? v * (1.0f - 2.0f * q) : 0.f;
+    const int io = lane == 0 ? 0 : ((lane & 1) ? lane + 1 : lane - 1);
+    const float from = __shfl_sync(0xffffffffu, vff, io & 31);
+    if (link) {
+        // dJ/dg+(t) of this node's own opposite population: the halfway
+        // link's value, or the VIBB share 2q, and the drag's dependence on it
+        float acc = nff < 0 ? v : v * (2.0f * q);
+        if (window) acc -= D.inv_W * ex;
+        lamT[(long long)io * A.N + n] = acc;
+    } else if (dir) {
+        const int z = (int)fast_quot((uint32_t)n, A.by_nxy), r = n - z * A.nx * A.ny;
+        const int y = (int)fast_quot((uint32_t)r, A.by_nx), xx = r - y * A.nx;
+        const int t = wrapi(xx - ei[0], A.nx) + A.nx * (wrapi(y - ei[1], A.ny) + A.ny * wrapi(z - ei[2], A.nz));
+        lamT[(long long)lane * A.N + t] = v + (lane > 0 ? from : 0.f);
+    }
+    float4 own = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (vibb) {
+        D.l_dJdq[L] += (double)v * (double)gq;
+        own = make_float4(v * gf.x, v * gf.y, v * gf.z, v * gf.w);
+        atomicAdd(&share_next[nff], make_float4(v * gff.x, v * gff.y, v * gff.z, v * gff.w));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        own.x += __shfl_xor_sync(0xffffffffu, own.x, o);
+        own.y += __shfl_xor_sync(0xffffffffu, own.y, o);
+        own.z += __shfl_xor_sync(0xffffffffu, own.z, o);
+        own.w += __shfl_xor_sync(0xffffffffu, own.w, o);
+    }
+    if (lane == 0) atomicAdd(&share_next[n], own);
 }
 
 // dJ/dq -> dJ/d(control point position, weight) through Eq. (27) and Eq. (4).
@@ -538,13 +696,15 @@ __global__ void __launch_bounds__(256) k_adj_grad(AdjDev D) {
 struct lbm_adj {
     lbm_config cfg;
     int T, W, K, C;          // steps, window, checkpoint interval, checkpoints
-    int ncp, nlinks;
+    bool keep_all;           // every step's kept data is held, else one segment's
+    int ncp, nlinks, nnodes;
     long long N;
     size_t S;                // bytes of one state (19 N floats)
+    size_t kept;             // bytes that one step keeps for the adjoint
     char *ws;
     cudaStream_t stream;
-    size_t o_state[2], o_ckpt, o_seg, o_lam[2], o_llam, o_solid, o_lmask, o_linkid, o_lnf, o_ldir, o_lnff, o_lq,
-        o_dqf, o_dqs, o_dJdq, o_cp, o_K, o_J, o_grad, total;
+    size_t o_state[2], o_ckpt, o_kept, o_lam[2], o_share[2], o_kind, o_nnode, o_nbase, o_nmask, o_lnf, o_ldir, o_lnff,
+        o_lq, o_dqf, o_dqs, o_dJdq, o_cp, o_K, o_J, o_grad, total;
     bool have_forward;
     char err[256];
 };
@@ -595,10 +755,16 @@ void world_cps(const lbm_particle *p, std::vector<double> &cp) {
             cp[3 * k + a] = p->x[a] + R[3 * a] * p->cp[k][0] + R[3 * a + 1] * p->cp[k][1] + R[3 * a + 2] * p->cp[k][2];
 }
 
-// Frozen flags (M >= 1, periodic minimum image) and the links, in node then
-// direction order.
-void classify_links(const lbm_config *c, const lbm_particle *p, std::vector<uint8_t> &solid,
-                    std::vector<uint32_t> &lmask, std::vector<int> &nf, std::vector<int> &dir, std::vector<int> &nff) {
+// The node kinds from the frozen flags (M >= 1, periodic minimum image), the
+// fluid nodes with links (node, directions, first link) and the links, in node
+// then direction order.
+struct Links {
+    std::vector<uint8_t> kind;
+    std::vector<int> node, base, nf, dir, nff;
+    std::vector<uint32_t> mask;
+};
+void classify_links(const lbm_config *c, const lbm_particle *p, Links &k) {
+    std::vector<uint8_t> solid;
     const int nx = c->nx, ny = c->ny, nz = c->nz;
     const long long N = (long long)nx * ny * nz;
     std::vector<double> cp;
@@ -621,28 +787,44 @@ void classify_links(const lbm_config *c, const lbm_particle *p, std::vector<uint
                 }
                 solid[x + (size_t)nx * (y + (size_t)ny * z)] = M >= 1.0;
             }
-    lmask.assign((size_t)N, 0u);
-    nf.clear();
-    dir.clear();
-    nff.clear();
+    k = Links();
+    k.kind.assign((size_t)N, kPlain);
     auto wrap = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };
     for (int z = 0; z < nz; z++)
         for (int y = 0; y < ny; y++)
             for (int x = 0; x < nx; x++) {
                 const long long n = x + (long long)nx * (y + (long long)ny * z);
-                if (solid[(size_t)n]) continue;
+                if (solid[(size_t)n]) {
+                    k.kind[(size_t)n] = kLeftOut;
+                    continue;
+                }
+                uint32_t mask = 0;
+                const int base = (int)k.nf.size();
                 for (int i = 1; i < Q; i++) {
                     const int ex = L19::e(i, 0), ey = L19::e(i, 1), ez = L19::e(i, 2);
                     const long long s = wrap(x - ex, nx) + (long long)nx * (wrap(y - ey, ny) + (long long)ny * wrap(z - ez, nz));
                     if (!solid[(size_t)s]) continue;
                     const long long f2 = wrap(x + ex, nx) + (long long)nx * (wrap(y + ey, ny) + (long long)ny * wrap(z + ez, nz));
-                    lmask[(size_t)n] |= 1u << i;
-                    nf.push_back((int)n);
-                    dir.push_back(i);
-                    nff.push_back(solid[(size_t)f2] ? -1 : (int)f2);
+                    mask |= 1u << i;
+                    k.nf.push_back((int)n);
+                    k.dir.push_back(i);
+                    k.nff.push_back(solid[(size_t)f2] ? -1 : (int)f2);
+                }
+                if (mask) {
+                    k.kind[(size_t)n] = kLeftOut;
+                    k.node.push_back((int)n);
+                    k.base.push_back(base);
+                    k.mask.push_back(mask);
                 }
             }
+    for (int f2 : k.nff)
+        if (f2 >= 0 && k.kind[(size_t)f2] == kPlain) k.kind[(size_t)f2] = kShared;
 }
+
+// Kept data of every step up to this much (a thirty-fifth of the GPU's
+// memory; 96^3 keeps 600 steps): the adjoint then runs no forward step again.
+// Larger runs keep a state every ceil(sqrt(T)) steps and one segment's data.
+constexpr size_t kKeepAllBytes = (size_t)8 << 30;
 
 void adj_layout(lbm_adj *a) {
     size_t o = 0;
@@ -651,17 +833,19 @@ void adj_layout(lbm_adj *a) {
         o = align_up(o + bytes);
         return at;
     };
-    const size_t L = (size_t)std::max(1, a->nlinks), N = (size_t)a->N;
+    const size_t L = (size_t)std::max(1, a->nlinks), N = (size_t)a->N, M = (size_t)std::max(1, a->nnodes);
     a->o_state[0] = take(a->S);
     a->o_state[1] = take(a->S);
-    a->o_ckpt = take(a->S * (size_t)a->C);
-    a->o_seg = take(a->S * (size_t)std::max(1, a->K - 1));
+    a->o_ckpt = take(a->keep_all ? 0 : a->S * (size_t)a->C);
+    a->o_kept = take(a->kept * (size_t)(a->keep_all ? a->T : a->K));
     a->o_lam[0] = take(a->S);
     a->o_lam[1] = take(a->S);
-    a->o_llam = take(L * 4);
-    a->o_solid = take(N);
-    a->o_lmask = take(N * 4);
-    a->o_linkid = take(N * Q * 4);
+    a->o_share[0] = take(N * 16);
+    a->o_share[1] = take(N * 16);
+    a->o_kind = take(N);
+    a->o_nnode = take(M * 4);
+    a->o_nbase = take(M * 4);
+    a->o_nmask = take(M * 4);
     a->o_lnf = take(L * 4);
     a->o_ldir = take(L * 4);
     a->o_lnff = take(L * 4);
@@ -676,16 +860,20 @@ void adj_layout(lbm_adj *a) {
     a->total = o;
 }
 
-void adj_sizes(lbm_adj *a, const lbm_config *c, int T, int W, int ncp, int nlinks) {
+void adj_sizes(lbm_adj *a, const lbm_config *c, int T, int W, int ncp, const Links &k) {
     a->cfg = *c;
     a->T = T;
     a->W = W;
     a->K = std::max(1, (int)std::ceil(std::sqrt((double)T)));
     a->C = (T + a->K - 1) / a->K;
     a->ncp = ncp;
-    a->nlinks = nlinks;
+    a->nlinks = (int)k.nf.size();
+    a->nnodes = (int)k.node.size();
     a->N = (long long)c->nx * c->ny * c->nz;
-    a->S = (size_t)Q * (size_t)a->N * 4;
+    a->S = align_up((size_t)Q * (size_t)a->N * 4);
+    const size_t L = (size_t)std::max(1, a->nlinks);
+    a->kept = align_up((size_t)a->N * 16) + 2 * align_up(L * 16) + align_up(L * 4);
+    a->keep_all = a->kept <= kKeepAllBytes / (size_t)T;
 }
 
 AdjDev adj_dev(lbm_adj *a) {
@@ -695,11 +883,18 @@ AdjDev adj_dev(lbm_adj *a) {
     D.c.rho0 = (float)c.rho0;
     D.c.omega = (float)(1.0 / c.tau);
     D.c.gfac = (float)(1.0 - 0.5 / c.tau);
-    for (int k = 0; k < 3; k++) D.c.F[k] = (float)c.force[k];
+    for (int k = 0; k < 3; k++) {
+        D.c.F[k] = (float)c.force[k];
+        D.c.Fg[k] = D.c.gfac * D.c.F[k];
+    }
+    D.c.by_nxy = fast_div((uint32_t)(c.nx * c.ny));
+    D.c.by_nx = fast_div((uint32_t)c.nx);
     char *w = a->ws;
-    D.solid = reinterpret_cast<const uint8_t *>(w + a->o_solid);
-    D.lmask = reinterpret_cast<const uint32_t *>(w + a->o_lmask);
-    D.linkid = reinterpret_cast<const int *>(w + a->o_linkid);
+    D.kind = reinterpret_cast<const uint8_t *>(w + a->o_kind);
+    D.n_node = reinterpret_cast<const int *>(w + a->o_nnode);
+    D.n_base = reinterpret_cast<const int *>(w + a->o_nbase);
+    D.n_mask = reinterpret_cast<const uint32_t *>(w + a->o_nmask);
+    D.nnodes = a->nnodes;
     D.l_nf = reinterpret_cast<const int *>(w + a->o_lnf);
     D.l_dir = reinterpret_cast<const int *>(w + a->o_ldir);
     D.l_nff = reinterpret_cast<const int *>(w + a->o_lnff);
@@ -707,7 +902,6 @@ AdjDev adj_dev(lbm_adj *a) {
     D.l_dqdMf = reinterpret_cast<double *>(w + a->o_dqf);
     D.l_dqdMs = reinterpret_cast<double *>(w + a->o_dqs);
     D.l_dJdq = reinterpret_cast<double *>(w + a->o_dJdq);
-    D.l_lam = reinterpret_cast<float *>(w + a->o_llam);
     D.nlinks = a->nlinks;
     D.cp = reinterpret_cast<const double *>(w + a->o_cp);
     D.K = reinterpret_cast<const double *>(w + a->o_K);
@@ -718,11 +912,56 @@ AdjDev adj_dev(lbm_adj *a) {
     return D;
 }
 
-dim3 node_grid(const lbm_adj *a) {
-    return dim3((a->cfg.nx + 31) / 32, (a->cfg.ny + 3) / 4, (a->cfg.nz + 1) / 2);
+Kept kept_slot(lbm_adj *a, int slot) {
+    char *p = a->ws + a->o_kept + a->kept * (size_t)slot;
+    const size_t L = (size_t)std::max(1, a->nlinks);
+    Kept k;
+    k.mom = reinterpret_cast<float4 *>(p);
+    p += align_up((size_t)a->N * 16);
+    k.l_f = reinterpret_cast<float4 *>(p);
+    p += align_up(L * 16);
+    k.l_ff = reinterpret_cast<float4 *>(p);
+    p += align_up(L * 16);
+    k.l_gq = reinterpret_cast<float *>(p);
+    return k;
 }
 
 float *state(lbm_adj *a, size_t off) { return reinterpret_cast<float *>(a->ws + off); }
+
+unsigned span_grid(const lbm_adj *a) { return (unsigned)((a->N + 255) / 256); }
+
+// The link kernels run with no link node too: the span kernel behind them
+// relies on their wait for the step before.
+unsigned link_grid(const lbm_adj *a, int per_block) {
+    return (unsigned)std::max(1, (a->nnodes + per_block - 1) / per_block);
+}
+
+// One forward step S -> R on the stream, one adjoint step lamN -> lamT.
+template <bool kForce, bool kWide>
+void forward_step_t(lbm_adj *a, const AdjDev &D, const float *S, float *R, const Kept &kept, int window, int t) {
+    launch_pdl(k_adj_step_links<kForce>, dim3(link_grid(a, 8 * kLinkNodes)), 256, a->stream, D, S, R, kept, window);
+    launch_pdl(k_adj_step<kForce, kWide>, dim3(span_grid(a)), 256, a->stream, D, S, R, kept, t & 1);
+}
+template <bool kForce, bool kWide>
+void adjoint_step_t(lbm_adj *a, const AdjDev &D, const Kept &kept, const float *lamN, float *lamT, float4 *share,
+                    float4 *share_next, int window, int t) {
+    launch_pdl(k_adj_back_links, dim3(link_grid(a, 8)), 256, a->stream, D, kept, lamN, lamT, share, share_next, window);
+    launch_pdl(k_adj_back<kForce, kWide>, dim3(span_grid(a)), 256, a->stream, D, kept.mom, lamN, lamT, share, t & 1);
+}
+template <typename... X>
+void forward_step(lbm_adj *a, const X &...x) {
+    const bool force = a->cfg.force[0] != 0.0 || a->cfg.force[1] != 0.0 || a->cfg.force[2] != 0.0;
+    const bool wide = a->N >= (1ll << 30);
+    if (wide) force ? forward_step_t<true, true>(a, x...) : forward_step_t<false, true>(a, x...);
+    else force ? forward_step_t<true, false>(a, x...) : forward_step_t<false, false>(a, x...);
+}
+template <typename... X>
+void adjoint_step(lbm_adj *a, const X &...x) {
+    const bool force = a->cfg.force[0] != 0.0 || a->cfg.force[1] != 0.0 || a->cfg.force[2] != 0.0;
+    const bool wide = a->N >= (1ll << 30);
+    if (wide) force ? adjoint_step_t<true, true>(a, x...) : adjoint_step_t<false, true>(a, x...);
+    else force ? adjoint_step_t<true, false>(a, x...) : adjoint_step_t<false, false>(a, x...);
+}
 
 }  // namespace
 
@@ -731,12 +970,10 @@ extern "C" {
 int lbm_adj_workspace_size(const lbm_config *cfg, const lbm_particle *p, int T, int W, size_t *bytes) {
     if (const char *m = adj_check(cfg, p, T, W)) return afail(nullptr, LBM_ERR_BAD_ARG, "%s", m);
     if (!bytes) return afail(nullptr, LBM_ERR_BAD_ARG, "bytes is NULL");
-    std::vector<uint8_t> solid;
-    std::vector<uint32_t> lmask;
-    std::vector<int> nf, dir, nff;
-    classify_links(cfg, p, solid, lmask, nf, dir, nff);
+    Links k;
+    classify_links(cfg, p, k);
     lbm_adj a;
-    adj_sizes(&a, cfg, T, W, p->n_cp, (int)nf.size());
+    adj_sizes(&a, cfg, T, W, p->n_cp, k);
     adj_layout(&a);
     *bytes = a.total;
     return LBM_OK;
@@ -749,13 +986,11 @@ int lbm_adj_init(const lbm_config *cfg, const lbm_particle *p, int T, int W, voi
     if (const char *m = adj_check(cfg, p, T, W)) return afail(nullptr, LBM_ERR_BAD_ARG, "%s", m);
     if (!dev_ws || reinterpret_cast<uintptr_t>(dev_ws) % kAlign)
         return afail(nullptr, LBM_ERR_BAD_ARG, "workspace NULL or not 256-byte aligned");
-    std::vector<uint8_t> solid;
-    std::vector<uint32_t> lmask;
-    std::vector<int> nf, dir, nff;
-    classify_links(cfg, p, solid, lmask, nf, dir, nff);
+    Links k;
+    classify_links(cfg, p, k);
     lbm_adj *a = new (std::nothrow) lbm_adj();
     if (!a) return afail(nullptr, LBM_ERR_BAD_ARG, "out of host memory");
-    adj_sizes(a, cfg, T, W, p->n_cp, (int)nf.size());
+    adj_sizes(a, cfg, T, W, p->n_cp, k);
     adj_layout(a);
     if (ws_bytes < a->total) {
         const size_t need = a->total;
@@ -766,20 +1001,19 @@ int lbm_adj_init(const lbm_config *cfg, const lbm_particle *p, int T, int W, voi
     a->stream = static_cast<cudaStream_t>(cuda_stream);
     a->have_forward = false;
     std::snprintf(a->err, sizeof(a->err), "no error");
-    std::vector<int> linkid((size_t)Q * a->N, -1);
-    for (size_t L = 0; L < nf.size(); L++) linkid[(size_t)dir[L] * a->N + nf[L]] = (int)L;
-    const size_t Lb = nf.size() * 4;
-    int rc = acheck(a, cudaMemsetAsync(a->ws, 0, a->total, a->stream), "cudaMemsetAsync");
+    int rc = LBM_OK;
     auto up = [&](size_t off, const void *src, size_t bytes) {
         if (rc == LBM_OK && bytes)
             rc = acheck(a, cudaMemcpyAsync(a->ws + off, src, bytes, cudaMemcpyHostToDevice, a->stream), "cudaMemcpyAsync");
     };
-    up(a->o_solid, solid.data(), solid.size());
-    up(a->o_lmask, lmask.data(), lmask.size() * 4);
-    up(a->o_linkid, linkid.data(), linkid.size() * 4);
-    up(a->o_lnf, nf.data(), Lb);
-    up(a->o_ldir, dir.data(), Lb);
-    up(a->o_lnff, nff.data(), Lb);
+    const size_t Lb = k.nf.size() * 4, Mb = k.node.size() * 4;
+    up(a->o_kind, k.kind.data(), k.kind.size());
+    up(a->o_nnode, k.node.data(), Mb);
+    up(a->o_nbase, k.base.data(), Mb);
+    up(a->o_nmask, k.mask.data(), Mb);
+    up(a->o_lnf, k.nf.data(), Lb);
+    up(a->o_ldir, k.dir.data(), Lb);
+    up(a->o_lnff, k.nff.data(), Lb);
     if (rc == LBM_OK) rc = acheck(a, cudaStreamSynchronize(a->stream), "cudaStreamSynchronize");
     if (rc != LBM_OK) {
         std::snprintf(g_adj_error, sizeof(g_adj_error), "%s", a->err);
@@ -805,17 +1039,18 @@ int lbm_adj_forward(lbm_adj *a, const double *cp_world, const double *K, double 
     const AdjDev D = adj_dev(a);
     const int lgrid = std::max(1, std::min(1024, (a->nlinks + 255) / 256));
     if (a->nlinks > 0) k_adj_q<<<lgrid, 256, 0, a->stream>>>(D);
-    float *s0 = state(a, a->o_state[0]), *s1 = state(a, a->o_state[1]);
-    k_adj_init<<<1216, 256, 0, a->stream>>>(D, s0, (float)a->cfg.u0[0], (float)a->cfg.u0[1], (float)a->cfg.u0[2]);
-    const dim3 grid = node_grid(a);
+    // state 0, and every K-th state of a run that keeps checkpoints, is
+    // written where the adjoint's segments start from
+    float *buf[2] = {state(a, a->o_state[0]), state(a, a->o_state[1])};
+    auto ckpt = [&](int c) { return state(a, a->o_ckpt + a->S * (size_t)c); };
+    float *src = a->keep_all ? buf[0] : ckpt(0);
+    k_adj_init<<<1216, 256, 0, a->stream>>>(D, src, (float)a->cfg.u0[0], (float)a->cfg.u0[1], (float)a->cfg.u0[2]);
+    const Kept none = {};
     for (int t = 0; t < a->T; t++) {
-        if (t % a->K == 0) {
-            rc = acheck(a, cudaMemcpyAsync(a->ws + a->o_ckpt + (size_t)(t / a->K) * a->S, s0, a->S,
-                                           cudaMemcpyDeviceToDevice, a->stream), "cudaMemcpyAsync(checkpoint)");
-            if (rc != LBM_OK) return rc;
-        }
-        k_adj_step<<<grid, 256, 0, a->stream>>>(D, s0, s1, t >= a->T - a->W ? 1 : 0);
-        std::swap(s0, s1);
+        const bool mark = !a->keep_all && (t + 1) % a->K == 0 && t + 1 < a->T;
+        float *dst = mark ? ckpt((t + 1) / a->K) : (src == buf[0] ? buf[1] : buf[0]);
+        forward_step(a, D, src, dst, a->keep_all ? kept_slot(a, t) : none, t >= a->T - a->W ? 1 : 0, t);
+        src = dst;
     }
     long long jfix = 0;
     rc = acheck(a, cudaGetLastError(), "forward launch");
@@ -834,26 +1069,32 @@ int lbm_adj_backward(lbm_adj *a, double *dJ_dcp, double *dJ_dK) {
     const AdjDev D = adj_dev(a);
     int rc = acheck(a, cudaMemsetAsync(a->ws + a->o_dJdq, 0, (size_t)std::max(1, a->nlinks) * 8, a->stream), "cudaMemsetAsync");
     if (rc == LBM_OK) rc = acheck(a, cudaMemsetAsync(a->ws + a->o_lam[0], 0, a->S, a->stream), "cudaMemsetAsync");
+    for (int k = 0; k < 2; k++)
+        if (rc == LBM_OK)
+            rc = acheck(a, cudaMemsetAsync(a->ws + a->o_share[k], 0, (size_t)a->N * 16, a->stream), "cudaMemsetAsync");
     if (rc == LBM_OK) rc = acheck(a, cudaMemsetAsync(a->ws + a->o_grad, 0, (size_t)a->ncp * 32, a->stream), "cudaMemsetAsync");
     if (rc != LBM_OK) return rc;
     float *lamN = state(a, a->o_lam[0]), *lamT = state(a, a->o_lam[1]);
-    const dim3 grid = node_grid(a);
-    const int lgrid = std::max(1, std::min(1024, (a->nlinks + 127) / 128));
-    for (int c = a->C - 1; c >= 0; c--) {
-        const int t0 = c * a->K, t1 = std::min(a->T, t0 + a->K);
-        // states t0 .. t1-1 of the segment: the checkpoint, then recomputed
-        std::vector<float *> seg((size_t)(t1 - t0));
-        seg[0] = reinterpret_cast<float *>(a->ws + a->o_ckpt + (size_t)c * a->S);
-        for (int k = 1; k < t1 - t0; k++) {
-            seg[(size_t)k] = reinterpret_cast<float *>(a->ws + a->o_seg + (size_t)(k - 1) * a->S);
-            k_adj_step<<<grid, 256, 0, a->stream>>>(D, seg[(size_t)k - 1], seg[(size_t)k], 0);
+    float4 *share = reinterpret_cast<float4 *>(a->ws + a->o_share[0]);
+    float4 *share_next = reinterpret_cast<float4 *>(a->ws + a->o_share[1]);
+    float *buf[2] = {state(a, a->o_state[0]), state(a, a->o_state[1])};
+    for (int c = a->keep_all ? 0 : a->C - 1; c >= 0; c--) {
+        const int t0 = a->keep_all ? 0 : c * a->K, t1 = a->keep_all ? a->T : std::min(a->T, t0 + a->K);
+        if (!a->keep_all) {
+            // the segment's kept data, from its checkpoint
+            const float *src = state(a, a->o_ckpt + a->S * (size_t)c);
+            for (int t = t0; t < t1; t++) {
+                float *dst = src == buf[0] ? buf[1] : buf[0];
+                forward_step(a, D, src, dst, kept_slot(a, t - t0), 0, t);
+                src = dst;
+            }
         }
         for (int t = t1 - 1; t >= t0; t--) {
             const int window = t >= a->T - a->W ? 1 : 0;
-            const float *S = seg[(size_t)(t - t0)];
-            k_adj_back<<<grid, 256, 0, a->stream>>>(D, S, lamN, lamT, window);
-            if (a->nlinks > 0) k_adj_vibb<<<lgrid, 128, 0, a->stream>>>(D, S, lamT);
+            const Kept kept = kept_slot(a, t - t0);
+            adjoint_step(a, D, kept, lamN, lamT, share, share_next, window, t);
             std::swap(lamN, lamT);
+            std::swap(share, share_next);
         }
     }
     if (a->nlinks > 0) k_adj_grad<<<std::max(1, std::min(256, (a->nlinks + 255) / 256)), 256, 0, a->stream>>>(D);

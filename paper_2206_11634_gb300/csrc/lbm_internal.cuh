@@ -677,6 +677,28 @@ __device__ __forceinline__ void brick_coords(const Params &P, int b, int &bx, in
     bz = b / (P.nbx * P.nby);
 }
 
+// Quotient by a divisor fixed on the host, for 0 <= n < 2^31, in three
+// instructions (Granlund and Montgomery, PLDI 1994) instead of the twenty-odd
+// of a division by a run-time value.
+struct FastDiv {
+    uint32_t d, m, s;
+};
+inline FastDiv fast_div(uint32_t d) {
+    FastDiv f;
+    f.d = d;
+    f.s = 0;
+    while ((1ull << f.s) < d) f.s++;
+    f.m = (uint32_t)((((1ull << f.s) - d) << 32) / d + 1);
+    return f;
+}
+__host__ __device__ __forceinline__ uint32_t fast_quot(uint32_t n, const FastDiv &f) {
+#ifdef __CUDA_ARCH__
+    return (__umulhi(f.m, n) + n) >> f.s;
+#else
+    return (uint32_t)(((uint32_t)(((uint64_t)f.m * n) >> 32) + (uint64_t)n) >> f.s);
+#endif
+}
+
 // Programmatic dependent launch.  launch_dependents: the next kernel of the
 // stream may start once every CTA of this one has called it (or ended).
 // wait: until the kernels this one was launched behind are complete and their
