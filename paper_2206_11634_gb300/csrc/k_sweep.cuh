@@ -582,72 +582,18 @@ struct LinkScratch {
     unsigned long long fix[BRICK / 32][MAXPB][6];  // the warp's fixed-point force/torque terms
 };
 
-// A fluid node with at least one particle link, in a brick some particle
-// reaches: pull, walls, VIBB / halfway bounce-back on the particle links with
-// their momentum exchange, collide, store.
-template <typename S, int Q, bool kForce>
-__device__ __noinline__ void boundary_node(const Params &P, const SmemParticles &sp, int x, int y, int z, int lx,
-                                           int ly, int lz, int bx0, int by0, int bz0, int n,
-                                           ForceSink<typename Codec<S>::C> sink, int *nlinks) {
-    using L = Lat<Q>;
-    using Cd = Codec<S>;
-    using C = typename Cd::C;
-    const S *A = (const S *)P.fA;
-    S *B = (S *)P.fB;
-    const long long N = P.N;
-    const C rho0 = Prm<C>::rho0(P);
-    int xs[3], ys[3], zs[3];
-    neighbour_coords(P, x, y, z, xs, ys, zs);
-    C fown[Q];
-    C drho_f = 0, m_f[3] = {0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < Q; k++) {
-        fown[k] = Cd::ld(A + (long long)k * N + n, (C)L::w(k), rho0);
-        drho_f += fown[k];
-        m_f[0] += fown[k] * L::e(k, 0);
-        m_f[1] += fown[k] * L::e(k, 1);
-        m_f[2] += fown[k] * L::e(k, 2);
-    }
-    C u_f[3];
-    const C inv_rho_f = C(1) / (rho0 + drho_f);
-    for (int a = 0; a < 3; a++) u_f[a] = (m_f[a] - C(0.5) * Prm<C>::F(P, a)) * inv_rho_f;
-    C fin[Q];
-    int srcs[Q];
-    uint32_t links = 0;
-    fin[0] = fown[0];
-#pragma unroll
-    for (int i = 1; i < Q; i++) {
-        const int sx = xs[1 - L::e(i, 0)], sy = ys[1 - L::e(i, 1)], sz = zs[1 - L::e(i, 2)];
-        if ((sx | sy | sz) < 0) {
-            fin[i] = fown[L::opp(i)];  // box wall: halfway bounce-back
-            srcs[i] = n;
-            continue;
-        }
-        const int src = sx + P.nx * (sy + P.ny * sz);
-        srcs[i] = src;
-        fin[i] = Cd::ld(A + (long long)i * N + src, (C)L::w(i), rho0);
-        if (P.flag_new[src] != 0) links |= 1u << i;
-    }
-    // each thread visits its own links only, so a warp runs as many link
-    // updates as its busiest node has links
-    C Mf_cache = 0;
-    int Mf_slot = -1;
-    while (links) {
-        const int i = __ffs(links) - 1;
-        links &= links - 1;
-        const FFData<C> ff = ff_fetch<S, Q>(P, x, y, z, L::opp(i));
-        fin[i] = particle_link<S, Q>(P, sp, i, x, y, z, lx, ly, lz, bx0, by0, bz0, (int)P.flag_new[srcs[i]] - 1, ff,
-                                     fown[L::opp(i)], drho_f, u_f, sink, &Mf_cache, &Mf_slot);
-        (*nlinks)++;
-    }
-#pragma unroll
-    for (int i = 0; i < Q; i++) fin[i] = Cd::g_to_v(fin[i], (C)L::w(i));
-    collide_store<S, Q, kForce>(P, fin, B, N, n);
-}
-
 // Bricks some particle reaches: nodes without particle links take the plain
-// path (plus 19 flag reads); boundary and solid nodes go out of line; then
-// the deterministic reduction of the per-particle terms.
+// path (plus 19 flag reads); the links of a warp's nodes are spread over its
+// lanes, missing force points go out of line; then the deterministic reduction
+// of the per-particle terms.
+//
+// FP64 lattices are bound by the FP64 pipe here (64 cycles a warp
+// instruction, some 250 of them a link): with every node walking its own links
+// a warp paid for its busiest node's, up to nine, and a step of the 32x32x48
+// sphere spent 328 us in this kernel; spread over the lanes 104.  A
+// link's result waits in its node's own slot of the array being written
+// (which nothing reads in this step): no limit on a warp's links, and no
+// shared memory for FP64 results.
 template <typename S, int Q, bool kForce>
 __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, double (*red)[6], int *s_links,
                                         LinkScratch *ls, int b, int bx0, int by0, int bz0, int cnt) {
@@ -666,7 +612,7 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
     const C rho0 = Prm<C>::rho0(P);
 
     C acc[MAXPB][6];  // FP64 only
-    const ForceSink<C> sink{acc, ls->fix[warp]};
+    const ForceSink<C> sink{acc, ls->fix[warp], nullptr};
     if (sizeof(C) == 8) {
         for (int s = 0; s < cnt; s++)
             for (int c = 0; c < 6; c++) acc[s][c] = 0;
@@ -681,7 +627,6 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
     // brick's particles are loaded, so the two latencies overlap
     constexpr uint32_t kWall = 0xFFFFFFFFu;
     uint32_t nf[Q];
-    C fin[Q];
     {
         int xs[3], ys[3], zs[3];
         neighbour_coords(P, x, y, z, xs, ys, zs);
@@ -691,16 +636,6 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
             const int sx = xs[1 - L::e(i, 0)], sy = ys[1 - L::e(i, 1)], sz = zs[1 - L::e(i, 2)];
             const bool wall = (sx | sy | sz) < 0;
             nf[i] = (!active || wall) ? kWall : (uint32_t)P.flag_new[sx + P.nx * (sy + P.ny * sz)];
-        }
-        if (sizeof(C) == 8 && active) {  // FP64: the pulls in the same round
-#pragma unroll
-            for (int i = 0; i < Q; i++) {
-                const int sx = xs[1 - L::e(i, 0)], sy = ys[1 - L::e(i, 1)], sz = zs[1 - L::e(i, 2)];
-                const bool wall = (sx | sy | sz) < 0;
-                const S *ptr = wall ? A + (long long)L::opp(i) * N + n
-                                    : A + (long long)i * N + (sx + P.nx * (sy + P.ny * sz));
-                fin[i] = Cd::ld(ptr, (C)L::w(i), rho0);
-            }
         }
     }
     load_particle_records(P, sp, cnt, bx0, by0, bz0);  // ids staged by the caller
@@ -730,15 +665,7 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
             if (cand) nterms += solid_links<S, Q>(P, sp, s, j == owner, cand, lx, ly, lz, bx0, by0, bz0, sink);
         }
     }
-    if (sizeof(C) == 8) {
-        // FP64 storage: every node evaluates its own links
-        if (links) boundary_node<S, Q, kForce>(P, sp, x, y, z, lx, ly, lz, bx0, by0, bz0, n, sink, &nlinks);
-        else if (fluid) {
-#pragma unroll
-            for (int i = 0; i < Q; i++) fin[i] = Cd::g_to_v(fin[i], (C)L::w(i));
-            collide_store<S, Q, kForce>(P, fin, B, N, n);
-        }
-    } else {
+    {
         // the warp's links in a queue (lane order, then direction order);
         // all 32 lanes evaluate them, then each node takes its results back
         const int mine = __popc(links);
@@ -771,14 +698,20 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
                 const int t = warp * 32 + L_;  // the node's thread index in the brick
                 ForceSink<C> ds = sink;
                 ds.defer = &lt;
-                ls->result[warp][e] = (float)link_coop<S, Q>(P, sp, i, t % BX, (t / BX) % BY, t / (BX * BY), bx0,
-                                                             by0, bz0, ds);
+                const C val = link_coop<S, Q>(P, sp, i, t % BX, (t / BX) % BY, t / (BX * BY), bx0, by0, bz0, ds);
+                if (sizeof(C) == 8) {
+                    const int tn = (bx0 + t % BX) + P.nx * ((by0 + (t / BX) % BY) + P.ny * (bz0 + t / (BX * BY)));
+                    Cd::st(B + (long long)i * N + tn, val, (C)0, rho0);
+                } else {
+                    ls->result[warp][e] = (float)val;
+                }
                 nlinks++;
             }
-            warp_add_terms(ls->fix[warp], cnt, lt, lane);
+            if (sizeof(C) == 4) warp_add_terms(ls->fix[warp], cnt, lt, lane);
         }
         __syncwarp();
         if (fluid) {
+            C fin[Q];
             // pull after the link evaluation: populations held across the
             // out-of-line link calls would be spilled around them
             int xs[3], ys[3], zs[3];
@@ -787,7 +720,9 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
 #pragma unroll
             for (int i = 0; i < Q; i++) {
                 if (links & (1u << i)) {  // link results are offsets g
-                    fin[i] = Cd::g_to_v((C)ls->result[warp][k], (C)L::w(i));
+                    const C g = sizeof(C) == 8 ? Cd::ld_plain(B + (long long)i * N + n, (C)L::w(i), rho0)
+                                               : (C)ls->result[warp][k];
+                    fin[i] = Cd::g_to_v(g, (C)L::w(i));
                     k++;
                 } else {
                     const int sx = xs[1 - L::e(i, 0)], sy = ys[1 - L::e(i, 1)], sz = zs[1 - L::e(i, 2)];
