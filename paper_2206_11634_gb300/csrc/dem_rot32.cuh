@@ -1,0 +1,235 @@
+// Rotation sub-steps of a free particle in FP32 pairs.
+//
+// An FP64 warp instruction holds its SM sub-partition for 64 cycles on this
+// GPU and the n_s sub-steps of a step are one chain (26 such instructions
+// each), so in FP64 they took 110 us per step for n_s = 100.  Here a sub-step is
+// about 600 FP32 instructions (three components side by side).  A step of one particle with n_s = 100, the DEM kernel of an
+// FP64 lattice: 114 -> 62 us.
+//
+// The scheme is that of rotate_free_quad (k_particles.cu), in the variables
+//   u = h w_b / 2 (the half angle of a sub-step), tau = (h/2)^2 T_b,
+//   d = (c, s): s = u sin|u| / |u|, c = cos|u|:
+//     uh  = u + G + P(u)                  G_l = tau_l / I_l
+//     tau' = tau - 2 c s x tau + 2 s x (s x tau)
+//     u'  = uh + G' + P(uh + G' + P(uh))  P_l(u) = cI_l u_{l+1} u_{l+2}
+//     D'  = D (x) d.
+// What makes pairs of FP32 enough is what they hold: not the state, but its
+// change within the step.
+//   u = U_0 + 2 k G_0 + delta after k sub-steps, U_0 and G_0 in FP64 and put
+//   together in FP64 at the end; delta holds the gyroscopic terms and the
+//   turning of the torque, a small part of u;
+//   tau = tau_0 + theta; D = (sqrt(1 - |beta|^2), beta) from the identity, so
+//   |beta| is the half angle of the whole step, and q_0 (x) D is formed in FP64.
+// A pair carries 2^-48 of delta, theta and beta, which are at most 2^-8 of the
+// state under the conditions of rot32_applies: below FP64's rounding of the
+// state in each of its n_s steps.  Products that enter them are pairs too;
+// single FP32 is left for terms of second order (P(uh) - P(u) inside the inner
+// fixed-point sweep, s x (s x tau), 1 - c, |s| - |u|, (1 - D_0) s), whose
+// rounding is under 2^-54 of the state by the same conditions.  Measured
+// against 128-bit arithmetic over 1 to 400 sub-steps and angular velocities
+// from rest to the limit: see tests/test_rot32.py, which compiles this file
+// for the host.
+#pragma once
+
+#ifdef __CUDACC__
+#define ROT32_FN __host__ __device__ __forceinline__
+#else
+#include <cmath>
+#define ROT32_FN inline
+#endif
+
+namespace lbmmb {
+
+// value = h + l, |l| <= ulp(h) (not always rounded to nearest)
+struct Pair {
+    float h, l;
+};
+
+ROT32_FN float rot_fma(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(a, b, c);
+#else
+    return std::fmaf(a, b, c);
+#endif
+}
+ROT32_FN float rot_add(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    volatile float r = a + b;
+    return r;
+#endif
+}
+ROT32_FN float rot_mul(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    volatile float r = a * b;
+    return r;
+#endif
+}
+// v as a pair (on the device without FP64 conversions, see from_double)
+ROT32_FN Pair rot_split(double v) {
+    Pair p;
+#ifdef __CUDA_ARCH__
+    p.h = from_double<float>(v);
+    p.l = from_double<float>(v - to_double(p.h));
+#else
+    p.h = (float)v;
+    p.l = (float)(v - (double)p.h);
+#endif
+    return p;
+}
+// a + b exactly as h + l (Knuth)
+ROT32_FN Pair two_sum(float a, float b) {
+    Pair r;
+    r.h = rot_add(a, b);
+    const float bb = rot_add(r.h, -a);
+    r.l = rot_add(rot_add(a, -rot_add(r.h, -bb)), rot_add(b, -bb));
+    return r;
+}
+ROT32_FN Pair renorm(Pair a) {
+    Pair r;
+    r.h = rot_add(a.h, a.l);
+    r.l = rot_add(a.l, -rot_add(r.h, -a.h));
+    return r;
+}
+ROT32_FN Pair padd(Pair a, Pair b) {
+    Pair s = two_sum(a.h, b.h);
+    s.l = rot_add(s.l, rot_add(a.l, b.l));
+    return renorm(s);
+}
+ROT32_FN Pair pmul(Pair a, Pair b) {
+    Pair r;
+    r.h = rot_mul(a.h, b.h);
+    r.l = rot_fma(a.l, b.h, rot_fma(a.h, b.l, rot_fma(a.h, b.h, -r.h)));
+    return r;
+}
+// a x b - c x d
+ROT32_FN Pair pcross(Pair a, Pair b, Pair c, Pair d) {
+    const Pair p = pmul(a, b), q = pmul(c, d);
+    Pair s = two_sum(p.h, -q.h);
+    s.l = rot_add(s.l, rot_add(p.l, -q.l));
+    return renorm(s);
+}
+
+struct Rot32 {
+    Pair cI[3], iI[3];   // Euler coefficients, 1 / I
+    Pair U0[3], G0[3];   // at the start: h w_b / 2, (h/2)^2 T_b / I
+    Pair t0[3];          // (h/2)^2 T_b
+};
+struct Rot32Result {
+    Pair delta[3], beta[3];
+    bool ok;
+};
+
+constexpr float kRot32MaxHalfAngle2 = 1.0f / (1 << 30);  // |uh| <= 2^-15 in every sub-step
+
+// Whether the pairs carry FP64's accuracy: u0max is |h w_b / 2| at the start
+// plus the torque's share over the step; half the limits on a sub-step's and
+// the whole step's half angle are left to the gyroscopic terms, which cannot
+// double |w_b| within so small an angle (|cI| <= 1 as of any mass
+// distribution).  Fewer than kRot32MinSub sub-steps are left in FP64, where
+// the last roundings weigh more than the sub-steps' and the time is short
+// (n_s = 1 and 2 measured within 1.7 of FP64's error, from 10 on below it).
+constexpr int kRot32MinSub = 8;
+ROT32_FN bool rot32_applies(float u0max, int n_sub, float cImax) {
+    return n_sub >= kRot32MinSub && u0max <= 1.0f / (1 << 16) && u0max * (float)n_sub <= 1.0f / (1 << 9) &&
+           cImax <= 1.0001f;
+}
+
+ROT32_FN Rot32Result rot32_run(const Rot32 &R, int n_sub) {
+    Rot32Result o;
+    const Pair zero = {0.f, 0.f};
+    Pair base[3], th[3], g[3], u[3], P[3];
+#pragma unroll
+    for (int l = 0; l < 3; l++) {
+        o.delta[l] = o.beta[l] = th[l] = g[l] = zero;
+        base[l] = u[l] = R.U0[l];
+    }
+    o.ok = true;
+    for (int k = 0; k < n_sub; k++) {
+        float e0[3];
+        Pair uh[3], E[3];
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            const int a = (l + 1) % 3, b = (l + 2) % 3;
+            P[l] = pmul(pmul(R.cI[l], u[a]), u[b]);
+        }
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            E[l] = padd(R.G0[l], padd(g[l], P[l]));  // uh - u
+            uh[l] = padd(u[l], E[l]);
+            e0[l] = E[l].h;
+        }
+        const float a2 = rot_fma(uh[0].h, uh[0].h, rot_fma(uh[1].h, uh[1].h, rot_mul(uh[2].h, uh[2].h)));
+        if (!(a2 <= kRot32MaxHalfAngle2)) {
+            o.ok = false;
+            return o;
+        }
+        const float es = rot_mul(a2, rot_fma(a2, 1.0f / 120.0f, -1.0f / 6.0f));
+        const float cm1 = rot_mul(a2, rot_fma(a2, 1.0f / 24.0f, -0.5f));
+        Pair s[3], t[3], X[3];
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            s[l].h = uh[l].h;
+            s[l].l = rot_fma(uh[l].h, es, uh[l].l);
+            t[l] = padd(R.t0[l], th[l]);
+        }
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            const int a = (l + 1) % 3, b = (l + 2) % 3;
+            X[l] = pcross(s[a], t[b], s[b], t[a]);
+        }
+        Pair g1[3];
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            const int a = (l + 1) % 3, b = (l + 2) % 3;
+            // 2 s x X - 2 (c - 1) X
+            const float Y = rot_fma(s[a].h, X[b].h, -rot_mul(s[b].h, X[a].h));
+            const float corr = rot_mul(2.0f, rot_fma(-cm1, X[l].h, Y));
+            const Pair dt = {rot_mul(-2.0f, X[l].h), rot_fma(-2.0f, X[l].l, corr)};
+            th[l] = padd(th[l], dt);
+            g1[l] = pmul(R.iI[l], th[l]);
+        }
+        Pair v1[3];
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            const int a = (l + 1) % 3, b = (l + 2) % 3;
+            // P(uh) = P(u) + cI (u_a e_b + e_a u_b + e_a e_b), the second term in FP32
+            const float dP = rot_mul(R.cI[l].h, rot_fma(u[a].h, e0[b], rot_mul(e0[a], rot_add(u[b].h, e0[b]))));
+            Pair q = P[l];
+            q.l = rot_add(q.l, dP);
+            v1[l] = padd(uh[l], padd(R.G0[l], padd(g1[l], renorm(q))));
+        }
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            const int a = (l + 1) % 3, b = (l + 2) % 3;
+            const Pair P1 = pmul(pmul(R.cI[l], v1[a]), v1[b]);
+            // delta' = delta + g + g' + P(u) + P(v1)
+            o.delta[l] = padd(o.delta[l], padd(padd(g[l], g1[l]), padd(P[l], P1)));
+        }
+        // D (x) d: beta + s + beta x s + (D_0 - 1) s + (c - 1) beta
+        const float d0m1 = rot_mul(-0.5f, rot_fma(o.beta[0].h, o.beta[0].h,
+                                                  rot_fma(o.beta[1].h, o.beta[1].h, rot_mul(o.beta[2].h, o.beta[2].h))));
+        Pair nb[3];
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            const int a = (l + 1) % 3, b = (l + 2) % 3;
+            Pair w = pcross(o.beta[a], s[b], o.beta[b], s[a]);
+            w.l = rot_add(w.l, rot_fma(d0m1, s[l].h, rot_mul(cm1, o.beta[l].h)));
+            nb[l] = padd(o.beta[l], padd(renorm(s[l]), w));
+        }
+#pragma unroll
+        for (int l = 0; l < 3; l++) {
+            o.beta[l] = nb[l];
+            const Pair g2 = {2.0f * R.G0[l].h, 2.0f * R.G0[l].l};
+            base[l] = padd(base[l], g2);
+            g[l] = g1[l];
+            u[l] = padd(base[l], o.delta[l]);
+        }
+    }
+    return o;
+}
+
+}  // namespace lbmmb

@@ -7,6 +7,7 @@
 //                  Euler's equations in the body frame (Eq. (1)).
 #include "k_flags.cuh"
 #include "dem_fp64.cuh"
+#include "dem_rot32.cuh"
 
 namespace lbmmb {
 
@@ -646,23 +647,11 @@ __device__ __forceinline__ double dneg_if(double v, bool neg) {
     return __longlong_as_double(__double_as_longlong(v) ^ (neg ? (long long)0x8000000000000000ull : 0ll));
 }
 
-// Tw_lane: this lane's component of the world-frame torque (lane 0: not
-// used); the new attitude and world angular velocity go to q_out[4] and
-// w_out[3] (which may be p's own).
-__device__ void rotate_free_quad(unsigned mk, const DevParticle &p, double Tw_lane, double h, int n_sub,
-                                 double *q_out, double *w_out) {
-    const QuadLanes L = quad_lanes();
+// The quads of mk: n_sub sub-steps of (q, wb) under the body-frame torque Tb.
+__device__ void rotate_sub_steps(unsigned mk, const QuadLanes &L, const DevParticle &p, double h, int n_sub, double &q,
+                                 double &wb, double Tb) {
     const int lane = L.lane;
     const int m = lane == 0 ? 0 : lane - 1;
-    double q = p.q[lane];
-    const double Tw = lane == 0 ? 0.0 : Tw_lane;
-    double wb = qrotate(mk, L, q, lane == 0 ? 0.0 : p.w[m], false);
-    double Tb = qrotate(mk, L, q, Tw, false);
-    if (__all_sync(mk, wb == 0.0 && Tb == 0.0)) {  // nothing turns
-        q_out[lane] = q;
-        if (lane > 0) w_out[m] = p.w[m];
-        return;
-    }
     const double hh = 0.5 * h, qh2 = 0.25 * h * h;
     // per-lane constants (lane 0 holds the quaternion's scalar part only)
     const double cIhh = lane == 0 ? 0.0 : hh * p.cI[m];
@@ -721,6 +710,100 @@ __device__ void rotate_free_quad(unsigned mk, const DevParticle &p, double Tw_la
         const double dp1 = qget(mk, d, L.p1), dp2 = qget(mk, d, L.p2), dp3 = qget(mk, d, L.p3);
         q = fma(dneg_if(q3, neg3), dp3, fma(dneg_if(q2, neg2), dp2, fma(dneg_if(q1, neg1), dp1, q0 * d)));
     }
+}
+
+// The same in FP32 pairs (dem_rot32.cuh) for the quads where they carry
+// FP64's accuracy: lane 0 of a quad runs its particle's sub-steps.  Returns
+// whether this quad was taken.
+__device__ bool rotate_pairs(unsigned mk, const QuadLanes &L, const DevParticle &p, double h, int n_sub, double &q,
+                             double &wb, double Tb) {
+    const int lane = L.lane;
+    const int m = lane == 0 ? 0 : lane - 1;
+    const float c = lane == 0 ? 0.f : p.cI_f[m], dw = lane == 0 ? 0.f : p.iI_f[m] * from_double<float>(Tb);
+    const float w = lane == 0 ? 0.f : from_double<float>(wb), hh_f = 0.5f / (float)n_sub;
+    float w2 = w * w, d2 = dw * dw, cm = fabsf(c);
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+        w2 += __shfl_xor_sync(mk, w2, o, 4);
+        d2 += __shfl_xor_sync(mk, d2, o, 4);
+        cm = fmaxf(cm, __shfl_xor_sync(mk, cm, o, 4));
+    }
+    const bool fits = rot32_applies(hh_f * (sqrtf(w2) + sqrtf(d2)), n_sub, cm);
+    const unsigned mf = __ballot_sync(mk, fits);
+    if (!fits) return false;
+    // this lane's component as pairs, gathered by lane 0
+    const double hh = 0.5 * h, t = hh * hh * Tb;
+    const Pair mine[5] = {rot_split(p.cI[m]), rot_split(p.iI[m]), rot_split(hh * wb), rot_split(t * p.iI[m]),
+                          rot_split(t)};
+    Rot32 R;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        Pair got[5];
+#pragma unroll
+        for (int k = 0; k < 5; k++) {
+            got[k].h = __shfl_sync(mf, mine[k].h, 1 + a, 4);
+            got[k].l = __shfl_sync(mf, mine[k].l, 1 + a, 4);
+        }
+        R.cI[a] = got[0];
+        R.iI[a] = got[1];
+        R.U0[a] = got[2];
+        R.G0[a] = got[3];
+        R.t0[a] = got[4];
+    }
+    Rot32Result r = {};
+    if (lane == 0) r = rot32_run(R, n_sub);
+    __syncwarp(mf);
+    Pair db[2];  // this lane's delta and beta (lane 0: unused)
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const Pair d = {__shfl_sync(mf, r.delta[a].h, 0, 4), __shfl_sync(mf, r.delta[a].l, 0, 4)};
+        const Pair b = {__shfl_sync(mf, r.beta[a].h, 0, 4), __shfl_sync(mf, r.beta[a].l, 0, 4)};
+        if (m == a) {
+            db[0] = d;
+            db[1] = b;
+        }
+    }
+    const bool ok = __shfl_sync(mf, (int)r.ok, 0, 4) != 0;
+    // w_b: the start's, the torque's (n_s sub-steps of h T / I, h = 1 / n_s)
+    // and delta = h/2 of the rest
+    const double delta = to_double(db[0].h) + to_double(db[0].l);
+    const double beta = lane == 0 ? 0.0 : to_double(db[1].h) + to_double(db[1].l);
+    const double wn = fma(2.0 * n_sub, delta, fma(p.iI[m], Tb, wb));
+    // D = (sqrt(1 - |beta|^2), beta), |beta|^2 <= 2^-16: the next term of the
+    // series is below 2^-69
+    const double b2 = qsum3(mf, L, beta * beta);
+    const double al = -b2 * fma(b2, fma(b2, fma(b2, 5.0 / 128.0, 1.0 / 16.0), 1.0 / 8.0), 0.5);
+    const double d = lane == 0 ? 1.0 + al : beta;
+    const double q0 = qget(mf, q, 0), q1 = qget(mf, q, 1), q2 = qget(mf, q, 2), q3 = qget(mf, q, 3);
+    const double dp1 = qget(mf, d, L.p1), dp2 = qget(mf, d, L.p2), dp3 = qget(mf, d, L.p3);
+    if (!ok) return false;
+    q = fma(dneg_if(q3, L.s3 < 0.0), dp3, fma(dneg_if(q2, L.s2 < 0.0), dp2, fma(dneg_if(q1, L.s1 < 0.0), dp1, q0 * d)));
+    wb = wn;
+    return true;
+}
+
+// A free particle's rotation over one step by its quad of lanes; mk holds the
+// lanes of every quad of this warp that takes part.  Tw_lane: this lane's
+// component of the world-frame torque (lane 0: not used); the new attitude and
+// world angular velocity go to q_out[4] and w_out[3] (which may be p's own).
+__device__ void rotate_free_quad(unsigned mk, const DevParticle &p, double Tw_lane, double h, int n_sub,
+                                 double *q_out, double *w_out) {
+    const QuadLanes L = quad_lanes();
+    const int lane = L.lane;
+    const int m = lane == 0 ? 0 : lane - 1;
+    double q = p.q[lane];
+    const double Tw = lane == 0 ? 0.0 : Tw_lane;
+    double wb = qrotate(mk, L, q, lane == 0 ? 0.0 : p.w[m], false);
+    const double Tb = qrotate(mk, L, q, Tw, false);
+    if (__all_sync(mk, wb == 0.0 && Tb == 0.0)) {  // nothing turns
+        q_out[lane] = q;
+        if (lane > 0) w_out[m] = p.w[m];
+        return;
+    }
+    const bool done = rotate_pairs(mk, L, p, h, n_sub, q, wb, Tb);
+    const unsigned rest = __ballot_sync(mk, !done);
+    if (!done) rotate_sub_steps(rest, L, p, h, n_sub, q, wb, Tb);
+    __syncwarp(mk);
     // renormalise once per LBM step, back to world frame
     double n2 = q * q;
     n2 += __shfl_xor_sync(mk, n2, 1, 4);
