@@ -316,10 +316,10 @@ const char *lbm_last_error(const lbm_handle *h);
  * phase is one kernel launch for all cases.  The particles being fixed, the
  * node flags cannot change: the first three steps after particles are set run
  * the flag pass, later steps leave it out (as lbm_step() does for a lattice
- * whose particles are all fixed).  Those static steps run as replays of a
- * CUDA graph of 16 steps captured on first use (the step numbers live in
- * device counters, so the same graph serves every later call); a remainder of
- * fewer than 16 steps is launched directly.  The paper steps one lattice; the
+ * whose particles are all fixed) and run two kernels each, launched one while
+ * the one before still runs.  (A batch whose recorded geometry does not fit
+ * replays a CUDA graph of 16 brick-sweep steps instead; a remainder of
+ * fewer than 16 steps is launched directly.)  The paper steps one lattice; the
  * batched form has no counterpart there.
  *
  * All cases share the lattice (D3Q19 or D3Q15) and the storage (FP32, FP16

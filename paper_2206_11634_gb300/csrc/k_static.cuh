@@ -157,9 +157,8 @@ template <typename S, int Q, bool kForce>
 __device__ __forceinline__ void static_plain_node(const Params &P, int n) {
     if (n >= P.N) return;
     const bool skip = P.sskip[n] != 0;
-    const int nxy = P.nx * P.ny;
-    const int z = n / nxy, r = n - z * nxy;
-    const int y = r / P.nx, x = r - y * P.nx;
+    const int z = (int)fast_quot((uint32_t)n, P.by_nxy), r = n - z * P.nx * P.ny;
+    const int y = (int)fast_quot((uint32_t)r, P.by_nx), x = r - y * P.nx;
     typename Codec<S>::C fin[Q];
     plain_pull<S, Q, true>(P, x, y, z, n, fin);
     if (!skip) collide_store<S, Q, kForce, true>(P, fin, (S *)P.fB, P.N, n);
@@ -394,6 +393,12 @@ __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links(Params P
 // batched lattices: the same two kernels over all cases
 // ---------------------------------------------------------------------------
 
+// The two kernels of a step wait for one another as the single lattice's do
+// (k_static_plain).  The step's parity comes with the launch: step numbers are
+// not needed here, and counting a step's CTAs down to advance a device
+// counter, one atomic on one address per CTA, took 7 % of a step (64 boxes,
+// FP32, ms a step: 1.558, without it 1.453; FP16 1.208, 1.103).
+
 // plain_chunk spans per CTA as k_sweep_plain_batch; the CTA holding a case's
 // first span also clears that case's per-step region for the next step (the
 // binning, which clears it otherwise, does not run in fixed-geometry steps).
@@ -402,9 +407,9 @@ __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links(Params P
 // 64-case batch (six spilled 88 bytes and was 2-6 % slower).
 template <typename S, int Q, bool kForce>
 __global__ void __launch_bounds__(BRICK, 5) k_static_plain_batch(BatchArgs B) {
+    pdl_launch_dependents();
     const int total = B.span_off[B.ncases];
-    const unsigned step = *(volatile const unsigned *)(B.ctr + 1);
-    const Params *row = B.tab + (size_t)(step & 1) * B.ncases;
+    const Params *row = B.tab + (size_t)B.parity * B.ncases;
     const int g0 = blockIdx.x * B.plain_chunk;
     const int g1 = min(total, g0 + B.plain_chunk);
     // the case's parameters in shared memory (re-read when the CTA's spans
@@ -430,32 +435,25 @@ __global__ void __launch_bounds__(BRICK, 5) k_static_plain_batch(BatchArgs B) {
         }
         static_plain_node<S, Q, kForce>(P, (g - B.span_off[c]) * BRICK + (int)threadIdx.x);
     }
-    advance_step_when_last(B.ctr + 3, B.ctr + 1);
+    pdl_wait();
 }
 
-// One warp per kStaticNodesPerWarp link nodes of a case (each case at least one warp, whose
-// first also adds the case's constant parts); the last CTA advances the
-// particle chain's step counter.
+// One warp per kStaticNodesPerWarp link nodes of a case (each case at least one
+// warp, which also adds the case's constant parts).
 template <typename S, int Q, bool kForce>
 __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links_batch(BatchArgs B) {
     __shared__ StaticScratch ss;
-    const unsigned step = *(volatile const unsigned *)B.ctr;
-    const Params *row = B.tab + (size_t)(step & 1) * B.ncases;
+    pdl_wait();
+    pdl_launch_dependents();
+    const Params *row = B.tab + (size_t)B.parity * B.ncases;
     const int warps = B.swarp_off[B.ncases];
     const int gw = blockIdx.x * (BRICK / 32) + (int)(threadIdx.x >> 5);
-    if (gw < warps) {
-        int lo = 0, hi = B.ncases - 1;  // the case whose warp range holds gw
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) / 2;
-            if (B.swarp_off[mid] <= gw) lo = mid;
-            else hi = mid - 1;
-        }
-        const Params &P = row[lo];
-        const int wl = gw - B.swarp_off[lo];
-        if (wl == 0) static_constants(P, threadIdx.x & 31, 32);
-        if (wl * kStaticNodesPerWarp < P.snodes_n) static_links_warp<S, Q, kForce, kStaticNodesPerWarp>(P, ss, wl);
-    }
-    advance_step_when_last(B.ctr + 2, B.ctr);
+    if (gw >= warps) return;
+    const int c = case_of(B.swarp_off, B.ncases, gw);  // whose warp range holds gw
+    const Params &P = row[c];
+    const int wl = gw - B.swarp_off[c];
+    if (wl == 0) static_constants(P, threadIdx.x & 31, 32);
+    if (wl * kStaticNodesPerWarp < P.snodes_n) static_links_warp<S, Q, kForce, kStaticNodesPerWarp>(P, ss, wl);
 }
 
 }  // namespace lbmmb

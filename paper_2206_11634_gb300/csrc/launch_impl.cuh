@@ -168,22 +168,22 @@ void launch_static_links_t(const Params &P, cudaStream_t st) {
 template <typename S>
 void launch_static_plain_batch_t(const BatchArgs &B, int Q, bool force, int grid, cudaStream_t st) {
     if (Q == 19) {
-        if (force) k_static_plain_batch<S, 19, true><<<grid, BRICK, 0, st>>>(B);
-        else k_static_plain_batch<S, 19, false><<<grid, BRICK, 0, st>>>(B);
+        if (force) launch_pdl(k_static_plain_batch<S, 19, true>, grid, BRICK, st, B);
+        else launch_pdl(k_static_plain_batch<S, 19, false>, grid, BRICK, st, B);
     } else {
-        if (force) k_static_plain_batch<S, 15, true><<<grid, BRICK, 0, st>>>(B);
-        else k_static_plain_batch<S, 15, false><<<grid, BRICK, 0, st>>>(B);
+        if (force) launch_pdl(k_static_plain_batch<S, 15, true>, grid, BRICK, st, B);
+        else launch_pdl(k_static_plain_batch<S, 15, false>, grid, BRICK, st, B);
     }
 }
 template <typename S>
 void launch_static_links_batch_t(const BatchArgs &B, int Q, bool force, int warps, cudaStream_t st) {
     const int grid = (warps + BRICK / 32 - 1) / (BRICK / 32);
     if (Q == 19) {
-        if (force) k_static_links_batch<S, 19, true><<<grid, BRICK, 0, st>>>(B);
-        else k_static_links_batch<S, 19, false><<<grid, BRICK, 0, st>>>(B);
+        if (force) launch_pdl(k_static_links_batch<S, 19, true>, grid, BRICK, st, B);
+        else launch_pdl(k_static_links_batch<S, 19, false>, grid, BRICK, st, B);
     } else {
-        if (force) k_static_links_batch<S, 15, true><<<grid, BRICK, 0, st>>>(B);
-        else k_static_links_batch<S, 15, false><<<grid, BRICK, 0, st>>>(B);
+        if (force) launch_pdl(k_static_links_batch<S, 15, true>, grid, BRICK, st, B);
+        else launch_pdl(k_static_links_batch<S, 15, false>, grid, BRICK, st, B);
     }
 }
 

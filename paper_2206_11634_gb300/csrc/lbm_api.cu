@@ -1264,7 +1264,7 @@ struct lbm_batch {
     int g_chain, plain_chunk;
     int total_spans, bin_items, total_swarps;
     int static_state;            // fixed-geometry sweep of all cases: 0 not built, 1 built, -1 did not fit
-    bool graph_fixed;            // the captured graph runs the fixed-geometry sweep
+    int64_t ctr_steps;           // step number that the device counters hold
     std::vector<Params> tab_host;  // the device table's rows
     bool dirty;
     int64_t steps;
@@ -1412,6 +1412,7 @@ BatchArgs batch_args(lbm_batch *b) {
     B.ctr = reinterpret_cast<unsigned *>(b->ws + b->ctr_off);
     B.g_chain = b->g_chain;
     B.plain_chunk = b->plain_chunk;
+    B.parity = 0;
     B.swarp_off = reinterpret_cast<const int *>(b->ws + b->swarp_off);
     return B;
 }
@@ -1441,26 +1442,28 @@ void by_batch_storage(int storage, Fn &&fn) {
     }
 }
 
-// nsteps steps on the batch's streams, forked from and joined into b->cap
-// (the sequence a graph is captured from).
-int batch_issue(lbm_batch *b, int nsteps, bool flags, bool fixed) {
+// nsteps steps of the fixed-geometry sweep on b->cap, the first of them step
+// number `first`: the link and the plain kernel in stream order (k_static.cuh).
+int batch_issue_fixed(lbm_batch *b, int nsteps, int64_t first) {
+    BatchArgs B = batch_args(b);
+    const int plain_grid = (b->total_spans + b->plain_chunk - 1) / b->plain_chunk;
+    for (int t = 0; t < nsteps; t++) {
+        B.parity = (int)((first + t) & 1);
+        by_batch_storage(b->storage, [&](auto D) { D.static_links(B, b->Q, b->force, b->total_swarps, b->cap); });
+        by_batch_storage(b->storage, [&](auto D) { D.static_plain(B, b->Q, b->force, plain_grid, b->cap); });
+    }
+    return bcheck(b, cudaGetLastError(), "batched step launch");
+}
+
+// nsteps steps of the brick sweeps on the batch's streams, forked from and
+// joined into b->cap (the sequence a graph is captured from).
+int batch_issue(lbm_batch *b, int nsteps, bool flags) {
     const BatchArgs B = batch_args(b);
     const int plain_grid = (b->total_spans + b->plain_chunk - 1) / b->plain_chunk;
     cudaError_t e = cudaEventRecord(b->ev_fork, b->cap);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->hi, b->ev_fork, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->aux, b->ev_fork, 0);
-    for (int t = 0; fixed && t < nsteps && e == cudaSuccess; t++) {
-        // fixed-geometry sweep: the link nodes after the previous step's plain
-        // nodes, the plain nodes after the previous step's link nodes
-        if (t > 0) e = cudaStreamWaitEvent(b->hi, b->ev_plain, 0);
-        if (e == cudaSuccess && t > 0) e = cudaStreamWaitEvent(b->aux, b->ev_near, 0);
-        if (e != cudaSuccess) break;
-        by_batch_storage(b->storage, [&](auto D) { D.static_links(B, b->Q, b->force, b->total_swarps, b->hi); });
-        by_batch_storage(b->storage, [&](auto D) { D.static_plain(B, b->Q, b->force, plain_grid, b->aux); });
-        e = cudaEventRecord(b->ev_plain, b->aux);
-        if (e == cudaSuccess) e = cudaEventRecord(b->ev_near, b->hi);
-    }
-    for (int t = 0; !fixed && t < nsteps && e == cudaSuccess; t++) {
+    for (int t = 0; t < nsteps && e == cudaSuccess; t++) {
         launch_bin_batch(B, b->bin_items, b->hi);
         e = cudaEventRecord(b->ev_bin, b->hi);
         if (e != cudaSuccess) break;
@@ -1581,11 +1584,11 @@ int lbm_batch_init(const lbm_config *cfgs, int ncases, void *dev_ws, size_t ws_b
     for (int c = 0; c < ncases; c++)
         for (int a = 0; a < 3; a++) b->force = b->force || cfgs[c].force[a] != 0.0;
     b->g_chain = kDefaultBatchChainCtas;
-    b->plain_chunk = kDefaultBatchPlainChunk;
+    b->plain_chunk = storage_bytes(cfgs[0].storage) == 2 ? kDefaultBatchPlainChunk16 : kDefaultBatchPlainChunk;
     b->steps = 0;
     b->static_steps = 0;
     b->static_state = 0;
-    b->graph_fixed = false;
+    b->ctr_steps = 0;
     b->total_swarps = 0;
     std::snprintf(b->err, sizeof(b->err), "no error");
     int rc = LBM_OK;
@@ -1653,46 +1656,65 @@ int lbm_batch_step(lbm_batch *b, int nsteps) {
     // every particle of a batch is fixed: the first kStaticFlagSteps steps
     // after particles are set run the flag pass (then both flag buffers and
     // the per-brick solid marks hold the flags); the fixed geometry is then
-    // recorded once, and the later steps run the fixed-geometry sweep (or the
-    // brick sweeps without the flag pass, if it did not fit), as replays of
-    // one captured graph of kBatchGraphSteps steps and a direct remainder
+    // recorded once, and the later steps run the fixed-geometry sweep.  If it
+    // did not fit they run the brick sweeps without the flag pass, as replays
+    // of one captured graph of kBatchGraphSteps steps and a direct remainder
     const int direct = std::min(nsteps, std::max(0, kStaticFlagSteps - b->static_steps));
-    if (direct > 0) rc = batch_issue(b, direct, true, false);
+    // the brick sweeps take their step numbers from device counters, which the
+    // fixed-geometry sweep leaves alone
+    auto set_counters = [&](int64_t at) {
+        if (b->ctr_steps == at) return (int)LBM_OK;
+        const unsigned v[4] = {(unsigned)at, (unsigned)at, 0u, 0u};
+        b->ctr_steps = at;
+        return bcheck(b, cudaMemcpyAsync(b->ws + b->ctr_off, v, sizeof(v), cudaMemcpyHostToDevice, b->cap),
+                      "cudaMemcpyAsync(counters)");
+    };
+    if (direct > 0) {
+        rc = set_counters(b->steps);
+        if (rc == LBM_OK) rc = batch_issue(b, direct, true);
+        b->ctr_steps += direct;
+    }
     if (rc != LBM_OK) return rc;
     if (direct < nsteps && b->static_state == 0) {
         rc = batch_build_static(b, b->steps + direct);
         if (rc != LBM_OK) return rc;
     }
-    const bool fixed = b->static_state == 1;
-    const int reps = (nsteps - direct) / kBatchGraphSteps;
-    const int rest = (nsteps - direct) % kBatchGraphSteps;
-    if (reps > 0 && b->exec && b->graph_fixed != fixed) drop_graph(b);
-    if (reps > 0 && !b->exec) {
-        // replays read the step numbers from the device counters, so the same
-        // graph serves every later call
-        cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return bcheck(b, e, "cudaStreamBeginCapture");
-        const int rc_issue = batch_issue(b, kBatchGraphSteps, false, fixed);
-        cudaGraph_t g = nullptr;
-        e = cudaStreamEndCapture(b->cap, &g);
-        if (rc_issue != LBM_OK) {
-            if (g) cudaGraphDestroy(g);
-            return rc_issue;
+    if (b->static_state == 1) {
+        rc = batch_issue_fixed(b, nsteps - direct, b->steps + direct);
+        if (rc != LBM_OK) return rc;
+    } else if (direct < nsteps) {
+        rc = set_counters(b->steps + direct);
+        if (rc != LBM_OK) return rc;
+        const int reps = (nsteps - direct) / kBatchGraphSteps;
+        const int rest = (nsteps - direct) % kBatchGraphSteps;
+        if (reps > 0 && !b->exec) {
+            // replays read the step numbers from the device counters, so the
+            // same graph serves every later call
+            cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
+            if (e != cudaSuccess) return bcheck(b, e, "cudaStreamBeginCapture");
+            const int rc_issue = batch_issue(b, kBatchGraphSteps, false);
+            cudaGraph_t g = nullptr;
+            e = cudaStreamEndCapture(b->cap, &g);
+            if (rc_issue != LBM_OK) {
+                if (g) cudaGraphDestroy(g);
+                return rc_issue;
+            }
+            if (e != cudaSuccess) return bcheck(b, e, "cudaStreamEndCapture");
+            b->graph = g;
+            // the kernel nodes keep the priorities of the streams they were
+            // captured from (the particle chain above the plain sweep)
+            e = cudaGraphInstantiateWithFlags(&b->exec, g, cudaGraphInstantiateFlagUseNodePriority);
+            if (e != cudaSuccess) {
+                drop_graph(b);
+                return bcheck(b, e, "cudaGraphInstantiate");
+            }
+            b->graph_steps = kBatchGraphSteps;
         }
-        if (e != cudaSuccess) return bcheck(b, e, "cudaStreamEndCapture");
-        b->graph = g;
-        // the kernel nodes keep the priorities of the streams they were
-        // captured from (the particle chain above the plain sweep)
-        e = cudaGraphInstantiateWithFlags(&b->exec, g, cudaGraphInstantiateFlagUseNodePriority);
-        if (e != cudaSuccess) {
-            drop_graph(b);
-            return bcheck(b, e, "cudaGraphInstantiate");
-        }
-        b->graph_steps = kBatchGraphSteps;
-        b->graph_fixed = fixed;
+        for (int k = 0; k < reps && rc == LBM_OK; k++)
+            rc = bcheck(b, cudaGraphLaunch(b->exec, b->cap), "cudaGraphLaunch");
+        if (rc == LBM_OK && rest > 0) rc = batch_issue(b, rest, false);
+        b->ctr_steps += nsteps - direct;
     }
-    for (int k = 0; k < reps && rc == LBM_OK; k++) rc = bcheck(b, cudaGraphLaunch(b->exec, b->cap), "cudaGraphLaunch");
-    if (rc == LBM_OK && rest > 0) rc = batch_issue(b, rest, false, fixed);
     if (rc == LBM_OK) rc = bcheck(b, cudaEventRecord(b->ev_post, b->cap), "cudaEventRecord");
     if (rc == LBM_OK) rc = bcheck(b, cudaStreamWaitEvent(b->stream, b->ev_post, 0), "cudaStreamWaitEvent");
     if (rc != LBM_OK) return rc;

@@ -82,7 +82,9 @@ constexpr int kDefaultPlainPerSm = 0;
 // Batched lattices: CTAs per case of the flag and near sweeps, bricks per CTA
 // of the plain sweep (lbm_batch_tune chooses them by measurement).
 constexpr int kDefaultBatchChainCtas = 4;
-constexpr int kDefaultBatchPlainChunk = 2;
+// 64 boxes of sides 48-128, ms a step with 1 / 2 / 4 / 8 spans a CTA: FP32
+// 1.487 / 1.453 / 1.485 / 1.541, FP16 1.193 / 1.103 / 1.081 / 1.076.
+constexpr int kDefaultBatchPlainChunk = 2, kDefaultBatchPlainChunk16 = 4;
 constexpr int kDefaultChainPerSm = 0;
 
 // FP32 DEM limits: its per-particle tables live in one CTA's shared memory.
@@ -318,11 +320,34 @@ struct DevParticle {
     double nx[3], nv[3], nq[4], nw[3];
 };
 
+// Quotient by a divisor fixed on the host, for 0 <= n < 2^31, in three
+// instructions (Granlund and Montgomery, PLDI 1994) instead of the twenty-odd
+// of a division by a run-time value.
+struct FastDiv {
+    uint32_t d, m, s;
+};
+inline FastDiv fast_div(uint32_t d) {
+    FastDiv f;
+    f.d = d;
+    f.s = 0;
+    while ((1ull << f.s) < d) f.s++;
+    f.m = (uint32_t)((((1ull << f.s) - d) << 32) / d + 1);
+    return f;
+}
+__host__ __device__ __forceinline__ uint32_t fast_quot(uint32_t n, const FastDiv &f) {
+#ifdef __CUDA_ARCH__
+    return (__umulhi(f.m, n) + n) >> f.s;
+#else
+    return (uint32_t)(((uint32_t)(((uint64_t)f.m * n) >> 32) + (uint64_t)n) >> f.s);
+#endif
+}
+
 // Everything a kernel needs, passed by value.
 struct Params {
     int nx, ny, nz, Q;
     int per[3];
     long long N;
+    FastDiv by_nxy, by_nx;    // a node index to (x, y, z)
     int nbx, nby, nbz, nbricks;
     int np, n_sub, vibb, missing_force;
     int q_exact;              // link fraction by Newton on Eq. (26) instead of Eq. (27)
@@ -427,6 +452,8 @@ inline void fill_scalar_params(const lbm_config &c, Params &P) {
     P.nx = c.nx; P.ny = c.ny; P.nz = c.nz; P.Q = c.lattice;
     for (int a = 0; a < 3; a++) P.per[a] = c.periodic[a] != 0;
     P.N = (long long)c.nx * c.ny * c.nz;
+    P.by_nxy = fast_div((uint32_t)((long long)c.nx * c.ny));
+    P.by_nx = fast_div((uint32_t)c.nx);
     P.nbx = (c.nx + BX - 1) / BX;
     P.nby = (c.ny + BY - 1) / BY;
     P.nbz = (c.nz + BZ - 1) / BZ;
@@ -677,28 +704,6 @@ __device__ __forceinline__ void brick_coords(const Params &P, int b, int &bx, in
     bz = b / (P.nbx * P.nby);
 }
 
-// Quotient by a divisor fixed on the host, for 0 <= n < 2^31, in three
-// instructions (Granlund and Montgomery, PLDI 1994) instead of the twenty-odd
-// of a division by a run-time value.
-struct FastDiv {
-    uint32_t d, m, s;
-};
-inline FastDiv fast_div(uint32_t d) {
-    FastDiv f;
-    f.d = d;
-    f.s = 0;
-    while ((1ull << f.s) < d) f.s++;
-    f.m = (uint32_t)((((1ull << f.s) - d) << 32) / d + 1);
-    return f;
-}
-__host__ __device__ __forceinline__ uint32_t fast_quot(uint32_t n, const FastDiv &f) {
-#ifdef __CUDA_ARCH__
-    return (__umulhi(f.m, n) + n) >> f.s;
-#else
-    return (uint32_t)(((uint32_t)(((uint64_t)f.m * n) >> 32) + (uint64_t)n) >> f.s);
-#endif
-}
-
 // Programmatic dependent launch.  launch_dependents: the next kernel of the
 // stream may start once every CTA of this one has called it (or ended).
 // wait: until the kernels this one was launched behind are complete and their
@@ -749,6 +754,7 @@ struct BatchArgs {
     int plain_chunk;        // spans per CTA of the plain sweep
     const int *swarp_off;   // [ncases + 1] prefix sums of the cases' link-node warps (>= 1 each;
                             // fixed-geometry sweep)
+    int parity;             // fixed-geometry sweep: parity of the step
 };
 
 // The case's Params for the current step into shared memory (all threads).

@@ -80,3 +80,30 @@ def test_back_to_back_steps_same_bits(pkg, box):
         torch.cuda.synchronize()
     for x, y in zip(state(a), state(b)):
         assert np.array_equal(x, y)
+
+
+def test_batch_particles_set_again(pkg):
+    """A batch whose particles are set again after an odd number of
+    fixed-geometry steps (which do not advance the brick sweeps' step counters):
+    the same bits as single lattices through the same calls."""
+    def held(n, shift):
+        return pkg.make_particle([[0, 0, 0], [1.0, 0.5, 0]], [8.0, 9.0], (n / 2 + shift, n / 2 - 0.3, n / 2 + 0.1),
+                                 fixed=1, mass=1.0, inertia=np.eye(3))
+    sizes = [24, 33, 29]
+    kw = [dict(nx=n, ny=n, nz=n, storage="f32", periodic=(1, 1, 1), tau=0.8, force=(1e-5, 0, 0), n_sub=0,
+               max_particles=1) for n in sizes]
+    bt = pkg.Batch(kw)
+    singles = [pkg.Lattice(k["nx"], k["ny"], k["nz"], **{a: v for a, v in k.items() if a not in ("nx", "ny", "nz")})
+               for k in kw]
+    for shift, calls in ((0.2, (3, 4, 1)), (0.9, (1, 6, 17, 2)), (-0.4, (20,))):
+        for c, n in enumerate(sizes):
+            bt.set_particles(c, [held(n, shift)])
+            singles[c].set_particles([held(n, shift)])
+        for k in calls:
+            bt.step(k)
+            for lat in singles:
+                lat.step(k)
+        for c, lat in enumerate(singles):
+            assert np.array_equal(bt.populations(c).cpu().numpy(), lat.populations().cpu().numpy())
+            for a, b in zip(bt.forces(c), lat.forces()):
+                assert np.array_equal(a, b)
