@@ -326,9 +326,9 @@ __device__ __forceinline__ FFData<typename Codec<S>::C> ff_fetch(const Params &P
         for (int k = 0; k < Q; k++) {
             const C fk = Cd::ld(A + (long long)k * P.N + nff, (C)L::w(k), rho0);
             f.drho += fk;
-            f.m[0] += fk * L::e(k, 0);
-            f.m[1] += fk * L::e(k, 1);
-            f.m[2] += fk * L::e(k, 2);
+            f.m[0] = add_e(f.m[0], L::e(k, 0), fk);
+            f.m[1] = add_e(f.m[1], L::e(k, 1), fk);
+            f.m[2] = add_e(f.m[2], L::e(k, 2), fk);
             if (k == io) f.g_io = fk;
         }
     }
@@ -559,9 +559,9 @@ __device__ __noinline__ typename Codec<S>::C link_coop(const Params &P, const Sm
     for (int k = 0; k < Q; k++) {
         const C fk = Cd::ld(A + (long long)k * N + n, (C)L::w(k), rho0);
         drho_f += fk;
-        m_f[0] += fk * L::e(k, 0);
-        m_f[1] += fk * L::e(k, 1);
-        m_f[2] += fk * L::e(k, 2);
+        m_f[0] = add_e(m_f[0], L::e(k, 0), fk);
+        m_f[1] = add_e(m_f[1], L::e(k, 1), fk);
+        m_f[2] = add_e(m_f[2], L::e(k, 2), fk);
         if (k == io) fown_io = fk;
     }
     C u_f[3];
@@ -573,19 +573,29 @@ __device__ __noinline__ typename Codec<S>::C link_coop(const Params &P, const Sm
                                &Mf_cache, &Mf_slot);
 }
 
-// Shared scratch of the warp-cooperative link evaluation: per warp a queue of
-// (lane, direction) link entries and their results.
+// Links a warp's nodes can have.
 constexpr int kLinkQueue = 32 * 18;
+// Shared scratch of the cooperative link evaluation: the brick's links in
+// thread order, then direction order, as (thread << 5) | direction, and their
+// results.
 struct LinkScratch {
-    unsigned short entry[BRICK / 32][kLinkQueue];
-    float result[BRICK / 32][kLinkQueue];
+    unsigned short entry[BRICK / 32 * kLinkQueue];
+    float result[BRICK / 32 * kLinkQueue];
+    int warp_links[BRICK / 32];
     unsigned long long fix[BRICK / 32][MAXPB][6];  // the warp's fixed-point force/torque terms
 };
 
 // Bricks some particle reaches: nodes without particle links take the plain
-// path (plus 19 flag reads); the links of a warp's nodes are spread over its
-// lanes, missing force points go out of line; then the deterministic reduction
-// of the per-particle terms.
+// path (plus 19 flag reads); the links of the brick's nodes are spread over its
+// threads, missing force points go out of line; then the deterministic
+// reduction of the per-particle terms.
+//
+// A brick has some 64 links: in one queue they are two warps' worth of the
+// link code (about 1400 instructions), in a queue per warp they were six to
+// eight warps' with most lanes idle, competing for the issue slots.  One queue,
+// and one-subtraction indices for the flags and pulls: 200 metaballs in 256^3
+// 566 -> 492 us, one metaball in 128x128x256 22.8 -> 18.3, the FP64 sphere 91 ->
+// 69.
 //
 // FP64 lattices are bound by the FP64 pipe here (64 cycles a warp
 // instruction, some 250 of them a link): with every node walking its own links
@@ -627,7 +637,24 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
     // brick's particles are loaded, so the two latencies overlap
     constexpr uint32_t kWall = 0xFFFFFFFFu;
     uint32_t nf[Q];
-    {
+    if (P.idx32 && y > 0 && y < P.ny - 1 && z > 0 && z < P.nz - 1) {
+        // a row off the y and z faces (a warp is a row): one subtraction per
+        // neighbour, corrected on the x-face lanes (plain_pull's indices).
+        // Lanes past the row's end read inside the lattice too.
+        const int nx = P.nx, nxy = P.nx * P.ny;
+        int cm = 0, cp = 0;
+        bool wm = false, wp = false;
+        if (x == 0) { if (P.per[0]) cm = nx; else wm = true; }
+        if (x == nx - 1) { if (P.per[0]) cp = -nx; else wp = true; }
+        nf[0] = active ? (uint32_t)P.flag_new[(unsigned)n] : 1u;
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            const int ex = L::e(i, 0);
+            const uint32_t f = P.flag_new[(unsigned)(n - (ex + nx * L::e(i, 1) + nxy * L::e(i, 2)) +
+                                                    (ex > 0 ? cm : (ex < 0 ? cp : 0)))];
+            nf[i] = (!active || (ex > 0 && wm) || (ex < 0 && wp)) ? kWall : f;
+        }
+    } else {
         int xs[3], ys[3], zs[3];
         neighbour_coords(P, x, y, z, xs, ys, zs);
         nf[0] = active ? (uint32_t)P.flag_new[n] : 1u;
@@ -666,8 +693,8 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
         }
     }
     {
-        // the warp's links in a queue (lane order, then direction order);
-        // all 32 lanes evaluate them, then each node takes its results back
+        // the brick's links in one queue; each warp evaluates 32 of them at a
+        // time, then each node takes its results back
         const int mine = __popc(links);
         int incl = mine;
 #pragma unroll
@@ -675,27 +702,36 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += v;
         }
-        const int first = incl - mine;
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        if (lane == 31) ls->warp_links[warp] = incl;
+        __syncthreads();
+        int first = incl - mine, total = 0;
+#pragma unroll
+        for (int w = 0; w < BRICK / 32; w++) {
+            const int v = ls->warp_links[w];
+            if (w < warp) first += v;
+            total += v;
+        }
         {
             uint32_t m = links;
             for (int k = first; m; k++) {
                 const int i = __ffs(m) - 1;
                 m &= m - 1;
-                ls->entry[warp][k] = (unsigned short)((lane << 5) | i);
+                ls->entry[k] = (unsigned short)((tid << 5) | i);
             }
         }
-        __syncwarp();
-        // rounds of 32 links; each round's force terms are summed over the
-        // warp (no per-link atomics on the warp's totals)
-        for (int r = 0; r < total; r += 32) {
+        __syncthreads();
+        // the force terms of a warp's 32 links are summed over the warp (no
+        // per-link atomics on the warp's totals).  The first warps of the two
+        // CTAs of an SM would share its sub-partitions: half the grid starts
+        // two further on (exact sums only: FP64 partials keep one order).
+        const int turn = sizeof(C) == 8 || blockIdx.x >= gridDim.x / 2 ? warp : (warp + BRICK / 32 - 2) % (BRICK / 32);
+        for (int r = turn * 32; r < total; r += BRICK) {
             const int e = r + lane;
             LinkTerms lt;
             lt.s = -1;
             if (e < total) {
-                const int ent = ls->entry[warp][e];
-                const int L_ = ent >> 5, i = ent & 31;
-                const int t = warp * 32 + L_;  // the node's thread index in the brick
+                const int ent = ls->entry[e];
+                const int t = ent >> 5, i = ent & 31;  // the node's thread in the brick, the direction
                 ForceSink<C> ds = sink;
                 ds.defer = &lt;
                 const C val = link_coop<S, Q>(P, sp, i, t % BX, (t / BX) % BY, t / (BX * BY), bx0, by0, bz0, ds);
@@ -703,33 +739,26 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
                     const int tn = (bx0 + t % BX) + P.nx * ((by0 + (t / BX) % BY) + P.ny * (bz0 + t / (BX * BY)));
                     Cd::st(B + (long long)i * N + tn, val, (C)0, rho0);
                 } else {
-                    ls->result[warp][e] = (float)val;
+                    ls->result[e] = (float)val;
                 }
                 nlinks++;
             }
             if (sizeof(C) == 4) warp_add_terms(ls->fix[warp], cnt, lt, lane);
         }
-        __syncwarp();
+        __syncthreads();
         if (fluid) {
-            C fin[Q];
             // pull after the link evaluation: populations held across the
             // out-of-line link calls would be spilled around them
-            int xs[3], ys[3], zs[3];
-            neighbour_coords(P, x, y, z, xs, ys, zs);
+            C fin[Q];
+            plain_pull<S, Q, false>(P, x, y, z, n, fin);
             int k = first;
 #pragma unroll
-            for (int i = 0; i < Q; i++) {
+            for (int i = 1; i < Q; i++) {
                 if (links & (1u << i)) {  // link results are offsets g
                     const C g = sizeof(C) == 8 ? Cd::ld_plain(B + (long long)i * N + n, (C)L::w(i), rho0)
-                                               : (C)ls->result[warp][k];
+                                               : (C)ls->result[k];
                     fin[i] = Cd::g_to_v(g, (C)L::w(i));
                     k++;
-                } else {
-                    const int sx = xs[1 - L::e(i, 0)], sy = ys[1 - L::e(i, 1)], sz = zs[1 - L::e(i, 2)];
-                    const bool wall = (sx | sy | sz) < 0;
-                    const S *ptr = wall ? A + (long long)L::opp(i) * N + n
-                                        : A + (long long)i * N + (sx + P.nx * (sy + P.ny * sz));
-                    fin[i] = Cd::ldv(ptr, (C)L::w(i), rho0);
                 }
             }
             collide_store<S, Q, kForce>(P, fin, B, N, n);  // collide-space values
