@@ -29,11 +29,19 @@
 #include "k_plain.cuh"
 
 namespace lbmmb {
-// Resident CTAs per SM of the near sweep: its link evaluation needs more than
-// the 64 registers per thread that four 256-thread CTAs leave (it spilled to
-// local memory there, and one brick's latency sets the step when few bricks
-// are near), so it is compiled for two.
+// Resident CTAs per SM of the fixed-geometry link kernels and of the batched
+// near sweep.
 constexpr int kNearCtasPerSm = 2;
+// ... and of the near sweep, by the near bricks expected (P.near_many).  A few
+// bricks wait for one brick's latency, which registers shorten (two CTAs: 128
+// registers; FP64 one CTA: 255); thousands wait for the latencies of all, and
+// more CTAs overlap more of them although they spill (four: 64 registers).
+// Near sweep in us at 2 / 3 / 4 CTAs: 200 metaballs in 256^3 417 / 357 / 320, 50
+// in 128x128x256 122 / 113 / 112, 12 there 47 / 49 / 57, one there 15.9 / 17.8 /
+// 18.1; FP64 at 1 / 2: one sphere in 32x32x48 43 / 60, 25 metaballs in 128^3 451 /
+// 413.
+template <typename S, bool kMany>
+constexpr int kNearCtas = sizeof(S) == 8 ? (kMany ? 2 : 1) : (kMany ? 4 : 2);
 
 template <typename C>
 __device__ __forceinline__ C warp_sum(C v) {
@@ -531,7 +539,7 @@ __device__ __noinline__ int solid_links(const Params &P, const SmemParticles &sp
 // the solid node and x_ff's flag and populations are all fetched in one
 // round, then the link is evaluated as in particle_link.
 template <typename S, int Q>
-__device__ __noinline__ typename Codec<S>::C link_coop(const Params &P, const SmemParticles &sp, int i, int lx, int ly,
+__device__ __forceinline__ typename Codec<S>::C link_coop(const Params &P, const SmemParticles &sp, int i, int lx, int ly,
                                                       int lz, int bx0, int by0, int bz0,
                                                       ForceSink<typename Codec<S>::C> sink) {
     using L = Lat<Q>;
@@ -595,7 +603,8 @@ struct LinkScratch {
 // eight warps' with most lanes idle, competing for the issue slots.  One queue,
 // and one-subtraction indices for the flags and pulls: 200 metaballs in 256^3
 // 566 -> 492 us, one metaball in 128x128x256 22.8 -> 18.3, the FP64 sphere 91 ->
-// 69.
+// 69.  All of it inline (calls saved and restored most registers, and below FP64
+// the unused FP64 partials held 384 bytes of stack a thread): 417, 15.9, 60.
 //
 // FP64 lattices are bound by the FP64 pipe here (64 cycles a warp
 // instruction, some 250 of them a link): with every node walking its own links
@@ -605,7 +614,7 @@ struct LinkScratch {
 // (which nothing reads in this step): no limit on a warp's links, and no
 // shared memory for FP64 results.
 template <typename S, int Q, bool kForce>
-__device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, double (*red)[6], int *s_links,
+__device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, double (*red)[6], int *s_links,
                                         LinkScratch *ls, int b, int bx0, int by0, int bz0, int cnt) {
     using L = Lat<Q>;
     using Cd = Codec<S>;
@@ -621,7 +630,7 @@ __device__ __noinline__ void near_brick(const Params &P, SmemParticles &sp, doub
     S *B = (S *)P.fB;
     const C rho0 = Prm<C>::rho0(P);
 
-    C acc[MAXPB][6];  // FP64 only
+    C acc[sizeof(C) == 8 ? MAXPB : 1][6];  // FP64 only
     const ForceSink<C> sink{acc, ls->fix[warp], nullptr};
     if (sizeof(C) == 8) {
         for (int s = 0; s < cnt; s++)
@@ -895,8 +904,8 @@ __device__ __forceinline__ void near_work(const Params &P, SmemParticles &sp, do
     }
     if (tid == 0 && done) atomicAdd(&P.counters[CNT_NEAR], done);
 }
-template <typename S, int Q, bool kForce>
-__global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_sweep_near(Params P) {
+template <typename S, int Q, bool kForce, bool kMany>
+__global__ void __launch_bounds__(BRICK, kNearCtas<S, kMany>) k_sweep_near(Params P) {
     __shared__ SmemParticles sp;
     __shared__ double red[BRICK / 32][6];
     __shared__ int s_links;

@@ -47,18 +47,27 @@ void launch_sweep_plain_t(const Params &P, cudaStream_t st) {
         else k_sweep_plain<S, 15, false><<<grid, BRICK, 0, st>>>(P);
     }
 }
-template <typename S>
-void launch_sweep_near_t(const Params &P, cudaStream_t st) {
+template <typename S, bool kMany>
+void launch_sweep_near_n(const Params &P, cudaStream_t st) {
     const bool force = P.F[0] != 0.0 || P.F[1] != 0.0 || P.F[2] != 0.0;
-    const int cap = P.chain_grid > 0 ? P.chain_grid : kNearCtasPerSm * sm_count();
+    const int cap = P.chain_grid > 0 ? P.chain_grid : kNearCtas<S, kMany> * sm_count();
     const int grid = P.nbricks < cap ? P.nbricks : cap;
     if (P.Q == 19) {
-        if (force) k_sweep_near<S, 19, true><<<grid, BRICK, 0, st>>>(P);
-        else k_sweep_near<S, 19, false><<<grid, BRICK, 0, st>>>(P);
+        if (force) k_sweep_near<S, 19, true, kMany><<<grid, BRICK, 0, st>>>(P);
+        else k_sweep_near<S, 19, false, kMany><<<grid, BRICK, 0, st>>>(P);
     } else {
-        if (force) k_sweep_near<S, 15, true><<<grid, BRICK, 0, st>>>(P);
-        else k_sweep_near<S, 15, false><<<grid, BRICK, 0, st>>>(P);
+        if (force) k_sweep_near<S, 15, true, kMany><<<grid, BRICK, 0, st>>>(P);
+        else k_sweep_near<S, 15, false, kMany><<<grid, BRICK, 0, st>>>(P);
     }
+}
+template <typename S>
+void launch_sweep_near_t(const Params &P, cudaStream_t st) {
+    // FP64 is bound by one brick's FP64 instructions while each SM has at most
+    // one of them; the others' turning point lies between the 2700 bricks
+    // expected for 12 metaballs (two CTAs faster) and the 11600 for 50
+    const int many = sizeof(S) == 8 ? sm_count() + 1 : 40 * sm_count();
+    if (P.near_expected >= many) launch_sweep_near_n<S, true>(P, st);
+    else launch_sweep_near_n<S, false>(P, st);
 }
 // persistent, at the plain sweep's occupancy (4 CTAs per SM)
 template <typename S>

@@ -207,6 +207,7 @@ struct lbm_handle {
     int nsm;       // SMs of the device
     int plain_per_sm, chain_per_sm;  // launch schedule (lbm_set_schedule)
     int bin_clean[2];     // the per-step region of that parity is known to be all zero
+    int near_expected;    // near bricks to expect (set_particles)
     int plain_spec;       // the particles' search boxes cover under a tenth of the bricks (set_particles)
     int plain_after_near; // the plain sweep of a step follows its near sweep (else runs beside the chain)
     int plain_spec_mode;  // lbm_set_plain_speculation: -1 auto (plain_spec), 0 off, 1 on
@@ -302,6 +303,7 @@ Params make_params(lbm_handle *h) {
     P.plain_grid = h->plain_per_sm > 0 ? h->plain_per_sm * h->nsm : 0;
     P.chain_grid = h->chain_per_sm > 0 ? h->chain_per_sm * h->nsm : 0;
     P.plain_spec = h->plain_spec_mode >= 0 ? h->plain_spec_mode : h->plain_spec;
+    P.near_expected = h->near_expected;
     P.idx32 = (long long)c.lattice * (long long)c.nx * c.ny * c.nz <= 0x7fffffffLL;
     P.status = at<int>(h, h->L.status);
     P.counters = at<int>(h, bin_region(h, h->steps) + (size_t)h->L.nbricks * 4);
@@ -543,6 +545,7 @@ int init_handle(const lbm_config *cfg, void *dev_ws, size_t ws_bytes, void *cuda
         h->plain_per_sm = kDefaultPlainPerSm;
         h->chain_per_sm = kDefaultChainPerSm;
         h->plain_spec = 1;
+        h->near_expected = 0;
         h->plain_after_near = 1;
         h->plain_spec_mode = -1;
         h->bin_clean[0] = h->bin_clean[1] = 1;  // the workspace is cleared below
@@ -622,15 +625,11 @@ __global__ void k_clear_ranges(ClearRanges R) {
             R.p[r][k] = 0u;
 }
 
-// Whether the plain sweep may issue its pulls before it knows if the near
-// sweep takes the brick: worth it when the near set is a small share of the
-// bricks (its pulls are then wasted on few bricks), not when many particles
-// fill the box.  Estimated from each particle's bounding sphere (control
-// points, the radius where M falls to c0, Rs) plus two nodes of margin,
-// counted in whole bricks.
-static int plain_speculates(const lbm_config &c, const lbm_particle *host, int n) {
+// Near bricks to expect: from each particle's bounding sphere (control points,
+// the radius where M falls to c0, Rs) plus two nodes of margin, counted in whole
+// bricks (bricks shared by particles count for each).
+static double near_bricks_expected(const lbm_config &c, const lbm_particle *host, int n) {
     const int nbx = (c.nx + BX - 1) / BX, nby = (c.ny + BY - 1) / BY, nbz = (c.nz + BZ - 1) / BZ;
-    const double nbricks = (double)nbx * nby * nbz;
     double near = 0.0;
     for (int j = 0; j < n; j++) {
         const lbm_particle &p = host[j];
@@ -643,7 +642,7 @@ static int plain_speculates(const lbm_config &c, const lbm_particle *host, int n
         near += std::fmin(std::ceil(d / BX) + 1, nbx) * std::fmin(std::ceil(d / BY) + 1, nby) *
                 std::fmin(std::ceil(d / BZ) + 1, nbz);
     }
-    return near < 0.1 * nbricks ? 1 : 0;
+    return near;
 }
 
 int lbm_set_particles(lbm_handle *h, const lbm_particle *host, int n) {
@@ -796,7 +795,12 @@ int lbm_set_particles(lbm_handle *h, const lbm_particle *host, int n) {
     h->all_fixed = 1;
     for (int j = 0; j < n; j++)
         if (!host[j].fixed) h->all_fixed = 0;
-    h->plain_spec = plain_speculates(h->cfg, host, n);
+    // the plain sweep may issue its pulls before it knows if the near sweep
+    // takes the brick when the near set is a small share of the bricks (its
+    // pulls are then wasted on few), not when many particles fill the box
+    const double near = near_bricks_expected(h->cfg, host, n);
+    h->near_expected = (int)std::fmin(near, 1e9);
+    h->plain_spec = near < 0.1 * (double)h->L.nbricks ? 1 : 0;
     // with few near bricks the flag pass and near sweep are short and run
     // faster alone, and the plain sweep then overlaps the DEM and the next
     // binning and flag pass; with many, the near sweep is long and the plain

@@ -354,6 +354,7 @@ struct Params {
     int plain_grid;           // CTAs of k_sweep_plain (0: one per brick)
     int chain_grid;           // CTAs of the persistent k_flags / k_sweep_near (0: default)
     int plain_spec;           // few near bricks expected: the plain sweep pulls before its skip entry arrives
+    int near_expected;        // near bricks expected (an upper estimate from the particles' extent)
     int idx32;                // Q N < 2^31: population indices fit 32 bits
     int dem_mode;             // enum DemKernel: which DEM kernels run
     int fc_valid;             // Fc/Tc hold the contact load of the current state (0 after set_particles)

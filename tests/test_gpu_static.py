@@ -107,3 +107,21 @@ def test_batch_particles_set_again(pkg):
             assert np.array_equal(bt.populations(c).cpu().numpy(), lat.populations().cpu().numpy())
             for a, b in zip(bt.forces(c), lat.forces()):
                 assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("storage,Q", [("f32", 19), ("f32", 15), ("f16", 19), ("bf16", 15)])
+def test_many_near_bricks_same_bits(pkg, monkeypatch, storage, Q):
+    # about 9 700 near bricks expected: beyond the count from which the near
+    # sweep runs four CTAs per SM instead of two
+    monkeypatch.setitem(BOXES, "many", (97, 89, 91, (1, 0, 1), [
+        (16.2 + 32.1 * i, 14.7 + 29.3 * j, 23.1 + 45.2 * k, 13.0 + 0.2 * i)
+        for i in range(3) for j in range(3) for k in range(2)]))
+    runs = []
+    for fixed in (1, 0):
+        lat = lattice(pkg, "many", storage, Q, fixed)
+        lat.step(5)
+        runs.append(state(lat))
+    (f1, F1, T1, n1), (f0, F0, T0, n0) = runs
+    assert n1 == n0 and n1 > 0
+    assert np.array_equal(f1, f0)
+    assert np.array_equal(F1, F0) and np.array_equal(T1, T0)
