@@ -13,10 +13,10 @@ template <typename S, int Q>
 __global__ void __launch_bounds__(BRICK) k_flags_batch(BatchArgs B) {
     __shared__ Params sP;
     __shared__ SmemParticles sp;
-    __shared__ int s_next[2];
+    __shared__ Claim s_next[2];
     const int c = blockIdx.x / B.g_chain, lb = blockIdx.x % B.g_chain;
     load_case_params(B, c, B.ctr, sP);
-    flags_work<S, Q>(sP, sp, s_next, lb);
+    flags_work<S, Q>(sP, sp, s_next, lb, B.g_chain);
 }
 
 // g_chain CTAs per case over its near bricks; the last CTA of the launch
@@ -28,10 +28,10 @@ __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_sweep_near_batch(Batc
     __shared__ double red[BRICK / 32][6];
     __shared__ int s_links;
     __shared__ LinkScratch ls;
-    __shared__ int s_next[2];
+    __shared__ NearStage st;
     const int c = blockIdx.x / B.g_chain;
     load_case_params(B, c, B.ctr, sP);
-    near_work<S, Q, kForce>(sP, sp, red, s_links, ls, s_next);
+    near_work<S, Q, kForce>(sP, sp, red, s_links, ls, st, B.g_chain);
     advance_step_when_last(B.ctr + 2, B.ctr);
 }
 

@@ -42,18 +42,63 @@ __device__ __forceinline__ C geq_i(int ex, int ey, int ez, C w, C drho, C rho, C
 // low-y, high-y, low-z or high-z face.
 constexpr uint32_t kSolidAny = 0x80u;
 
+// M in FP64 out of line: few nodes need it, and inline it and the refill held
+// registers that other CTAs can use.
+__device__ __noinline__ inline double metaball64_far(const Params &P, const DevParticle &p, int x, int y, int z) {
+    return metaball64(P, p, (double)x, (double)y, (double)z);
+}
+
+// Local refilling, §2.3.3.  Reading: f_i' at x_new counts as known
+// (Eq. (30)) when it streams in from x_new + e_i and that node was a fluid
+// node of the previous step; then f_i = f_i'(x_new+e_i) + 6 w_i rho0
+// e_i.u_w, else f_i = f^eq_i(rho0, u_new); u_w = u_new is the surface
+// velocity at x_new of the particle that uncovered it.  The values become
+// the node's post-collision populations.
 template <typename S, int Q>
-__device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, int b) {
+__device__ __noinline__ void refill_node(const Params &P, int x, int y, int z, long long n, int old) {
     using L = Lat<Q>;
     using Cd = Codec<S>;
     using C = typename Cd::C;
-    constexpr bool kF64 = sizeof(C) == 8;
+    const DevParticle &pj = P.parts[old - 1];
+    double r[3] = {minimg_d(P, 0, (double)x - pj.x[0]), minimg_d(P, 1, (double)y - pj.x[1]),
+                   minimg_d(P, 2, (double)z - pj.x[2])};
+    const C ux = (C)(pj.v[0] + pj.w[1] * r[2] - pj.w[2] * r[1]);
+    const C uy = (C)(pj.v[1] + pj.w[2] * r[0] - pj.w[0] * r[2]);
+    const C uz = (C)(pj.v[2] + pj.w[0] * r[1] - pj.w[1] * r[0]);
+    const C rho0 = (C)P.rho0;
+    S *A = (S *)P.fA;
+    const long long N = P.N;
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+        const int ex = L::e(i, 0), ey = L::e(i, 1), ez = L::e(i, 2);
+        int sx = x + ex, sy = y + ey, sz = z + ez;
+        bool in = true;
+        if (sx < 0 || sx >= P.nx) { if (P.per[0]) sx = (sx + P.nx) % P.nx; else in = false; }
+        if (sy < 0 || sy >= P.ny) { if (P.per[1]) sy = (sy + P.ny) % P.ny; else in = false; }
+        if (sz < 0 || sz >= P.nz) { if (P.per[2]) sz = (sz + P.nz) % P.nz; else in = false; }
+        const C w = (C)L::w(i);
+        // offset form (g = f - w rho0; opposite directions share w)
+        C g;
+        const long long nb = (long long)sx + (long long)P.nx * ((long long)sy + (long long)P.ny * sz);
+        if (i != 0 && in && P.flag_old[nb] == 0) {
+            const int io = L::opp(i);
+            g = Cd::ld_plain(A + (long long)io * N + nb, w, rho0) +
+                C(6) * w * rho0 * (ex * ux + ey * uy + ez * uz);
+        } else {
+            g = geq_i<C>(ex, ey, ez, w, C(0), rho0, ux, uy, uz);
+        }
+        Cd::st(A + (long long)i * N + n, g, w, rho0);
+    }
+    atomicAdd(&P.counters[CNT_NREFILL], 1);
+}
+
+template <typename S, int Q>
+__device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, int b) {
     const int tid = threadIdx.x;
-    int cnt = P.bcount[b];
+    const int cnt = brick_count(P, b);
     // the list's slots are read in the same round as its count (slots past
     // the count hold stale ids and are not used)
     const int raw_id = tid < MAXPB ? P.blist[b * MAXPB + tid] : 0;
-    if (cnt > MAXPB) cnt = MAXPB;
     __syncthreads();  // the previous brick's use of sp and of the list is over
     // ascending particle order makes the list, and hence every sum over it,
     // independent of the scatter's atomic order: lane s of warp 0 places its
@@ -62,8 +107,11 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
         const int id = tid < cnt ? raw_id : 0x7fffffff;
         int rank = 0;
         for (int o = 0; o < cnt; o++) rank += __shfl_sync(0xffffffffu, id, o) < id;
-        if (tid < cnt) P.blist[b * MAXPB + rank] = id;
-        if (tid == 0) P.bcount[b] = cnt;
+        if (tid < cnt) {
+            P.blist[b * MAXPB + rank] = id;
+            sp.id[rank] = id;
+        }
+        if (tid == 0) sp.n = cnt;
     }
     __shared__ unsigned s_faces;
     if (tid == 0) s_faces = 0u;
@@ -78,7 +126,7 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
     // the previous flag (the refill below needs it), issued with the
     // particles' loads so that the two latencies overlap
     const uint16_t old = active ? P.flag_old[n] : (uint16_t)0;
-    if (cnt > 0) load_smem_particles(P, sp, b, bx0, by0, bz0);
+    if (cnt > 0) load_particle_records(P, sp, cnt, bx0, by0, bz0);
 
     // owner: the covering particle with the largest M, ties to the lower
     // index (the list is ascending); with one cover its FP32 decision is
@@ -87,6 +135,8 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
     int own = -1;
     if (active && cnt > 0) {
         int own_s = -1;
+        // FP64 lattices: thresholds at which FP32 has no band left
+        const bool exact = sizeof(typename Codec<S>::C) == 8 && !(P.c0_f > 1e-30f && P.c0_f < 1e30f);
         double own_M = -1.0;  // FP64 M of the current owner, < 0 until computed
         for (int s = 0; s < cnt; s++) {
             if (!in_bound(P, sp, s, lx, ly, lz)) continue;  // outside s: M < c0 there
@@ -94,8 +144,8 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
             const float M = metaball32(P, sp, s, (float)lx, (float)ly, (float)lz, unsure);
             bool inside;
             double Md = -1.0;
-            if (kF64 || unsure) {
-                Md = metaball64(P, P.parts[sp.id[s]], (double)x, (double)y, (double)z);
+            if (unsure || exact) {
+                Md = metaball64_far(P, P.parts[sp.id[s]], x, y, z);
                 inside = Md >= P.c0;
             } else {
                 inside = M >= P.c0_f;
@@ -106,8 +156,8 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
                 own_M = Md;
                 continue;
             }
-            if (own_M < 0.0) own_M = metaball64(P, P.parts[sp.id[own_s]], (double)x, (double)y, (double)z);
-            if (Md < 0.0) Md = metaball64(P, P.parts[sp.id[s]], (double)x, (double)y, (double)z);
+            if (own_M < 0.0) own_M = metaball64_far(P, P.parts[sp.id[own_s]], x, y, z);
+            if (Md < 0.0) Md = metaball64_far(P, P.parts[sp.id[s]], x, y, z);
             if (Md > own_M) {
                 own_s = s;
                 own_M = Md;
@@ -138,57 +188,23 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
         if (tid == 0 && P.brick_solid) P.brick_solid[b] = (uint8_t)s_faces;
     }
 
-    // Local refilling, §2.3.3.  Reading: f_i' at x_new counts as known
-    // (Eq. (30)) when it streams in from x_new + e_i and that node was a fluid
-    // node of the previous step; then f_i = f_i'(x_new+e_i) + 6 w_i rho0
-    // e_i.u_w, else f_i = f^eq_i(rho0, u_new); u_w = u_new is the surface
-    // velocity at x_new of the particle that uncovered it.  The values become
-    // the node's post-collision populations.
-    if (active && fl == 0) {
-        if (old != 0) {
-            const DevParticle &pj = P.parts[old - 1];
-            double r[3] = {minimg_d(P, 0, (double)x - pj.x[0]), minimg_d(P, 1, (double)y - pj.x[1]),
-                           minimg_d(P, 2, (double)z - pj.x[2])};
-            const C ux = (C)(pj.v[0] + pj.w[1] * r[2] - pj.w[2] * r[1]);
-            const C uy = (C)(pj.v[1] + pj.w[2] * r[0] - pj.w[0] * r[2]);
-            const C uz = (C)(pj.v[2] + pj.w[0] * r[1] - pj.w[1] * r[0]);
-            const C rho0 = (C)P.rho0;
-            S *A = (S *)P.fA;
-            const long long N = P.N;
-#pragma unroll
-            for (int i = 0; i < Q; i++) {
-                const int ex = L::e(i, 0), ey = L::e(i, 1), ez = L::e(i, 2);
-                int sx = x + ex, sy = y + ey, sz = z + ez;
-                bool in = true;
-                if (sx < 0 || sx >= P.nx) { if (P.per[0]) sx = (sx + P.nx) % P.nx; else in = false; }
-                if (sy < 0 || sy >= P.ny) { if (P.per[1]) sy = (sy + P.ny) % P.ny; else in = false; }
-                if (sz < 0 || sz >= P.nz) { if (P.per[2]) sz = (sz + P.nz) % P.nz; else in = false; }
-                const C w = (C)L::w(i);
-                // offset form (g = f - w rho0; opposite directions share w)
-                C g;
-                const long long nb = (long long)sx + (long long)P.nx * ((long long)sy + (long long)P.ny * sz);
-                if (i != 0 && in && P.flag_old[nb] == 0) {
-                    const int io = L::opp(i);
-                    g = Cd::ld_plain(A + (long long)io * N + nb, w, rho0) +
-                        C(6) * w * rho0 * (ex * ux + ey * uy + ez * uz);
-                } else {
-                    g = geq_i<C>(ex, ey, ez, w, C(0), rho0, ux, uy, uz);
-                }
-                Cd::st(A + (long long)i * N + n, g, w, rho0);
-            }
-            atomicAdd(&P.counters[CNT_NREFILL], 1);
-        }
-    }
+    if (active && fl == 0 && old != 0) refill_node<S, Q>(P, x, y, z, n, old);
 }
 
 // Persistent grid over the bricks listed this step and in the two steps
 // before; a brick listed in several of these lists is visited once (its most
 // recent listing).
-// The bricks are handed out one at a time from a per-step counter, as in the
-// near sweep (thread 0 fetches the next entry while the current brick runs;
-// s_next alternates between two slots).
+// The entries are handed out from a per-step counter, as in the near sweep
+// (thread 0 claims the next ones while the current brick runs; s_next
+// alternates between two slots): this step's one at a time, the older ones,
+// nearly all of which are listed again, eight at a time, a lane each, until few
+// are left (one at a time a CTA spent two barriers and three dependent loads on
+// each of them).
+struct Claim {
+    int first, size;
+};
 template <typename S, int Q>
-__device__ __forceinline__ void flags_work(const Params &P, SmemParticles &sp, int *s_next, int blk) {
+__device__ __forceinline__ void flags_work(const Params &P, SmemParticles &sp, Claim *s_next, int blk, int ctas) {
     const int t = P.step;
     const int r0 = t % 3, r1 = (t + 2) % 3, r2 = (t + 1) % 3;
     const int c0 = P.counters[CNT_LISTED];
@@ -196,32 +212,43 @@ __device__ __forceinline__ void flags_work(const Params &P, SmemParticles &sp, i
     const int c2 = t >= 2 ? P.wl_count[r2] : 0;
     if (blk == 0 && threadIdx.x == 0) P.wl_count[r0] = c0;  // read by the next two steps
     const int total = c0 + c1 + c2;
-    int nxt = 0;
-    if (threadIdx.x == 0) nxt = atomicAdd(&P.counters[CNT_FLAGS_NEXT], 1);
+    const int lane = threadIdx.x & 31;
+    Claim nxt = {0, 1};
+    if (threadIdx.x == 0) nxt.first = atomicAdd(&P.counters[CNT_FLAGS_NEXT], 1);
     for (int k = 0;; k ^= 1) {
         if (threadIdx.x == 0) s_next[k] = nxt;
         __syncthreads();
-        const int w = s_next[k];
-        if (w >= total) break;
-        if (threadIdx.x == 0) nxt = atomicAdd(&P.counters[CNT_FLAGS_NEXT], 1);
-        int b;
-        if (w < c0) {
-            b = P.wl_list[r0 * P.nbricks + w];
-        } else if (w < c0 + c1) {
-            b = P.wl_list[r1 * P.nbricks + (w - c0)];
-            if (P.stamp[b] == t) continue;      // also listed this step
-        } else {
-            b = P.wl_list[r2 * P.nbricks + (w - c0 - c1)];
-            if (P.stamp[b] >= t - 1) continue;  // listed again since
+        const Claim c = s_next[k];
+        if (c.first >= total) break;
+        if (threadIdx.x == 0) {
+            nxt.size = c.first >= c0 && total - c.first >= 16 * ctas ? 8 : 1;
+            nxt.first = atomicAdd(&P.counters[CNT_FLAGS_NEXT], nxt.size);
         }
-        flags_brick<S, Q>(P, sp, b);
+        const int w = c.first + lane;
+        int b = -1;  // the lane's brick (every warp holds the same)
+        if (lane < c.size && w < total) {
+            if (w < c0) {
+                b = P.wl_list[r0 * P.nbricks + w];
+            } else if (w < c0 + c1) {
+                b = P.wl_list[r1 * P.nbricks + (w - c0)];
+                if (P.stamp[b] == t) b = -1;      // also listed this step
+            } else {
+                b = P.wl_list[r2 * P.nbricks + (w - c0 - c1)];
+                if (P.stamp[b] >= t - 1) b = -1;  // listed again since
+            }
+        }
+        for (unsigned m = __ballot_sync(0xffffffffu, b >= 0); m; m &= m - 1)
+            flags_brick<S, Q>(P, sp, __shfl_sync(0xffffffffu, b, __ffs(m) - 1));
     }
 }
+// (Four CTAs per SM at 64 registers: 8 at 32 registers left more room to the
+// plain sweep beside them, 755 -> 717 us a step for 200 metaballs in 256^3, but
+// spilled where one brick's latency counts, 139 -> 145 us for one metaball.)
 template <typename S, int Q>
-__global__ void __launch_bounds__(BRICK) k_flags(Params P) {
+__global__ void __launch_bounds__(BRICK, 4) k_flags(Params P) {
     __shared__ SmemParticles sp;
-    __shared__ int s_next[2];
-    flags_work<S, Q>(P, sp, s_next, blockIdx.x);
+    __shared__ Claim s_next[2];
+    flags_work<S, Q>(P, sp, s_next, blockIdx.x, gridDim.x);
 }
 
 // Every node to f^eq(rho0, u0).

@@ -16,8 +16,34 @@ namespace lbmmb {
 // holds every node with M >= c0 (M >= c0 forces min |x - x_i|^2 <= sum K /
 // c0); grown by one node it also holds every fluid node with a link into
 // the particle.  The particle is appended to the list of each brick the grown
-// box meets (k_flags sorts the lists).
+// box meets (k_flags sorts the lists).  The boxes are loose (200 metaballs in
+// 256^3 meet 22 900 bricks, 6 000 of which hold a solid node), so a brick enters
+// the step's work lists only if M can reach c0 at one of its nodes or one node
+// away.  The flag pass, the near sweep and the sweep of its link-free bricks
+// have that much less to look at: 156 -> 109, 346 -> 248 and 118 -> 8 us there, a
+// step 864 -> 755 us.
 // ---------------------------------------------------------------------------
+// An upper bound of M over the brick grown by one node, from each control
+// point's distance to that box (periodic: |minimum image of x - c| is at least
+// that of the box's centre less half its extent), with a hundredth of a node,
+// 2^-16 of the distance and a thousandth of M for the FP32 rounding.
+__device__ __forceinline__ bool brick_reached(const Params &P, const DevParticle &p, int bxi, int byi, int bzi) {
+    const float org[3] = {(float)(bxi * BX), (float)(byi * BY), (float)(bzi * BZ)};
+    const float half[3] = {0.5f * (BX - 1), 0.5f * (BY - 1), 0.5f * (BZ - 1)};
+    float M = 0.f;
+    for (int k = 0; k < p.ncp; k++) {
+        float d2 = 0.f;
+        for (int a = 0; a < 3; a++) {
+            float m = df_minus_int(p.cpw_hl[k][a], org[a]) - half[a];
+            if (P.per[a]) m -= P.dim_f[a] * rintf(m * P.inv_n_f[a]);
+            const float d = fmaxf(fabsf(m) * (1.0f - 1.0f / 65536.0f) - (half[a] + 1.01f), 0.f);
+            d2 += d * d;
+        }
+        M += p.K_f[k] / d2;
+    }
+    // (NaN: reached; so is everything at thresholds near FP32's range)
+    return !(M * 1.001f < P.c0_f) || !(P.c0_f > 1e-30f && P.c0_f < 1e30f);
+}
 __device__ void bin_particle(const Params &P, int j) {
     const int t = threadIdx.x;
     DevParticle &p = P.parts[j];
@@ -59,38 +85,28 @@ __device__ void bin_particle(const Params &P, int j) {
     const int nxb = rx.hi - rx.lo + 1, nyb = ry.hi - ry.lo + 1, nzb = rz.hi - rz.lo + 1;
     if (nxb <= 0 || nyb <= 0 || nzb <= 0) return;
     const int total = nxb * nyb * nzb;
+    const int next = P.step + 1;
     for (int k = t; k < total; k += blockDim.x) {
         const int bxi = (rx.lo + k % nxb) % P.nbx;
         const int byi = (ry.lo + (k / nxb) % nyb) % P.nby;
         const int bzi = (rz.lo + k / (nxb * nyb)) % P.nbz;
         const int b = bxi + P.nbx * (byi + P.nby * bzi);
-        const int slot = atomicAdd(&P.bcount[b], 1);
+        const bool reached = brick_reached(P, p, bxi, byi, bzi);
+        const unsigned old = (unsigned)atomicAdd(&P.bcount[b], reached ? 1 + kReachOne : 1);
+        const int slot = (int)(old & 0xffffu);
         if (slot < MAXPB) P.blist[b * MAXPB + slot] = j;
         else atomicOr(&P.status[ST_ERR], ERRB_BRICK_OVERFLOW);
-        if (slot == 0) {  // first particle of this brick: list it for k_flags
-            const int pos = atomicAdd(&P.counters[CNT_LISTED], 1);
-            P.wl_list[(P.step % 3) * P.nbricks + pos] = b;
-            P.stamp[b] = P.step;
-            if (P.skip) P.skip[(P.step % 3) * P.nbricks + b] = P.step;
-        }
-    }
-    if (!P.pred_stamp_next) return;
-    // bricks the next step's near sweep takes: the box grown by two nodes (a
-    // link, plus one node of motion); every node the next refill writes and
-    // every node next to one lies inside
-    const BrickRange gx = brick_range(P, p, 0, 2.0), gy = brick_range(P, p, 1, 2.0), gz = brick_range(P, p, 2, 2.0);
-    const int gxb = gx.hi - gx.lo + 1, gyb = gy.hi - gy.lo + 1, gzb = gz.hi - gz.lo + 1;
-    if (gxb <= 0 || gyb <= 0 || gzb <= 0) return;
-    const int gtotal = gxb * gyb * gzb;
-    const int next = P.step + 1;
-    for (int k = t; k < gtotal; k += blockDim.x) {
-        const int bxi = (gx.lo + k % gxb) % P.nbx;
-        const int byi = (gy.lo + (k / gxb) % gyb) % P.nby;
-        const int bzi = (gz.lo + k / (gxb * gyb)) % P.nbz;
-        const int b = bxi + P.nbx * (byi + P.nby * bzi);
-        if (atomicExch(&P.pred_stamp_next[b], next) != next) {
-            const int pos = atomicAdd(&P.pred_count[next % 3], 1);
-            P.pred_list_next[pos] = b;
+        if (!reached || old >= (unsigned)kReachOne) continue;
+        // first particle to reach this brick: list it for k_flags, ...
+        const int pos = atomicAdd(&P.counters[CNT_LISTED], 1);
+        P.wl_list[(P.step % 3) * P.nbricks + pos] = b;
+        P.stamp[b] = P.step;
+        if (P.skip) P.skip[(P.step % 3) * P.nbricks + b] = P.step;
+        // ... and for the next step's near sweep: every node the next refill
+        // writes (solid now) and every node next to one lies in these bricks
+        if (P.pred_stamp_next && atomicExch(&P.pred_stamp_next[b], next) != next) {
+            const int pn = atomicAdd(&P.pred_count[next % 3], 1);
+            P.pred_list_next[pn] = b;
             if (P.skip) P.skip[(next % 3) * P.nbricks + b] = next;
         }
     }
@@ -154,7 +170,7 @@ __global__ void __launch_bounds__(256) k_force_reduce(Params P) {
             const int byi = (ry.lo + (k / nxb) % nyb) % P.nby;
             const int bzi = (rz.lo + k / (nxb * nyb)) % P.nbz;
             const int b = bxi + P.nbx * (byi + P.nby * bzi);
-            const int c = min(P.bcount[b], MAXPB);
+            const int c = brick_count(P, b);  // 0: no partials written
             for (int s = 0; s < c; s++) {
                 if (P.blist[b * MAXPB + s] == j) {
                     for (int q = 0; q < 6; q++) acc[q] += P.partial[((long long)b * MAXPB + s) * 6 + q];

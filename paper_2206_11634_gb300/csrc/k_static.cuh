@@ -44,7 +44,7 @@ __device__ __forceinline__ void static_build_brick(const Params &P, SmemParticle
     const int x = bx0 + lx, y = by0 + ly, z = bz0 + lz;
     const bool active = x < P.nx && y < P.ny && z < P.nz;
     const int n = x + P.nx * (y + P.ny * z);
-    const int cnt = min(P.bcount[b], MAXPB);
+    const int cnt = brick_count(P, b);
     __syncthreads();  // the previous brick is done with the shared state
     load_smem_particles(P, sp, b, bx0, by0, bz0);
     for (int e = lane; e < cnt * 6; e += 32) bs.fix[warp][e / 6][e % 6] = 0ull;

@@ -814,12 +814,11 @@ __device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, d
 // force point: it needs a solid node in the brick or a solid neighbour of one
 // of its nodes -- the brick's own mark, and for each of the 26 bricks around
 // it the faces turned towards it (all of them, for an edge or corner brick).
-// Called by every thread of the CTA (a barrier); the same answer in all.
-__device__ __forceinline__ bool brick_near_solid(const Params &P, int bxi, int byi, int bzi) {
-    const int tid = threadIdx.x;
+// Called by a whole warp; the same answer in all lanes.
+__device__ __forceinline__ bool brick_near_solid(const Params &P, int bxi, int byi, int bzi, int lane) {
     bool near_solid = false;
-    if (tid < 27) {
-        const int o[3] = {tid % 3 - 1, (tid / 3) % 3 - 1, tid / 9 - 1};
+    if (lane < 27) {
+        const int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
         int q[3] = {bxi + o[0], byi + o[1], bzi + o[2]};
         const int nbs[3] = {P.nbx, P.nby, P.nbz};
         bool in = true;
@@ -834,7 +833,7 @@ __device__ __forceinline__ bool brick_near_solid(const Params &P, int bxi, int b
         for (int a = 0; a < 3; a++)  // a brick below faces us with its high face, and so on
             if (o[a] != 0) near_solid = near_solid && (m & (1u << (2 * a + (o[a] < 0 ? 1 : 0)))) != 0;
     }
-    return __syncthreads_or(near_solid) != 0;
+    return __any_sync(0xffffffffu, near_solid);
 }
 
 // The sweep of the bricks listed this step (exactly those some particle's
@@ -845,62 +844,91 @@ __device__ __forceinline__ bool brick_near_solid(const Params &P, int bxi, int b
 // true) it is appended to the step's list for k_sweep_near_plain, which runs
 // after this kernel on the plain sweep's stream at the plain sweep's
 // occupancy, while this kernel keeps its CTAs for the link bricks.
-// Persistent grid;
-// the CTAs take the bricks one at a time from a per-step counter (a brick
-// with particle links costs about ten times one on the plain path, and a
-// fixed split left the busiest CTA near 1.45 times the mean).  Thread 0
-// fetches the next entry while the current brick runs; s_next holds it,
-// alternating between two slots so that a slot is rewritten only after
-// every thread has passed the barrier that follows its last read.
+// Persistent grid; the CTAs claim entries from a per-step counter (a brick with
+// particle links costs about ten times one on the plain path, and a fixed
+// split left the busiest CTA near 1.45 times the mean), up to eight at a time,
+// a warp looking at each: most entries are no link bricks (the predicted ones
+// are nearly all listed too), and looking at one is a chain of three loads.  The
+// claims shrink to one as this step's list runs out, so that no CTA is left with
+// several link bricks.  Thread 0 claims the next entries while the current ones
+// run; st.next holds them, alternating between two slots so that a slot is
+// rewritten only after every thread has passed the barrier that follows its
+// last read.
+constexpr int kNearClaim = BRICK / 32;
+struct NearStage {
+    Claim next[2];
+    int brick[kNearClaim], cnt[kNearClaim];  // -1: nothing to do; listed particles, 0: the plain path
+    int id[kNearClaim][MAXPB];
+};
 template <typename S, int Q, bool kForce, bool kSplit = false>
 __device__ __forceinline__ void near_work(const Params &P, SmemParticles &sp, double (*red)[6], int &s_links,
-                                          LinkScratch &ls, int *s_next) {
-    const int tid = threadIdx.x;
+                                          LinkScratch &ls, NearStage &st, int ctas) {
+    static_assert(MAXPB <= 32, "a lane per listed particle");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int t = P.step;
     const int c_exact = P.counters[CNT_LISTED];
     const int c_pred = P.pred_stamp_cur ? P.pred_count[t % 3] : 0;
     const int total = c_exact + c_pred;
     int done = 0;
-    int nxt = 0;
-    if (tid == 0) nxt = atomicAdd(&P.counters[CNT_NEAR_NEXT], 1);
+    Claim nxt = {0, 0};
+    const auto claim = [&](int from) {
+        nxt.size = from >= c_exact ? kNearClaim : min(max((c_exact - from) / (4 * ctas), 1), kNearClaim);
+        nxt.first = atomicAdd(&P.counters[CNT_NEAR_NEXT], nxt.size);
+    };
+    if (tid == 0) claim(0);
     for (int k = 0;; k ^= 1) {
-        if (tid == 0) s_next[k] = nxt;
-        __syncthreads();  // the previous brick is done with the shared state
-        const int w = s_next[k];
-        if (w >= total) break;
-        if (tid == 0) nxt = atomicAdd(&P.counters[CNT_NEAR_NEXT], 1);
-        int b;
-        if (w < c_exact) {
-            b = P.wl_list[(t % 3) * P.nbricks + w];
-        } else {
-            b = P.pred_list_cur[w - c_exact];
-            if (P.stamp[b] == t) continue;  // listed: taken above
+        if (tid == 0) st.next[k] = nxt;
+        __syncthreads();  // the previous bricks are done with the shared state
+        const Claim c = st.next[k];
+        if (c.first >= total) break;
+        if (tid == 0) claim(c.first);
+        if (warp < c.size) {
+            const int w = c.first + warp;
+            int b = -1, cnt = 0;
+            if (w < total) {
+                b = w < c_exact ? P.wl_list[(t % 3) * P.nbricks + w] : P.pred_list_cur[w - c_exact];
+                cnt = brick_count(P, b);
+                if (lane < MAXPB) st.id[warp][lane] = P.blist[b * MAXPB + lane];  // used up to cnt
+                const bool listed = w >= c_exact && P.stamp[b] == t;
+                int bxi, byi, bzi;
+                brick_coords(P, b, bxi, byi, bzi);
+                if (!brick_near_solid(P, bxi, byi, bzi, lane)) {
+                    // (FP64: it has no partials for k_force_reduce)
+                    if (sizeof(typename Codec<S>::C) == 8 && cnt > 0 && lane == 0) P.bcount[b] = 0;
+                    cnt = 0;
+                }
+                if (listed) b = -1;  // taken from this step's list
+            }
+            if (lane == 0) {
+                st.brick[warp] = b;
+                st.cnt[warp] = cnt;
+                // k_sweep_near_plain takes it (each brick is listed once a step)
+                if (kSplit && b >= 0 && cnt == 0) P.np_list[atomicAdd(P.np_count, 1)] = b;
+            }
         }
-        int bxi, byi, bzi;
-        brick_coords(P, b, bxi, byi, bzi);
-        const int bx0 = bxi * BX, by0 = byi * BY, bz0 = bzi * BZ;
-        int cnt = min(P.bcount[b], MAXPB);
-        // the brick's particle ids, staged with the neighbourhood check below
-        // (made visible by its barrier)
-        if (tid >= 32 && tid < 32 + cnt) sp.id[tid - 32] = P.blist[b * MAXPB + (tid - 32)];
-        if (tid == 0) sp.n = cnt;
-        if (cnt > 0 && P.brick_solid) {
-            if (!brick_near_solid(P, bxi, byi, bzi)) cnt = 0;
-        } else {
-            __syncthreads();
-        }
-        done++;
-        if (cnt == 0) {
-            if (kSplit) {  // k_sweep_near_plain takes it (each brick is listed once a step)
-                if (tid == 0) P.np_list[atomicAdd(P.np_count, 1)] = b;
+        __syncthreads();
+        for (int e = 0; e < c.size; e++) {
+            const int b = st.brick[e], cnt = st.cnt[e];
+            if (b < 0) continue;
+            done++;
+            if (kSplit && cnt == 0) continue;
+            int bxi, byi, bzi;
+            brick_coords(P, b, bxi, byi, bzi);
+            const int bx0 = bxi * BX, by0 = byi * BY, bz0 = bzi * BZ;
+            if (cnt == 0) {
+                const int x = bx0 + tid % BX, y = by0 + (tid / BX) % BY, z = bz0 + tid / (BX * BY);
+                if (x < P.nx && y < P.ny && z < P.nz) plain_node<S, Q, kForce>(P, x, y, z, x + P.nx * (y + P.ny * z));
                 continue;
             }
-            const int x = bx0 + tid % BX, y = by0 + (tid / BX) % BY, z = bz0 + tid / (BX * BY);
-            if (x < P.nx && y < P.ny && z < P.nz) plain_node<S, Q, kForce>(P, x, y, z, x + P.nx * (y + P.ny * z));
-            continue;
+            __syncthreads();  // the previous brick is done with the shared state
+            if (tid < cnt) sp.id[tid] = st.id[e][tid];
+            if (tid == 0) {
+                sp.n = cnt;
+                s_links = 0;
+            }
+            __syncthreads();
+            near_brick<S, Q, kForce>(P, sp, red, &s_links, &ls, b, bx0, by0, bz0, cnt);
         }
-        if (tid == 0) s_links = 0;
-        near_brick<S, Q, kForce>(P, sp, red, &s_links, &ls, b, bx0, by0, bz0, cnt);
     }
     if (tid == 0 && done) atomicAdd(&P.counters[CNT_NEAR], done);
 }
@@ -910,8 +938,8 @@ __global__ void __launch_bounds__(BRICK, kNearCtas<S, kMany>) k_sweep_near(Param
     __shared__ double red[BRICK / 32][6];
     __shared__ int s_links;
     __shared__ LinkScratch ls;
-    __shared__ int s_next[2];
-    near_work<S, Q, kForce, true>(P, sp, red, s_links, ls, s_next);
+    __shared__ NearStage st;
+    near_work<S, Q, kForce, true>(P, sp, red, s_links, ls, st, gridDim.x);
 }
 
 // The bricks of the near set that hold no particle link, as the near sweep

@@ -383,10 +383,10 @@ struct Params {
     int *wl_list;      // [3][nbricks]
     int *wl_count;     // [3], ring of list lengths (slot step % 3 is written by k_flags)
     int *stamp;        // [nbricks], last step the brick was listed
-    // Predicted near set of a step: the bricks within two nodes of the
-    // particles' search boxes of the step before (k_bin of that step scatters
-    // them).  The plain sweep skips these bricks; the near sweep covers them
-    // and the exactly listed ones, so a wrong prediction costs time only.
+    // Predicted near set of a step: the bricks listed in the step before (its
+    // k_bin lists them here too).  The plain sweep skips these bricks, since it
+    // runs beside the refill of nodes that were solid then; the near sweep
+    // covers them and the exactly listed ones.
     int *pred_stamp_cur;   // [nbricks], == step: predicted near this step
     int *pred_stamp_next;  // [nbricks], written for step + 1 (NULL: no prediction)
     int *pred_list_cur;    // [nbricks]
@@ -401,7 +401,7 @@ struct Params {
     // while the chain of t and the binning of t+1 run; the binning of t+1
     // writes the slots of t+1 and t+2 only.
     int *skip;             // [3][nbricks], NULL: none
-    int *bcount;       // [nbricks]
+    int *bcount;       // [nbricks], low half: particles binned; high half: those of them that reach the brick
     uint8_t *brick_solid;  // [nbricks], the brick held a solid node at its last classification
     int *blist;        // [nbricks][MAXPB]
     double *partial;   // [nbricks][MAXPB][6] (FP64 lattices)
@@ -607,7 +607,9 @@ __device__ __forceinline__ bool in_bound(const Params &P, const SmemParticles &s
 // FP32 M of listed particle s at brick-local integer offset (lx,ly,lz) plus a
 // fractional offset; `unsure` is set when the FP32 value cannot decide
 // M >= c0 (inside the relative band 2^-12 around c0, or a control point
-// closer than 1/2, where the rounding of its position dominates).
+// closer than 1/2, where the rounding of its position dominates, unless that
+// control point alone lifts both M and its FP32 value over the band: K / r^2
+// is 4 K there, less 2^-12 of it for the rounding; every other term is >= 0).
 //
 // Error budget: the control point's brick-relative position is rounded once
 // to FP32 (from the FP32 pair of its FP64 value, see df_minus_int: within a
@@ -630,12 +632,20 @@ __device__ __forceinline__ float metaball32(const Params &P, const SmemParticles
         if (P.per[1]) { if (dy > 0.5f * Ly) dy -= Ly; else if (dy < -0.5f * Ly) dy += Ly; }
         if (P.per[2]) { if (dz > 0.5f * Lz) dz -= Lz; else if (dz < -0.5f * Lz) dz += Lz; }
         float r2 = dx * dx + dy * dy + dz * dz;
-        close |= r2 < 0.25f;
+        close |= r2 < 0.25f && !(sp.K[s][k] * 3.99f >= P.c0_f);
         M += sp.K[s][k] * __frcp_rn(r2);  // correctly rounded 1/r2, then one more rounding
     }
     const float c0 = P.c0_f;
     unsure = close || fabsf(M - c0) <= c0 * (1.0f / 4096.0f);
     return M;
+}
+
+// Listed particles of a brick: those binned there, none if M of none of them
+// can reach c0 within a node of it (k_bin).
+constexpr int kReachOne = 1 << 16;
+__device__ __forceinline__ int brick_count(const Params &P, int b) {
+    const unsigned raw = (unsigned)P.bcount[b];
+    return raw < (unsigned)kReachOne ? 0 : min((int)(raw & 0xffffu), MAXPB);
 }
 
 // c - o rounded once to FP32, for c = hl[0] + hl[1] (an FP64 value split into
@@ -692,7 +702,7 @@ __device__ inline void load_particle_records(const Params &P, SmemParticles &sp,
 // Load the listed particles of brick b into shared memory (called by the
 // whole CTA; ends with __syncthreads()).
 __device__ inline void load_smem_particles(const Params &P, SmemParticles &sp, int b, int bx0, int by0, int bz0) {
-    const int cnt = min(P.bcount[b], MAXPB);
+    const int cnt = brick_count(P, b);
     if ((int)threadIdx.x < cnt) sp.id[threadIdx.x] = P.blist[b * MAXPB + threadIdx.x];
     if (threadIdx.x == 0) sp.n = cnt;
     __syncthreads();
