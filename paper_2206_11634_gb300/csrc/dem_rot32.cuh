@@ -2,9 +2,10 @@
 //
 // An FP64 warp instruction holds its SM sub-partition for 64 cycles on this
 // GPU and the n_s sub-steps of a step are one chain (26 such instructions
-// each), so in FP64 they took 110 us per step for n_s = 100.  Here a sub-step is
-// about 600 FP32 instructions (three components side by side).  A step of one particle with n_s = 100, the DEM kernel of an
-// FP64 lattice: 114 -> 62 us.
+// each), so in FP64 they took 110 us per step for n_s = 100.  A step of one
+// particle with n_s = 100, the DEM kernel of an FP64 lattice: 114 us in FP64, 62
+// as some 600 FP32 instructions of one lane, 36 with a lane per
+// component.
 //
 // The scheme is that of rotate_free_quad (k_particles.cu), in the variables
 //   u = h w_b / 2 (the half angle of a sub-step), tau = (h/2)^2 T_b,
@@ -138,97 +139,108 @@ ROT32_FN bool rot32_applies(float u0max, int n_sub, float cImax) {
            cImax <= 1.0001f;
 }
 
-ROT32_FN Rot32Result rot32_run(const Rot32 &R, int n_sub) {
-    Rot32Result o;
+// The sub-steps, written for one component at a time: X gives a component's
+// neighbours.  The host holds the three in an array (N = 3); on the device each
+// is a lane's (N = 1) and neighbours are shuffled.
+//
+// A lane's sub-step is about 330 instructions beside a chain of pair operations
+// nearly as long: products and sums are put together so that what is known
+// early is added early, and one sum is left after each of P, X, g' and P(v1).
+// (One lane for all three components, and the sums in the order of the formulas:
+// about 870 cycles a sub-step.)
+template <class X>
+ROT32_FN bool rot32_steps(const X &x, const Pair (&cI)[X::N], const Pair (&iI)[X::N], const Pair (&U0)[X::N],
+                          const Pair (&G0)[X::N], const Pair (&t0)[X::N], int n_sub, Pair (&delta)[X::N],
+                          Pair (&beta)[X::N]) {
+    constexpr int N = X::N;
     const Pair zero = {0.f, 0.f};
-    Pair base[3], th[3], g[3], u[3], P[3];
+    Pair base[N], th[N], t[N], g[N], u[N];
 #pragma unroll
-    for (int l = 0; l < 3; l++) {
-        o.delta[l] = o.beta[l] = th[l] = g[l] = zero;
-        base[l] = u[l] = R.U0[l];
+    for (int l = 0; l < N; l++) {
+        delta[l] = beta[l] = th[l] = g[l] = zero;
+        base[l] = u[l] = U0[l];
+        t[l] = t0[l];
     }
-    o.ok = true;
+    bool ok = true;
     for (int k = 0; k < n_sub; k++) {
-        float e0[3];
-        Pair uh[3], E[3];
+        Pair P[N], uh[N], e0[N], pre[N], dpre[N], sa[N], sb[N], so[N], Xc[N], v1[N], nb[N];
+        float cm1[N];
 #pragma unroll
-        for (int l = 0; l < 3; l++) {
-            const int a = (l + 1) % 3, b = (l + 2) % 3;
-            P[l] = pmul(pmul(R.cI[l], u[a]), u[b]);
+        for (int l = 0; l < N; l++) {
+            const Pair Gg = padd(G0[l], g[l]);
+            P[l] = pmul(pmul(cI[l], x.at(u, l, 1)), x.at(u, l, 2));
+            uh[l] = padd(padd(u[l], Gg), P[l]);
+            e0[l].h = rot_add(Gg.h, P[l].h);  // uh - u
         }
 #pragma unroll
-        for (int l = 0; l < 3; l++) {
-            E[l] = padd(R.G0[l], padd(g[l], P[l]));  // uh - u
-            uh[l] = padd(u[l], E[l]);
-            e0[l] = E[l].h;
-        }
-        const float a2 = rot_fma(uh[0].h, uh[0].h, rot_fma(uh[1].h, uh[1].h, rot_mul(uh[2].h, uh[2].h)));
-        if (!(a2 <= kRot32MaxHalfAngle2)) {
-            o.ok = false;
-            return o;
-        }
-        const float es = rot_mul(a2, rot_fma(a2, 1.0f / 120.0f, -1.0f / 6.0f));
-        const float cm1 = rot_mul(a2, rot_fma(a2, 1.0f / 24.0f, -0.5f));
-        Pair s[3], t[3], X[3];
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            s[l].h = uh[l].h;
-            s[l].l = rot_fma(uh[l].h, es, uh[l].l);
-            t[l] = padd(R.t0[l], th[l]);
+        for (int l = 0; l < N; l++) {
+            so[l] = uh[l];
+            sa[l] = x.at(uh, l, 1);
+            sb[l] = x.at(uh, l, 2);
+            const float a2 = rot_fma(uh[l].h, uh[l].h, rot_fma(sa[l].h, sa[l].h, rot_mul(sb[l].h, sb[l].h)));
+            ok = ok && a2 <= kRot32MaxHalfAngle2;
+            const float es = rot_mul(a2, rot_fma(a2, 1.0f / 120.0f, -1.0f / 6.0f));
+            cm1[l] = rot_mul(a2, rot_fma(a2, 1.0f / 24.0f, -0.5f));
+            so[l].l = rot_fma(so[l].h, es, so[l].l);
+            sa[l].l = rot_fma(sa[l].h, es, sa[l].l);
+            sb[l].l = rot_fma(sb[l].h, es, sb[l].l);
         }
 #pragma unroll
-        for (int l = 0; l < 3; l++) {
-            const int a = (l + 1) % 3, b = (l + 2) % 3;
-            X[l] = pcross(s[a], t[b], s[b], t[a]);
-        }
-        Pair g1[3];
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            const int a = (l + 1) % 3, b = (l + 2) % 3;
-            // 2 s x X - 2 (c - 1) X
-            const float Y = rot_fma(s[a].h, X[b].h, -rot_mul(s[b].h, X[a].h));
-            const float corr = rot_mul(2.0f, rot_fma(-cm1, X[l].h, Y));
-            const Pair dt = {rot_mul(-2.0f, X[l].h), rot_fma(-2.0f, X[l].l, corr)};
-            th[l] = padd(th[l], dt);
-            g1[l] = pmul(R.iI[l], th[l]);
-        }
-        Pair v1[3];
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            const int a = (l + 1) % 3, b = (l + 2) % 3;
+        for (int l = 0; l < N; l++) {
+            Xc[l] = pcross(sa[l], x.at(t, l, 2), sb[l], x.at(t, l, 1));
             // P(uh) = P(u) + cI (u_a e_b + e_a u_b + e_a e_b), the second term in FP32
-            const float dP = rot_mul(R.cI[l].h, rot_fma(u[a].h, e0[b], rot_mul(e0[a], rot_add(u[b].h, e0[b]))));
+            const float ea = x.at_h(e0, l, 1), eb = x.at_h(e0, l, 2), ua = x.at_h(u, l, 1), ub = x.at_h(u, l, 2);
+            const float dP = rot_mul(cI[l].h, rot_fma(ua, eb, rot_mul(ea, rot_add(ub, eb))));
             Pair q = P[l];
             q.l = rot_add(q.l, dP);
-            v1[l] = padd(uh[l], padd(R.G0[l], padd(g1[l], renorm(q))));
+            pre[l] = padd(padd(uh[l], G0[l]), renorm(q));
+            dpre[l] = padd(delta[l], padd(g[l], P[l]));
         }
 #pragma unroll
-        for (int l = 0; l < 3; l++) {
-            const int a = (l + 1) % 3, b = (l + 2) % 3;
-            const Pair P1 = pmul(pmul(R.cI[l], v1[a]), v1[b]);
+        for (int l = 0; l < N; l++) {
+            // theta' = theta - 2 X + 2 s x X - 2 (c - 1) X
+            const Pair m2X = {rot_mul(-2.0f, Xc[l].h), rot_mul(-2.0f, Xc[l].l)};
+            th[l] = padd(th[l], m2X);
+            const float Y = rot_fma(sa[l].h, x.at_h(Xc, l, 2), -rot_mul(sb[l].h, x.at_h(Xc, l, 1)));
+            th[l].l = rot_add(th[l].l, rot_mul(2.0f, rot_fma(-cm1[l], Xc[l].h, Y)));
+            th[l] = renorm(th[l]);
+            t[l] = padd(t0[l], th[l]);
+            g[l] = pmul(iI[l], th[l]);
+            v1[l] = padd(pre[l], g[l]);
+            dpre[l] = padd(dpre[l], g[l]);
+        }
+#pragma unroll
+        for (int l = 0; l < N; l++) {
+            // D (x) d: beta + s + beta x s + (D_0 - 1) s + (c - 1) beta
+            const Pair ba = x.at(beta, l, 1), bb = x.at(beta, l, 2);
+            const float d0m1 = rot_mul(-0.5f, rot_fma(beta[l].h, beta[l].h, rot_fma(ba.h, ba.h, rot_mul(bb.h, bb.h))));
+            Pair w = pcross(ba, sb[l], bb, sa[l]);
+            w.l = rot_add(w.l, rot_fma(d0m1, so[l].h, rot_mul(cm1[l], beta[l].h)));
+            nb[l] = padd(beta[l], padd(renorm(so[l]), w));
+        }
+#pragma unroll
+        for (int l = 0; l < N; l++) {
             // delta' = delta + g + g' + P(u) + P(v1)
-            o.delta[l] = padd(o.delta[l], padd(padd(g[l], g1[l]), padd(P[l], P1)));
-        }
-        // D (x) d: beta + s + beta x s + (D_0 - 1) s + (c - 1) beta
-        const float d0m1 = rot_mul(-0.5f, rot_fma(o.beta[0].h, o.beta[0].h,
-                                                  rot_fma(o.beta[1].h, o.beta[1].h, rot_mul(o.beta[2].h, o.beta[2].h))));
-        Pair nb[3];
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            const int a = (l + 1) % 3, b = (l + 2) % 3;
-            Pair w = pcross(o.beta[a], s[b], o.beta[b], s[a]);
-            w.l = rot_add(w.l, rot_fma(d0m1, s[l].h, rot_mul(cm1, o.beta[l].h)));
-            nb[l] = padd(o.beta[l], padd(renorm(s[l]), w));
-        }
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            o.beta[l] = nb[l];
-            const Pair g2 = {2.0f * R.G0[l].h, 2.0f * R.G0[l].l};
+            const Pair P1 = pmul(pmul(cI[l], x.at(v1, l, 1)), x.at(v1, l, 2));
+            const Pair g2 = {2.0f * G0[l].h, 2.0f * G0[l].l};
             base[l] = padd(base[l], g2);
-            g[l] = g1[l];
-            u[l] = padd(base[l], o.delta[l]);
+            u[l] = padd(padd(base[l], dpre[l]), P1);
+            delta[l] = padd(dpre[l], P1);
+            beta[l] = nb[l];
         }
     }
+    return ok;
+}
+
+// All three components in one thread.
+struct RotArray {
+    static constexpr int N = 3;
+    ROT32_FN Pair at(const Pair (&v)[3], int l, int o) const { return v[(l + o) % 3]; }
+    ROT32_FN float at_h(const Pair (&v)[3], int l, int o) const { return v[(l + o) % 3].h; }
+};
+ROT32_FN Rot32Result rot32_run(const Rot32 &R, int n_sub) {
+    Rot32Result o;
+    o.ok = rot32_steps(RotArray(), R.cI, R.iI, R.U0, R.G0, R.t0, n_sub, o.delta, o.beta);
     return o;
 }
 

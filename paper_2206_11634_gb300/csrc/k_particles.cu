@@ -729,8 +729,19 @@ __device__ void rotate_sub_steps(unsigned mk, const QuadLanes &L, const DevParti
 }
 
 // The same in FP32 pairs (dem_rot32.cuh) for the quads where they carry
-// FP64's accuracy: lane 0 of a quad runs its particle's sub-steps.  Returns
-// whether this quad was taken.
+// FP64's accuracy: lanes 1 to 3 of a quad hold a component each.  Returns whether
+// this quad was taken.
+struct RotLanes {
+    static constexpr int N = 1;
+    unsigned mk;
+    int l1, l2;
+    __device__ __forceinline__ float at_h(const Pair (&v)[1], int, int o) const {
+        return __shfl_sync(mk, v[0].h, o == 1 ? l1 : l2, 4);
+    }
+    __device__ __forceinline__ Pair at(const Pair (&v)[1], int l, int o) const {
+        return {at_h(v, l, o), __shfl_sync(mk, v[0].l, o == 1 ? l1 : l2, 4)};
+    }
+};
 __device__ bool rotate_pairs(unsigned mk, const QuadLanes &L, const DevParticle &p, double h, int n_sub, double &q,
                              double &wb, double Tb) {
     const int lane = L.lane;
@@ -747,43 +758,18 @@ __device__ bool rotate_pairs(unsigned mk, const QuadLanes &L, const DevParticle 
     const bool fits = rot32_applies(hh_f * (sqrtf(w2) + sqrtf(d2)), n_sub, cm);
     const unsigned mf = __ballot_sync(mk, fits);
     if (!fits) return false;
-    // this lane's component as pairs, gathered by lane 0
+    // this lane's component as pairs (lane 0: as lane 1)
     const double hh = 0.5 * h, t = hh * hh * Tb;
-    const Pair mine[5] = {rot_split(p.cI[m]), rot_split(p.iI[m]), rot_split(hh * wb), rot_split(t * p.iI[m]),
-                          rot_split(t)};
-    Rot32 R;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        Pair got[5];
-#pragma unroll
-        for (int k = 0; k < 5; k++) {
-            got[k].h = __shfl_sync(mf, mine[k].h, 1 + a, 4);
-            got[k].l = __shfl_sync(mf, mine[k].l, 1 + a, 4);
-        }
-        R.cI[a] = got[0];
-        R.iI[a] = got[1];
-        R.U0[a] = got[2];
-        R.G0[a] = got[3];
-        R.t0[a] = got[4];
-    }
-    Rot32Result r = {};
-    if (lane == 0) r = rot32_run(R, n_sub);
-    __syncwarp(mf);
-    Pair db[2];  // this lane's delta and beta (lane 0: unused)
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const Pair d = {__shfl_sync(mf, r.delta[a].h, 0, 4), __shfl_sync(mf, r.delta[a].l, 0, 4)};
-        const Pair b = {__shfl_sync(mf, r.beta[a].h, 0, 4), __shfl_sync(mf, r.beta[a].l, 0, 4)};
-        if (m == a) {
-            db[0] = d;
-            db[1] = b;
-        }
-    }
-    const bool ok = __shfl_sync(mf, (int)r.ok, 0, 4) != 0;
+    const Pair cI[1] = {rot_split(p.cI[m])}, iI[1] = {rot_split(p.iI[m])}, U0[1] = {rot_split(hh * wb)};
+    const Pair G0[1] = {rot_split(t * p.iI[m])}, t0[1] = {rot_split(t)};
+    Pair delta_p[1], beta_p[1];
+    const bool in_range = rot32_steps(RotLanes{mf, L.l1, L.l2}, cI, iI, U0, G0, t0, n_sub, delta_p, beta_p);
+    const unsigned bad = __ballot_sync(mf, !in_range && lane > 0) >> (threadIdx.x & 28u);
+    const bool ok = (bad & 0xeu) == 0u;  // of the quad's three components
     // w_b: the start's, the torque's (n_s sub-steps of h T / I, h = 1 / n_s)
     // and delta = h/2 of the rest
-    const double delta = to_double(db[0].h) + to_double(db[0].l);
-    const double beta = lane == 0 ? 0.0 : to_double(db[1].h) + to_double(db[1].l);
+    const double delta = to_double(delta_p[0].h) + to_double(delta_p[0].l);
+    const double beta = lane == 0 ? 0.0 : to_double(beta_p[0].h) + to_double(beta_p[0].l);
     const double wn = fma(2.0 * n_sub, delta, fma(p.iI[m], Tb, wb));
     // D = (sqrt(1 - |beta|^2), beta), |beta|^2 <= 2^-16: the next term of the
     // series is below 2^-69
