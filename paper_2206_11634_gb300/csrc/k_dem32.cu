@@ -135,13 +135,14 @@ struct SharedT {
     // walls: contact history
     int w_on[CAP][NWALL];
     float w_xcw[CAP][NWALL][3], w_xi[CAP][NWALL][3];
+    float w_ft[kWarpGroup ? CAP : 1][NWALL][6];  // warp tables: the walls' force and torque terms
 };
 // every particle in one CTA (k_dem32, and k_dem64c for a large contact group)
 using Shared = SharedT<kMaxP, kMaxItems, kDem32MaxCp, false, false>;
 // a contact group of up to 32 particles (k_dem64c, one CTA per group)
 using SharedSmall = SharedT<kSmallContactGroup, 256, kSmallContactGroup * MAXCP, true, false>;
-// a contact group of up to kTinyContactGroup particles (one warp each,
-// kTinyGroupsPerCta tables per CTA; at most 6 candidate pairs)
+// a contact group of up to kTinyContactGroup particles (k_dem64t, whose warps
+// share the tables; at most 6 candidate pairs)
 using SharedTiny = SharedT<kTinyContactGroup, 8, kTinyContactGroup * MAXCP, false, true>;
 
 // The threads that share one table: the CTA, or for warp tables the warp.
@@ -1182,7 +1183,7 @@ __global__ void __launch_bounds__(kClass == DEM_GROUP_LARGE ? kThreads : kSmallC
 }
 
 // ---------------------------------------------------------------------------
-// Contact groups of up to four particles, one warp each (k_dem64t).  Lane
+// Contact groups of up to four particles (k_dem64t).  Lane
 // kSegLanes * k + c works for particle k of the group (for k past the group's
 // size: particle k mod size, as a mirror): the particle's lanes all hold its
 // state (they integrate it from the same inputs in the same order, so they
@@ -1304,11 +1305,13 @@ __device__ __forceinline__ bool wall_geom_seg(const Params &P, const SH &S, int 
     return true;
 }
 
-// The walls' terms of particle k added to F, T (after its pair terms), run by
-// the particle's lanes (mask), which all write the contact history.
+// The walls' terms of particle k into w_ft, run by the particle's lanes (mask),
+// which all write them and the contact history; returns the walls in contact,
+// a bit each.  walls_add then adds them to F, T after the pair terms.
 template <class SH>
-__device__ void walls_seg(const Params &P, SH &S, int k, unsigned mask, float h, const float4 ca, const float4 cb,
-                          float F[3], float T[3]) {
+__device__ unsigned walls_seg(const Params &P, SH &S, int k, unsigned mask, float h, const float4 ca,
+                              const float4 cb) {
+    unsigned hits = 0u;
     for (int wall = 0; wall < NWALL; wall++) {
         const int ax = wall / 2, side = wall % 2;
         if (P.per[ax]) {
@@ -1337,21 +1340,35 @@ __device__ void walls_seg(const Params &P, SH &S, int k, unsigned mask, float h,
             : ax == 1 ? wall_geom_seg<1>(P, S, k, side, prel, start, xcw, delta, nv, xcp, valid, mask, ca, cb)
                       : wall_geom_seg<2>(P, S, k, side, prel, start, xcw, delta, nv, xcp, valid, mask, ca, cb);
         const int warm = valid ? CONTACT_WARM : 0;
+        float Fi[3], ti[3];
         if (hit) {
-            float wr[3], vi[3], Fi[3], ti[3];
+            float wr[3], vi[3];
             cross3f(S.w[k], xcp, wr);
             for (int a = 0; a < 3; a++) vi[a] = S.v[k][a] + wr[a];
             contact_law_f(P, delta, nv, vi, xi, h, Fi);
             cross3f(xcp, Fi, ti);
-            for (int a = 0; a < 3; a++) { F[a] += Fi[a]; T[a] += ti[a]; }
+            hits |= 1u << wall;
         }
         __syncwarp(mask);
         for (int a = 0; a < 3; a++) S.w_xcw[k][wall][a] = xcw[a];
         S.w_on[k][wall] = hit ? (warm | CONTACT_ON) : warm;
         if (hit)
-            for (int a = 0; a < 3; a++) S.w_xi[k][wall][a] = xi[a];
+            for (int a = 0; a < 3; a++) {
+                S.w_xi[k][wall][a] = xi[a];
+                S.w_ft[k][wall][a] = Fi[a];
+                S.w_ft[k][wall][3 + a] = ti[a];
+            }
+    }
+    return hits;
+}
+template <class SH>
+__device__ __forceinline__ void walls_add(const SH &S, int k, unsigned hits, float F[3], float T[3]) {
+    for (; hits; hits &= hits - 1) {
+        const float *t = S.w_ft[k][__ffs(hits) - 1];
+        for (int a = 0; a < 3; a++) { F[a] += t[a]; T[a] += t[3 + a]; }
     }
 }
+
 
 // Pair geometry of Eqs. (5)-(9), the steps of pair_geom_f, run by the whole
 // warp: lanes 0-15 hold the control points of particle i, lanes 16-31 those
@@ -1448,14 +1465,14 @@ __device__ bool pair_geom_w(const Params &P, const SH &S, int i, int j, const fl
     return true;
 }
 
-// Pair contacts of the candidate list, one item after the other, each by the
-// whole warp (every lane writes the results); results into it_res (zeros
+// Pair contacts of the candidate list, each by a whole warp (every lane writes
+// the results): items first, first + stride, ...; results into it_res (zeros
 // when not in contact), as pair_contacts.
 template <class SH>
-__device__ void pair_contacts_w(const Params &P, SH &S, float h) {
+__device__ void pair_contacts_w(const Params &P, SH &S, float h, int first, int stride) {
     const int np = S.n;
     const int total = min(S.ioff[np], SH::kItems);
-    for (int it = 0; it < total; it++) {
+    for (int it = first; it < total; it += stride) {
         int i = 0;  // last i with ioff[i] <= it
         while (i + 1 < np && S.ioff[i + 1] <= it) i++;
         const int j = S.up[i][it - S.ioff[i]];
@@ -1501,20 +1518,44 @@ __device__ void pair_contacts_w(const Params &P, SH &S, float h) {
 }
 }  // namespace
 
-// A contact group of up to kTinyContactGroup particles per warp,
-// kTinyGroupsPerCta warps per CTA: the sub-steps of k_dem64c with the lanes
-// split by particle (above).
-__global__ void __launch_bounds__(32 * kTinyGroupsPerCta, 1) k_dem64t(Params P) {
+// The tiny group's warps meet (bar.sync of kTinyWarps warps; nothing to meet in
+// a group of one particle, whose other warps have left).
+__device__ __forceinline__ void tiny_sync(int na) {
+    __syncwarp();
+    if (na > 1) asm volatile("bar.sync 1, %0;" ::"n"(32 * kTinyWarps) : "memory");
+}
+
+// A contact group of up to kTinyContactGroup particles per CTA: the sub-steps of
+// k_dem64c with the lanes of warp 0 split by particle (above).  A sub-step is
+// one chain of latencies: warp 0 integrates and publishes the particles, then it
+// takes the wall contacts while the other warps take the pair contacts, a pair
+// each (up to six), and adds both up, pairs first.
+// (One warp for all of it: 8500 cycles a sub-step for the settled floor of 50
+// metaballs in 128x128x256, n_s = 100; the DEM phase 427 us a step, now 281.)
+__global__ void __launch_bounds__(32 * kTinyWarps, 1) k_dem64t(Params P) {
     using SH = SharedTiny;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int wt = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
-    SH &S = reinterpret_cast<SH *>(smem_raw)[wt];
-    const int slot = (int)blockIdx.x * kTinyGroupsPerCta + wt;
-    if (slot >= P.dem_list[2 + DEM_GROUP_TINY]) return;  // the whole warp
+    SH &S = *reinterpret_cast<SH *>(smem_raw);
+    const int slot = (int)blockIdx.x;
+    if (slot >= P.dem_list[2 + DEM_GROUP_TINY]) return;  // the whole CTA
     const int *grp = dem_groups(P, DEM_GROUP_TINY) + 2 * slot;
     const int na = grp[1];
     const int *act = dem_active(P) + grp[0];
     const float h = P.h_f, hh = 0.5f * h, qh2 = 0.25f * h * h;
+    if (wt > 0) {
+        // the pair contacts of the start (unless known), of every sub-step and
+        // of the end
+        if (na == 1) return;
+        tiny_sync(na);
+        if (S.cpo[na] > SH::kCps) return;
+        for (int e = P.fc_valid ? 1 : 0; e < P.n_sub + 2; e++) {
+            tiny_sync(na);  // the particles are published
+            pair_contacts_w(P, S, e == 0 || e == P.n_sub + 1 ? 0.f : h, wt - 1, kTinyWarps - 1);
+            tiny_sync(na);  // warp 0 may add up
+        }
+        return;
+    }
     const int c = lane % kSegLanes;
     const unsigned seg = ((1u << kSegLanes) - 1u) << (lane - c);  // this lane's particle lanes
     const bool own = lane / kSegLanes < na;
@@ -1560,7 +1601,16 @@ __global__ void __launch_bounds__(32 * kTinyGroupsPerCta, 1) k_dem64t(Params P) 
     }
     if (lane < na) S.gid[lane] = act[lane];
     __syncwarp();
+    tiny_sync(na);
     if (S.cpo[na] > SH::kCps) return;
+    // the contact load of the published particles
+    auto contact_load = [&](float step, const float4 ca, const float4 cb, float F[3], float T[3]) {
+        tiny_sync(na);
+        const unsigned hits = walls_seg(P, S, k, seg, step, ca, cb);
+        tiny_sync(na);
+        gather_pairs(S, k, F, T);
+        walls_add(S, k, hits, F, T);
+    };
 
     // FP32 tables: position (hi + lo of the FP64 value), velocity, world
     // angular velocity from the body rate wf
@@ -1616,10 +1666,7 @@ __global__ void __launch_bounds__(32 * kTinyGroupsPerCta, 1) k_dem64t(Params P) 
     // contact load at the start: left by the previous step's DEM (same
     // state), unless the particles were set since
     if (!P.fc_valid) {
-        pair_contacts_w(P, S, 0.f);
-        __syncwarp();
-        gather_pairs(S, k, Fc, Tc);
-        walls_seg(P, S, k, seg, 0.f, rca, rcb, Fc, Tc);
+        contact_load(0.f, rca, rcb, Fc, Tc);
     } else {
         for (int a = 0; a < 3; a++) {
             Fc[a] = (float)P.Fc[3 * g + a];
@@ -1674,12 +1721,9 @@ __global__ void __launch_bounds__(32 * kTinyGroupsPerCta, 1) k_dem64t(Params P) 
             __syncwarp();
             build_lists(P, S, &dummy);
         }
-        pair_contacts_w(P, S, h);
-        __syncwarp();
         {
             float F[3], T[3];
-            gather_pairs(S, k, F, T);
-            walls_seg(P, S, k, seg, h, rca, rcb, F, T);
+            contact_load(h, rca, rcb, F, T);
             for (int a = 0; a < 3; a++) { Fc[a] = F[a]; Tc[a] = T[a]; }
             if (mov) {
                 // closing half-kick with the new contact load
@@ -1723,11 +1767,8 @@ __global__ void __launch_bounds__(32 * kTinyGroupsPerCta, 1) k_dem64t(Params P) 
         if (mov) rotate_cps(qf);
     }
     __syncwarp();
-    pair_contacts_w(P, S, 0.f);
-    __syncwarp();
     float F[3], T[3];
-    gather_pairs(S, k, F, T);
-    walls_seg(P, S, k, seg, 0.f, rca, rcb, F, T);
+    contact_load(0.f, rca, rcb, F, T);
     __syncwarp();  // every lane has read the particle records (the end state is written below)
     if (own) {
         if (c < NWALL) {  // lane c: the history of wall c
@@ -1767,17 +1808,15 @@ void launch_dem64c(const Params &P, cudaStream_t st) {
     // the dynamic shared memory limits are raised once per device
     static bool attr_set[64] = {};
     static_assert(sizeof(SharedSmall) <= 48 * 1024, "small contact-group tables exceed 48 KB");
-    static_assert(kTinyGroupsPerCta * sizeof(SharedTiny) <= 48 * 1024, "tiny contact-group tables exceed 48 KB");
+    static_assert(sizeof(SharedTiny) <= 48 * 1024, "tiny contact-group tables exceed 48 KB");
     const int big = (int)sizeof(Shared);
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !attr_set[dev])
         attr_set[dev] = cudaFuncSetAttribute(k_dem64c<Shared, DEM_GROUP_LARGE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, big) == cudaSuccess;
     // grids for the worst case (every group tiny, or small); at most np / 33
-    // groups are large.  A tiny-group CTA of 8 warps holds most of an SM's
-    // registers, so few other CTAs share the SM with its latency-bound chains.
-    k_dem64t<<<(P.np + kTinyGroupsPerCta - 1) / kTinyGroupsPerCta, 32 * kTinyGroupsPerCta,
-               kTinyGroupsPerCta * sizeof(SharedTiny), st>>>(P);
+    // groups are large
+    k_dem64t<<<P.np, 32 * kTinyWarps, sizeof(SharedTiny), st>>>(P);
     k_dem64c<SharedSmall, DEM_GROUP_SMALL><<<P.np / (kTinyContactGroup + 1) + 1, kSmallContactGroup,
                                              sizeof(SharedSmall), st>>>(P);
     k_dem64c<Shared, DEM_GROUP_LARGE><<<P.np / (kSmallContactGroup + 1) + 1, kThreads, big, st>>>(P);

@@ -92,8 +92,8 @@ constexpr int kDem32MaxParticles = 256;
 constexpr int kDem32MaxCp = 2048;     // control points of all particles
 constexpr int kDemMaxAdj = 16;        // candidate contact partners per particle and direction
 constexpr int kSmallContactGroup = 32;  // contact groups up to this size run one 32-thread CTA each
-constexpr int kTinyContactGroup = 4;    // ... up to this size one warp each, kTinyGroupsPerCta per CTA
-constexpr int kTinyGroupsPerCta = 8;
+constexpr int kTinyContactGroup = 4;    // ... up to this size kTinyWarps warps
+constexpr int kTinyWarps = 4;
 // k_dem64_plan's group classes (dem_groups)
 enum DemGroupClass { DEM_GROUP_TINY = 0, DEM_GROUP_SMALL = 1, DEM_GROUP_LARGE = 2 };
 
