@@ -27,11 +27,11 @@ __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_sweep_near_batch(Batc
     __shared__ SmemParticles sp;
     __shared__ double red[BRICK / 32][6];
     __shared__ int s_links;
-    __shared__ LinkScratch ls;
+    __shared__ LinkScratch<BRICK / 32> ls;
     __shared__ NearStage st;
     const int c = blockIdx.x / B.g_chain;
     load_case_params(B, c, B.ctr, sP);
-    near_work<S, Q, kForce>(sP, sp, red, s_links, ls, st, B.g_chain);
+    near_work<S, Q, kForce, false, BRICK>(sP, sp, red, s_links, ls, st, B.g_chain);
     advance_step_when_last(B.ctr + 2, B.ctr);
 }
 

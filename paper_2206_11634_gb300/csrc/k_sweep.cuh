@@ -1,4 +1,4 @@
-// The fused lattice sweep (one CTA per 32x4x2 brick, one node per thread).
+// The fused lattice sweep (one CTA per 32x4x2 brick, one or two nodes a thread).
 //
 // For every fluid node x (flags of this step):
 //   pull    f_i(x, t+1) = f+_i(x - e_i, t) from the read array (§2.2, Eq. (14));
@@ -32,14 +32,18 @@ namespace lbmmb {
 // Resident CTAs per SM of the fixed-geometry link kernels and of the batched
 // near sweep.
 constexpr int kNearCtasPerSm = 2;
-// ... and of the near sweep, by the near bricks expected (P.near_many).  A few
-// bricks wait for one brick's latency, which registers shorten (two CTAs: 128
-// registers; FP64 one CTA: 255); thousands wait for the latencies of all, and
-// more CTAs overlap more of them although they spill (four: 64 registers).
-// Near sweep in us at 2 / 3 / 4 CTAs: 200 metaballs in 256^3 417 / 357 / 320, 50
-// in 128x128x256 122 / 113 / 112, 12 there 47 / 49 / 57, one there 15.9 / 17.8 /
-// 18.1; FP64 at 1 / 2: one sphere in 32x32x48 43 / 60, 25 metaballs in 128^3 451 /
-// 413.
+// ... and of the near sweep, and its threads, by the near bricks expected
+// (P.near_expected).  A few bricks wait for one brick's latency: a thread per
+// node, two CTAs of 128 registers a thread (FP64 one of 255).  Thousands wait for
+// the latencies of all; there half of a CTA's warps have no link to evaluate, so
+// below FP64 a CTA has 128 threads, two nodes each, and four CTAs run per SM.
+// Near sweep in us: 200 metaballs in 256^3, 256 threads at 2 / 3 / 4 CTAs (64
+// registers at 4) 420 / 357 / 320 before the lists were culled and 248 after, 128
+// threads at 4 / 6 / 8 CTAs 238 / 246 / 318; 50 settled in 128x128x256 117 and 94;
+// one there 15.9 / 17.8 / 18.1 at 2 / 3 / 4; FP64 at 1 / 2: one sphere in 32x32x48
+// 43 / 60, 25 metaballs in 128^3 451 / 413.
+template <typename S, bool kMany>
+constexpr int kNearThreads = sizeof(S) != 8 && kMany ? BRICK / 2 : BRICK;
 template <typename S, bool kMany>
 constexpr int kNearCtas = sizeof(S) == 8 ? (kMany ? 2 : 1) : (kMany ? 4 : 2);
 
@@ -584,13 +588,13 @@ __device__ __forceinline__ typename Codec<S>::C link_coop(const Params &P, const
 // Links a warp's nodes can have.
 constexpr int kLinkQueue = 32 * 18;
 // Shared scratch of the cooperative link evaluation: the brick's links in
-// thread order, then direction order, as (thread << 5) | direction, and their
-// results.
+// thread order, then direction order, as (node << 5) | direction, each replaced
+// by its result (below FP64); kWarps warps.
+template <int kWarps>
 struct LinkScratch {
-    unsigned short entry[BRICK / 32 * kLinkQueue];
-    float result[BRICK / 32 * kLinkQueue];
-    int warp_links[BRICK / 32];
-    unsigned long long fix[BRICK / 32][MAXPB][6];  // the warp's fixed-point force/torque terms
+    uint32_t slot[BRICK / 32 * kLinkQueue];
+    int warp_links[kWarps];
+    unsigned long long fix[kWarps][MAXPB][6];  // the warp's fixed-point force/torque terms
 };
 
 // Bricks some particle reaches: nodes without particle links take the plain
@@ -604,7 +608,8 @@ struct LinkScratch {
 // and one-subtraction indices for the flags and pulls: 200 metaballs in 256^3
 // 566 -> 492 us, one metaball in 128x128x256 22.8 -> 18.3, the FP64 sphere 91 ->
 // 69.  All of it inline (calls saved and restored most registers, and below FP64
-// the unused FP64 partials held 384 bytes of stack a thread): 417, 15.9, 60.
+// the unused FP64 partials held 384 bytes of stack a thread): 417, 15.9, 60.  (CTAs
+// and threads: see kNearCtas.)
 //
 // FP64 lattices are bound by the FP64 pipe here (64 cycles a warp
 // instruction, some 250 of them a link): with every node walking its own links
@@ -613,19 +618,16 @@ struct LinkScratch {
 // link's result waits in its node's own slot of the array being written
 // (which nothing reads in this step): no limit on a warp's links, and no
 // shared memory for FP64 results.
-template <typename S, int Q, bool kForce>
+template <typename S, int Q, bool kForce, int kThreads>
 __device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, double (*red)[6], int *s_links,
-                                        LinkScratch *ls, int b, int bx0, int by0, int bz0, int cnt) {
+                                        LinkScratch<kThreads / 32> *ls, int b, int bx0, int by0, int bz0, int cnt) {
     using L = Lat<Q>;
     using Cd = Codec<S>;
     using C = typename Cd::C;
+    constexpr int kWarps = kThreads / 32, kRows = BRICK / kThreads;  // kRows nodes a thread
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
-    const int lx = tid % BX, ly = (tid / BX) % BY, lz = tid / (BX * BY);
-    const int x = bx0 + lx, y = by0 + ly, z = bz0 + lz;
-    const bool active = x < P.nx && y < P.ny && z < P.nz;
     const long long N = P.N;
-    const int n = x + P.nx * (y + P.ny * z);
     const S *A = (const S *)P.fA;
     S *B = (S *)P.fB;
     const C rho0 = Prm<C>::rho0(P);
@@ -641,70 +643,82 @@ __device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, d
     }
     int nlinks = 0;
 
-    // the node's flag and its neighbours' (y = x - e_i; kWall beyond a wall),
-    // read in one round by fluid and solid nodes alike and issued before the
-    // brick's particles are loaded, so the two latencies overlap
-    constexpr uint32_t kWall = 0xFFFFFFFFu;
-    uint32_t nf[Q];
-    if (P.idx32 && y > 0 && y < P.ny - 1 && z > 0 && z < P.nz - 1) {
-        // a row off the y and z faces (a warp is a row): one subtraction per
-        // neighbour, corrected on the x-face lanes (plain_pull's indices).
-        // Lanes past the row's end read inside the lattice too.
-        const int nx = P.nx, nxy = P.nx * P.ny;
-        int cm = 0, cp = 0;
-        bool wm = false, wp = false;
-        if (x == 0) { if (P.per[0]) cm = nx; else wm = true; }
-        if (x == nx - 1) { if (P.per[0]) cp = -nx; else wp = true; }
-        nf[0] = active ? (uint32_t)P.flag_new[(unsigned)n] : 1u;
-#pragma unroll
-        for (int i = 1; i < Q; i++) {
-            const int ex = L::e(i, 0);
-            const uint32_t f = P.flag_new[(unsigned)(n - (ex + nx * L::e(i, 1) + nxy * L::e(i, 2)) +
-                                                    (ex > 0 ? cm : (ex < 0 ? cp : 0)))];
-            nf[i] = (!active || (ex > 0 && wm) || (ex < 0 && wp)) ? kWall : f;
-        }
-    } else {
-        int xs[3], ys[3], zs[3];
-        neighbour_coords(P, x, y, z, xs, ys, zs);
-        nf[0] = active ? (uint32_t)P.flag_new[n] : 1u;
-#pragma unroll
-        for (int i = 1; i < Q; i++) {
-            const int sx = xs[1 - L::e(i, 0)], sy = ys[1 - L::e(i, 1)], sz = zs[1 - L::e(i, 2)];
-            const bool wall = (sx | sy | sz) < 0;
-            nf[i] = (!active || wall) ? kWall : (uint32_t)P.flag_new[sx + P.nx * (sy + P.ny * sz)];
-        }
-    }
-    load_particle_records(P, sp, cnt, bx0, by0, bz0);  // ids staged by the caller
-    const bool fluid = active && nf[0] == 0;
-    uint32_t links = 0;
-    if (fluid) {
-#pragma unroll
-        for (int i = 1; i < Q; i++)
-            if (nf[i] != 0 && nf[i] != kWall) links |= 1u << i;
-    }
+    uint32_t links[kRows];
+    bool fluid[kRows];
     int nterms = 0;  // missing-force-point terms this thread added
-    if (active && !fluid && P.missing_force) {
-        // per listed particle j, the directions whose neighbour is neither a
-        // fluid node next to j's own node nor a node of j
-        const int owner = (int)nf[0] - 1;
-        for (int s = 0; s < sp.n; s++) {
-            const int j = sp.id[s];
-            // a node outside another particle's bounding sphere is not inside
-            // it: solid_links would find nothing
-            if (j != owner && !in_bound(P, sp, s, lx, ly, lz)) continue;
-            uint32_t cand = 0;
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+        const int node = tid + r * kThreads;
+        const int lx = node % BX, ly = (node / BX) % BY, lz = node / (BX * BY);
+        const int x = bx0 + lx, y = by0 + ly, z = bz0 + lz;
+        const bool active = x < P.nx && y < P.ny && z < P.nz;
+        const int n = x + P.nx * (y + P.ny * z);
+        // the node's flag and its neighbours' (y = x - e_i; kWall beyond a wall),
+        // read in one round by fluid and solid nodes alike and issued before the
+        // brick's particles are loaded, so the two latencies overlap
+        constexpr uint32_t kWall = 0xFFFFFFFFu;
+        uint32_t nf[Q];
+        if (P.idx32 && y > 0 && y < P.ny - 1 && z > 0 && z < P.nz - 1) {
+            // a row off the y and z faces (a warp is a row): one subtraction per
+            // neighbour, corrected on the x-face lanes (plain_pull's indices).
+            // Lanes past the row's end read inside the lattice too.
+            const int nx = P.nx, nxy = P.nx * P.ny;
+            int cm = 0, cp = 0;
+            bool wm = false, wp = false;
+            if (x == 0) { if (P.per[0]) cm = nx; else wm = true; }
+            if (x == nx - 1) { if (P.per[0]) cp = -nx; else wp = true; }
+            nf[0] = active ? (uint32_t)P.flag_new[(unsigned)n] : 1u;
 #pragma unroll
             for (int i = 1; i < Q; i++) {
-                const bool seen = (nf[i] == 0 && j == owner) || nf[i] == (uint32_t)(j + 1);
-                if (!seen) cand |= 1u << i;
+                const int ex = L::e(i, 0);
+                const uint32_t f = P.flag_new[(unsigned)(n - (ex + nx * L::e(i, 1) + nxy * L::e(i, 2)) +
+                                                        (ex > 0 ? cm : (ex < 0 ? cp : 0)))];
+                nf[i] = (!active || (ex > 0 && wm) || (ex < 0 && wp)) ? kWall : f;
             }
-            if (cand) nterms += solid_links<S, Q>(P, sp, s, j == owner, cand, lx, ly, lz, bx0, by0, bz0, sink);
+        } else {
+            int xs[3], ys[3], zs[3];
+            neighbour_coords(P, x, y, z, xs, ys, zs);
+            nf[0] = active ? (uint32_t)P.flag_new[n] : 1u;
+#pragma unroll
+            for (int i = 1; i < Q; i++) {
+                const int sx = xs[1 - L::e(i, 0)], sy = ys[1 - L::e(i, 1)], sz = zs[1 - L::e(i, 2)];
+                const bool wall = (sx | sy | sz) < 0;
+                nf[i] = (!active || wall) ? kWall : (uint32_t)P.flag_new[sx + P.nx * (sy + P.ny * sz)];
+            }
+        }
+        if (r == 0) load_particle_records(P, sp, cnt, bx0, by0, bz0);  // ids staged by the caller
+        fluid[r] = active && nf[0] == 0;
+        links[r] = 0;
+        if (fluid[r]) {
+#pragma unroll
+            for (int i = 1; i < Q; i++)
+                if (nf[i] != 0 && nf[i] != kWall) links[r] |= 1u << i;
+        }
+        if (active && !fluid[r] && P.missing_force) {
+            // per listed particle j, the directions whose neighbour is neither a
+            // fluid node next to j's own node nor a node of j
+            const int owner = (int)nf[0] - 1;
+            for (int s = 0; s < sp.n; s++) {
+                const int j = sp.id[s];
+                // a node outside another particle's bounding sphere is not inside
+                // it: solid_links would find nothing
+                if (j != owner && !in_bound(P, sp, s, lx, ly, lz)) continue;
+                uint32_t cand = 0;
+#pragma unroll
+                for (int i = 1; i < Q; i++) {
+                    const bool seen = (nf[i] == 0 && j == owner) || nf[i] == (uint32_t)(j + 1);
+                    if (!seen) cand |= 1u << i;
+                }
+                if (cand) nterms += solid_links<S, Q>(P, sp, s, j == owner, cand, lx, ly, lz, bx0, by0, bz0, sink);
+            }
         }
     }
     {
         // the brick's links in one queue; each warp evaluates 32 of them at a
         // time, then each node takes its results back
-        const int mine = __popc(links);
+        int mine = 0;
+#pragma unroll
+        for (int r = 0; r < kRows; r++) mine += __popc(links[r]);
         int incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -715,32 +729,35 @@ __device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, d
         __syncthreads();
         int first = incl - mine, total = 0;
 #pragma unroll
-        for (int w = 0; w < BRICK / 32; w++) {
+        for (int w = 0; w < kWarps; w++) {
             const int v = ls->warp_links[w];
             if (w < warp) first += v;
             total += v;
         }
         {
-            uint32_t m = links;
-            for (int k = first; m; k++) {
-                const int i = __ffs(m) - 1;
-                m &= m - 1;
-                ls->entry[k] = (unsigned short)((tid << 5) | i);
-            }
+            int k = first;
+#pragma unroll
+            for (int r = 0; r < kRows; r++)
+                for (uint32_t m = links[r]; m; m &= m - 1)
+                    ls->slot[k++] = (uint32_t)(((tid + r * kThreads) << 5) | (__ffs(m) - 1));
         }
         __syncthreads();
         // the force terms of a warp's 32 links are summed over the warp (no
-        // per-link atomics on the warp's totals).  The first warps of the two
-        // CTAs of an SM would share its sub-partitions: half the grid starts
-        // two further on (exact sums only: FP64 partials keep one order).
-        const int turn = sizeof(C) == 8 || blockIdx.x >= gridDim.x / 2 ? warp : (warp + BRICK / 32 - 2) % (BRICK / 32);
-        for (int r = turn * 32; r < total; r += BRICK) {
+        // per-link atomics on the warp's totals).  The first warps of an SM's
+        // CTAs would share its sub-partitions: the CTAs start at different ones
+        // (exact sums only: FP64 partials keep one order).
+        int turn = warp;
+        if (sizeof(C) == 4) {
+            if (kWarps == 8) turn = blockIdx.x >= gridDim.x / 2 ? warp : (warp + kWarps - 2) % kWarps;
+            else turn = (warp + (int)blockIdx.x) % kWarps;
+        }
+        for (int r = turn * 32; r < total; r += kThreads) {
             const int e = r + lane;
             LinkTerms lt;
             lt.s = -1;
             if (e < total) {
-                const int ent = ls->entry[e];
-                const int t = ent >> 5, i = ent & 31;  // the node's thread in the brick, the direction
+                const int ent = (int)ls->slot[e];
+                const int t = ent >> 5, i = ent & 31;  // the node in the brick, the direction
                 ForceSink<C> ds = sink;
                 ds.defer = &lt;
                 const C val = link_coop<S, Q>(P, sp, i, t % BX, (t / BX) % BY, t / (BX * BY), bx0, by0, bz0, ds);
@@ -748,24 +765,29 @@ __device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, d
                     const int tn = (bx0 + t % BX) + P.nx * ((by0 + (t / BX) % BY) + P.ny * (bz0 + t / (BX * BY)));
                     Cd::st(B + (long long)i * N + tn, val, (C)0, rho0);
                 } else {
-                    ls->result[e] = (float)val;
+                    ls->slot[e] = __float_as_uint((float)val);
                 }
                 nlinks++;
             }
             if (sizeof(C) == 4) warp_add_terms(ls->fix[warp], cnt, lt, lane);
         }
         __syncthreads();
-        if (fluid) {
-            // pull after the link evaluation: populations held across the
-            // out-of-line link calls would be spilled around them
+        int k = first;
+#pragma unroll
+        for (int r = 0; r < kRows; r++) {
+            if (!fluid[r]) continue;
+            const int node = tid + r * kThreads;
+            const int x = bx0 + node % BX, y = by0 + (node / BX) % BY, z = bz0 + node / (BX * BY);
+            const int n = x + P.nx * (y + P.ny * z);
+            // pull after the link evaluation: populations held across it would
+            // be spilled
             C fin[Q];
             plain_pull<S, Q, false>(P, x, y, z, n, fin);
-            int k = first;
 #pragma unroll
             for (int i = 1; i < Q; i++) {
-                if (links & (1u << i)) {  // link results are offsets g
+                if (links[r] & (1u << i)) {  // link results are offsets g
                     const C g = sizeof(C) == 8 ? Cd::ld_plain(B + (long long)i * N + n, (C)L::w(i), rho0)
-                                               : (C)ls->result[k];
+                                               : (C)__uint_as_float(ls->slot[k]);
                     fin[i] = Cd::g_to_v(g, (C)L::w(i));
                     k++;
                 }
@@ -798,7 +820,7 @@ __device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, d
             __syncthreads();
             if (tid < 6) {
                 double t = 0.0;
-                for (int w = 0; w < BRICK / 32; w++) t += red[w][tid];
+                for (int w = 0; w < kWarps; w++) t += red[w][tid];
                 P.partial[((long long)b * MAXPB + s) * 6 + tid] = t;
             }
             __syncthreads();
@@ -860,10 +882,12 @@ struct NearStage {
     int brick[kNearClaim], cnt[kNearClaim];  // -1: nothing to do; listed particles, 0: the plain path
     int id[kNearClaim][MAXPB];
 };
-template <typename S, int Q, bool kForce, bool kSplit = false>
+template <typename S, int Q, bool kForce, bool kSplit, int kThreads>
 __device__ __forceinline__ void near_work(const Params &P, SmemParticles &sp, double (*red)[6], int &s_links,
-                                          LinkScratch &ls, NearStage &st, int ctas) {
+                                          LinkScratch<kThreads / 32> &ls, NearStage &st, int ctas) {
     static_assert(MAXPB <= 32, "a lane per listed particle");
+    static_assert(kSplit || kThreads == BRICK, "a thread per node on the plain path");
+    constexpr int kClaim = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int t = P.step;
     const int c_exact = P.counters[CNT_LISTED];
@@ -872,7 +896,7 @@ __device__ __forceinline__ void near_work(const Params &P, SmemParticles &sp, do
     int done = 0;
     Claim nxt = {0, 0};
     const auto claim = [&](int from) {
-        nxt.size = from >= c_exact ? kNearClaim : min(max((c_exact - from) / (4 * ctas), 1), kNearClaim);
+        nxt.size = from >= c_exact ? kClaim : min(max((c_exact - from) / (4 * ctas), 1), kClaim);
         nxt.first = atomicAdd(&P.counters[CNT_NEAR_NEXT], nxt.size);
     };
     if (tid == 0) claim(0);
@@ -927,19 +951,20 @@ __device__ __forceinline__ void near_work(const Params &P, SmemParticles &sp, do
                 s_links = 0;
             }
             __syncthreads();
-            near_brick<S, Q, kForce>(P, sp, red, &s_links, &ls, b, bx0, by0, bz0, cnt);
+            near_brick<S, Q, kForce, kThreads>(P, sp, red, &s_links, &ls, b, bx0, by0, bz0, cnt);
         }
     }
     if (tid == 0 && done) atomicAdd(&P.counters[CNT_NEAR], done);
 }
 template <typename S, int Q, bool kForce, bool kMany>
-__global__ void __launch_bounds__(BRICK, kNearCtas<S, kMany>) k_sweep_near(Params P) {
+__global__ void __launch_bounds__(kNearThreads<S, kMany>, kNearCtas<S, kMany>) k_sweep_near(Params P) {
+    constexpr int kThreads = kNearThreads<S, kMany>;
     __shared__ SmemParticles sp;
-    __shared__ double red[BRICK / 32][6];
+    __shared__ double red[kThreads / 32][6];
     __shared__ int s_links;
-    __shared__ LinkScratch ls;
+    __shared__ LinkScratch<kThreads / 32> ls;
     __shared__ NearStage st;
-    near_work<S, Q, kForce, true>(P, sp, red, s_links, ls, st, gridDim.x);
+    near_work<S, Q, kForce, true, kThreads>(P, sp, red, s_links, ls, st, gridDim.x);
 }
 
 // The bricks of the near set that hold no particle link, as the near sweep

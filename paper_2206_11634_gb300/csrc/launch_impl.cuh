@@ -50,14 +50,15 @@ void launch_sweep_plain_t(const Params &P, cudaStream_t st) {
 template <typename S, bool kMany>
 void launch_sweep_near_n(const Params &P, cudaStream_t st) {
     const bool force = P.F[0] != 0.0 || P.F[1] != 0.0 || P.F[2] != 0.0;
-    const int cap = P.chain_grid > 0 ? P.chain_grid : kNearCtas<S, kMany> * sm_count();
+    constexpr int kThreads = kNearThreads<S, kMany>;
+    const int cap = P.chain_grid > 0 ? P.chain_grid * (BRICK / kThreads) : kNearCtas<S, kMany> * sm_count();
     const int grid = P.nbricks < cap ? P.nbricks : cap;
     if (P.Q == 19) {
-        if (force) k_sweep_near<S, 19, true, kMany><<<grid, BRICK, 0, st>>>(P);
-        else k_sweep_near<S, 19, false, kMany><<<grid, BRICK, 0, st>>>(P);
+        if (force) k_sweep_near<S, 19, true, kMany><<<grid, kThreads, 0, st>>>(P);
+        else k_sweep_near<S, 19, false, kMany><<<grid, kThreads, 0, st>>>(P);
     } else {
-        if (force) k_sweep_near<S, 15, true, kMany><<<grid, BRICK, 0, st>>>(P);
-        else k_sweep_near<S, 15, false, kMany><<<grid, BRICK, 0, st>>>(P);
+        if (force) k_sweep_near<S, 15, true, kMany><<<grid, kThreads, 0, st>>>(P);
+        else k_sweep_near<S, 15, false, kMany><<<grid, kThreads, 0, st>>>(P);
     }
 }
 template <typename S>
