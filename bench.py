@@ -526,8 +526,8 @@ def run_gpu(args):
 def run_batch(args):
     """Workload 5: 64 independent periodic drag cases, sides 48..128, one
     fixed metaball each, stepped as a batch (one launch per kernel for all
-    cases, replayed CUDA graphs; the fixed geometry is recorded once and every
-    later step is the link and plain kernels of the fixed-geometry sweep)
+    cases; the fixed geometry is recorded once and every later step is the
+    link and plain kernels of the fixed-geometry sweep)
     after the autotuner picked the schedule.  value = aggregate MLUPS over all
     cases."""
     import torch

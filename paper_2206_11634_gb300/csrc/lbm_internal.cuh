@@ -750,8 +750,9 @@ void launch_dem64c(const Params &P, cudaStream_t st);  // k_dem32.cu
 // Batched lattices (lbm_batch_*): independent cases stepped together, one
 // launch per phase for all cases.  Each case keeps the single-lattice layout
 // in its own part of the workspace; its Params live in a device table with
-// one row per step parity, and the step numbers come from device counters, so
-// a captured CUDA graph replays correctly.
+// one row per step parity.  The step numbers of brick steps come from device
+// counters, so a captured CUDA graph replays correctly; the fixed-geometry
+// steps take their parity from the host and are launched directly.
 // ---------------------------------------------------------------------------
 struct BatchArgs {
     const Params *tab;      // [2][ncases], row = step parity

@@ -330,7 +330,7 @@ class Lattice:
 
 class Batch:
     """Independent lattices stepped together (lbm_batch_*): one launch per
-    phase for all cases, the steps of a call run as a captured CUDA graph.
+    phase for all cases.
     cases: list of make_config keyword dicts, each with nx, ny, nz."""
 
     def __init__(self, cases: list, *, device: str = "cuda", stream=None):
