@@ -27,6 +27,7 @@
 
 #include "k_flags.cuh"
 #include "k_plain.cuh"
+#include "row_index.cuh"
 
 namespace lbmmb {
 // Resident CTAs per SM of the fixed-geometry link kernels and of the batched
@@ -660,20 +661,17 @@ __device__ __forceinline__ void near_brick(const Params &P, SmemParticles &sp, d
         uint32_t nf[Q];
         if (P.idx32 && y > 0 && y < P.ny - 1 && z > 0 && z < P.nz - 1) {
             // a row off the y and z faces (a warp is a row): one subtraction per
-            // neighbour, corrected on the x-face lanes (plain_pull's indices).
-            // Lanes past the row's end read inside the lattice too.
-            const int nx = P.nx, nxy = P.nx * P.ny;
-            int cm = 0, cp = 0;
-            bool wm = false, wp = false;
-            if (x == 0) { if (P.per[0]) cm = nx; else wm = true; }
-            if (x == nx - 1) { if (P.per[0]) cp = -nx; else wp = true; }
-            nf[0] = active ? (uint32_t)P.flag_new[(unsigned)n] : 1u;
+            // neighbour (row_index.cuh).  Lanes past the row's end read as its
+            // last node does.
+            const int xl = min(x, P.nx - 1), nl = n - (x - xl), nxy = P.nx * P.ny;
+            const RowLane row = row_lane(xl, P.nx, P.per[0] != 0);
+            nf[0] = active ? (uint32_t)P.flag_new[(unsigned)nl] : 1u;
 #pragma unroll
             for (int i = 1; i < Q; i++) {
                 const int ex = L::e(i, 0);
-                const uint32_t f = P.flag_new[(unsigned)(n - (ex + nx * L::e(i, 1) + nxy * L::e(i, 2)) +
-                                                        (ex > 0 ? cm : (ex < 0 ? cp : 0)))];
-                nf[i] = (!active || (ex > 0 && wm) || (ex < 0 && wp)) ? kWall : f;
+                const uint32_t f =
+                    P.flag_new[(unsigned)row_neighbour(nl, P.nx, nxy, row, ex, L::e(i, 1), L::e(i, 2))];
+                nf[i] = (!active || row_wall(row, ex)) ? kWall : f;
             }
         } else {
             int xs[3], ys[3], zs[3];
