@@ -136,6 +136,35 @@ __global__ void __launch_bounds__(256) k_bin(Params P) {
     if ((int)blockIdx.x < P.np) bin_particle(P, blockIdx.x);
 }
 
+// The work lists of step - 1 as its binning would have left them, for a brick
+// step that follows fixed-geometry steps, which bin nothing: the bricks listed
+// at step `from` (the last with a flag pass; the flags have not changed since)
+// as this step's predicted near set, so that the plain sweep, which may run
+// beside the flag pass, leaves the nodes it refills and their neighbours alone;
+// and as the one older list that the flag pass looks at, so that it visits a
+// brick once.  The rings' other slots start empty.  One CTA, once per
+// lbm_set_particles at most.
+__global__ void __launch_bounds__(1024) k_relist(Params P, int from) {
+    const int t = P.step, last = (t + 2) % 3;
+    const int count = P.wl_count[from % 3];
+    for (int k = threadIdx.x; k < count; k += blockDim.x) {
+        const int b = P.wl_list[(from % 3) * P.nbricks + k];
+        P.wl_list[last * P.nbricks + k] = b;  // (in place when from and step - 1 share a slot)
+        P.stamp[b] = t - 1;
+        P.pred_stamp_cur[b] = t;
+        P.pred_list_cur[k] = b;
+        P.skip[(t % 3) * P.nbricks + b] = t;
+    }
+    __syncthreads();  // every thread has the count
+    if (threadIdx.x == 0) {
+        P.wl_count[last] = count;
+        P.wl_count[(t + 1) % 3] = 0;
+        P.pred_count[t % 3] = count;
+        P.pred_count[(t + 1) % 3] = 0;  // (the binning clears the third)
+    }
+}
+void launch_relist(const Params &P, int from, cudaStream_t st) { k_relist<<<1, 1024, 0, st>>>(P, from); }
+
 // Batched binning: one CTA per (case, particle), at least one per case.  The
 // first CTA of a case also clears the other parity's per-step region for the
 // next step (the forces of this step's predecessor stay readable until then).

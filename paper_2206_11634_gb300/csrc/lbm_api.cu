@@ -212,6 +212,7 @@ struct lbm_handle {
     int plain_after_near; // the plain sweep of a step follows its near sweep (else runs beside the chain)
     int plain_spec_mode;  // lbm_set_plain_speculation: -1 auto (plain_spec), 0 off, 1 on
     int64_t steps;
+    int64_t bin_step, flag_step;  // the last steps that ran the binning and the flag pass (-1: none)
     char err[256];
 };
 
@@ -546,6 +547,7 @@ int init_handle(const lbm_config *cfg, void *dev_ws, size_t ws_bytes, void *cuda
         h->chain_per_sm = kDefaultChainPerSm;
         h->plain_spec = 1;
         h->near_expected = 0;
+        h->bin_step = h->flag_step = -1;
         h->plain_after_near = 1;
         h->plain_spec_mode = -1;
         h->bin_clean[0] = h->bin_clean[1] = 1;  // the workspace is cleared below
@@ -871,6 +873,7 @@ int lbm_step(lbm_handle *h, int nsteps) {
         if (fixed_sweep && h->static_state == 0) {
             // record the fixed geometry once, from this step's brick lists
             { ProfScope s(h, 0, true, hs); launch_bin(P, hs); }
+            h->bin_step = h->steps;
             h->bin_clean[rp ^ 1] = 1;
             e = cudaMemsetAsync(h->ws + h->L.sskip, 0, (size_t)h->L.N, hs);
             if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + h->L.scount, 0, 8, hs);
@@ -921,11 +924,15 @@ int lbm_step(lbm_handle *h, int nsteps) {
                 if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
                 forked_aux = true;
             }
+            // after fixed-geometry steps, which bin nothing
+            if (h->bin_step != h->steps - 1) launch_relist(P, (int)h->flag_step, hs);
             { ProfScope s(h, 0, true, hs); launch_bin(P, hs); }
+            h->bin_step = h->steps;
             h->bin_clean[rp ^ 1] = 1;
             e = cudaEventRecord(h->ev_bin, hs);
             if (e != cudaSuccess) return cuda_check(h, e, "event record");
             { ProfScope s(h, 1, !geom_static, hs); if (!geom_static) by_storage<DoFlags>(h->cfg.storage, P, hs); }
+            if (!geom_static) h->flag_step = h->steps;
             // the near sweep reads the halo the previous plain sweep wrote (this
             // wait is issued before ev_plain is recorded again below; the plain
             // sweep of the call before was joined into `stream` before the fork,
@@ -1674,6 +1681,13 @@ int lbm_batch_step(lbm_batch *b, int nsteps) {
                       "cudaMemcpyAsync(counters)");
     };
     if (direct > 0) {
+        // after fixed-geometry steps, which bin nothing (ctr_steps - 1 was the
+        // last brick step, and ran the flag pass)
+        for (int c = 0; c < b->n && b->ctr_steps != b->steps; c++) {
+            Params P = b->tab_host[(size_t)(b->steps & 1) * b->n + c];
+            P.step = (int)b->steps;
+            launch_relist(P, (int)(b->ctr_steps - 1), b->cap);
+        }
         rc = set_counters(b->steps);
         if (rc == LBM_OK) rc = batch_issue(b, direct, true);
         b->ctr_steps += direct;

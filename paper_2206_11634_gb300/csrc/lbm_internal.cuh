@@ -739,6 +739,7 @@ inline void launch_pdl(void (*kernel)(K...), dim3 grid, int block, cudaStream_t 
 
 // Launchers of the particle-side kernels (k_particles.cu).
 void launch_bin(const Params &P, cudaStream_t st);
+void launch_relist(const Params &P, int from, cudaStream_t st);  // before the binning of P.step
 void launch_force_reduce(const Params &P, cudaStream_t st);
 // st2 and the two events serve the FP64-integrator DEM (inactive particles on
 // st2, forked from st after the plan and joined back)
