@@ -36,12 +36,12 @@
 // ceil(sqrt(T)) steps instead and run each segment forward again from it.
 //
 // A step, forward or adjoint, is two kernels on disjoint nodes in programmatic
-// dependent launches (as the fixed-geometry sweep, k_static.cuh): one for the
-// fluid nodes with links, whose links are spread over a warp's lanes, and one
-// for the others, over 256-node spans.  96^3, T = 500, on a GB300: forward
-// 27 us a step (44 with the links of a node one after another in its thread),
-// adjoint 30 (113, with a recomputed forward step, a second gather and a
-// separate atomic scatter per link); 32^3: 5.6 and 5.7 (18 and 42).
+// dependent launches, ordered as the fixed-geometry sweep's (k_static.cuh): one
+// over 256-node spans for the nodes without links, then one for the fluid nodes
+// with links, whose links are spread over a warp's lanes.  96^3, T = 500, on a
+// GB300: forward 28 us a step (44 with the links of a node one after another in
+// its thread), adjoint 29 (113, with a recomputed forward step, a second gather
+// and a separate atomic scatter per link); 32^3: 5.7 and 6.5 (18 and 42).
 //
 // Finally dJ/dq goes through Eq. (27) and Eq. (4) to the control points and
 // weights (FP64).
@@ -214,6 +214,7 @@ struct AdjDev {
     unsigned long long *J_fix;  // sum of the window's drag (2^-40 units)
     double *grad;             // [ncp][4]: dJ/dx, dJ/dy, dJ/dz, dJ/dK
     float inv_W;
+    StepGate gate;
 };
 // What a forward step keeps for the adjoint (mom NULL: nothing).
 struct Kept {
@@ -348,13 +349,14 @@ __device__ __forceinline__ void adj_collide(const AdjConst &A, const float (&g)[
     }
 }
 
-// Forward step S -> R, the nodes without links (k_static_plain's waits).
-// Six CTAs per SM (40 registers): what bounds it is how many loads are in
-// flight beside the arithmetic; 96^3 at 4 / 5 / 6: 30.5, 28.9, 27.5 us a step.
+// Forward step S -> R, the nodes without links.  (S is not __restrict__: the
+// kernel is up before the step before has written it, which the read-only path
+// does not allow.)  Four CTAs per SM: with five and six (48 and 40 registers)
+// the pulled values are spilled; 96^3 at 4 / 5 / 6: 28.1, 28.9, 31.6 us a step.
 template <bool kForce, bool kWide>
-__global__ void __launch_bounds__(256, 6) k_adj_step(AdjDev D, const float *__restrict__ S, float *__restrict__ R,
-                                                      Kept kept, int reverse) {
-    pdl_launch_dependents();
+__global__ void __launch_bounds__(256, 4) k_adj_step(AdjDev D, const float *S, float *R, Kept kept, int reverse) {
+    pdl_wait();
+    gate_open(D.gate);
     const AdjConst &A = D.c;
     const int n = span_node(reverse != 0);
     if (n < A.N) {
@@ -365,7 +367,6 @@ __global__ void __launch_bounds__(256, 6) k_adj_step(AdjDev D, const float *__re
         for (int i = 0; i < Q; i++) gin[i] = pop<kWide>(S, A, i)[(unsigned)upstream(o, i)];
         if (take) adj_collide<kForce, kWide>(A, gin, n, R, kept.mom);
     }
-    pdl_wait();
 }
 
 // Forward step S -> R, the nodes with links: a warp takes kLinkNodes of them,
@@ -378,15 +379,19 @@ template <bool kForce>
 __global__ void __launch_bounds__(256, 2) k_adj_step_links(AdjDev D, const float *S, float *R, Kept kept, int window) {
     __shared__ unsigned short s_ent[8][kLinkNodes * 18];
     __shared__ float s_val[8][kLinkNodes * 18];
-    pdl_wait();
     pdl_launch_dependents();
     const AdjConst &A = D.c;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int w0 = (blockIdx.x * 8 + warp) * kLinkNodes;
-    if (w0 >= D.nnodes) return;
+    // (the node list is lbm_adj_init's: read before the gate)
     const bool has = lane < kLinkNodes && w0 + lane < D.nnodes;
     const int n = has ? D.n_node[w0 + lane] : 0, base = has ? D.n_base[w0 + lane] : 0;
     const uint32_t lm = has ? D.n_mask[w0 + lane] : 0u;
+    gate_pass(D.gate);
+    if (w0 >= D.nnodes) {
+        pdl_wait();
+        return;
+    }
     const int first_link = __shfl_sync(0xffffffffu, base, 0);
     const int first = base - first_link;  // the nodes' links follow one another
     int total = __popc(lm);
@@ -463,6 +468,7 @@ __global__ void __launch_bounds__(256, 2) k_adj_step_links(AdjDev D, const float
         for (int o = 16; o > 0; o >>= 1) drag += __shfl_xor_sync(0xffffffffu, drag, o);
         if (lane == 0 && drag) atomicAdd(D.J_fix, (unsigned long long)drag);
     }
+    pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -512,10 +518,10 @@ __device__ __forceinline__ float4 back_ab(const AdjConst &A, const BackSums &s, 
 // the next) and that the link kernel sums for the next step.
 // Four CTAs per SM: 96^3 at 3 / 4: 33.6, 31.2 us a step.
 template <bool kForce, bool kWide>
-__global__ void __launch_bounds__(256, 4) k_adj_back(AdjDev D, const float4 *__restrict__ mom,
-                                                      const float *__restrict__ lamN, float *__restrict__ lamT,
+__global__ void __launch_bounds__(256, 4) k_adj_back(AdjDev D, const float4 *mom, const float *lamN, float *lamT,
                                                       float4 *share, int reverse) {
-    pdl_launch_dependents();
+    pdl_wait();
+    gate_open(D.gate);
     const AdjConst &A = D.c;
     const int n = span_node(reverse != 0);
     if (n < A.N) {
@@ -560,36 +566,40 @@ __global__ void __launch_bounds__(256, 4) k_adj_back(AdjDev D, const float4 *__r
             }
         }
     }
-    pdl_wait();
 }
 
 // Adjoint step, the nodes with links: one warp per node, lane i its direction
 // i, so a node's links and their kept derivatives are read in one round.
 __global__ void __launch_bounds__(256) k_adj_back_links(AdjDev D, Kept kept, const float *lamN, float *lamT,
                                                          float4 *share, float4 *share_next, int window) {
-    pdl_wait();
     pdl_launch_dependents();
     const AdjConst &A = D.c;
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (w >= D.nnodes) return;
-    const int n = D.n_node[w], base = D.n_base[w];
-    const uint32_t lm = D.n_mask[w];
+    // (the node list and the links are lbm_adj_init's, q the forward call's:
+    // read before the gate)
+    const bool has = w < D.nnodes;
+    const int n = has ? D.n_node[w] : 0, base = has ? D.n_base[w] : 0;
+    const uint32_t lm = has ? D.n_mask[w] : 0u;
     const bool dir = lane < Q;
     const bool link = dir && ((lm >> lane) & 1u);
     const int L = base + __popc(lm & ((1u << lane) - 1u));
+    const int nff = link ? D.l_nff[L] : -1;
+    const float q = link ? D.l_q[L] : 0.f;
+    gate_pass(D.gate);
+    if (!has) {
+        pdl_wait();
+        return;
+    }
     const int ei[3] = {dir ? lat_e<19>(lane, 0) : 0, dir ? lat_e<19>(lane, 1) : 0, dir ? lat_e<19>(lane, 2) : 0};
     const float ex = (float)ei[0], ey = (float)ei[1], ez = (float)ei[2];
     const float wi = dir ? (float)lat_w<19>(lane) : 0.f;
     const float4 mo = kept.mom[n];
     const float4 x = share[n];
     float lam = dir ? lamN[(long long)lane * A.N + n] : 0.f;
-    int nff = -1;
-    float q = 0.f, gq = 0.f;
+    float gq = 0.f;
     float4 gf = make_float4(0.f, 0.f, 0.f, 0.f), gff = gf;
     if (link) {
-        nff = D.l_nff[L];
-        q = D.l_q[L];
         gq = kept.l_gq[L];
         gf = kept.l_f[L];
         gff = kept.l_ff[L];
@@ -650,6 +660,7 @@ __global__ void __launch_bounds__(256) k_adj_back_links(AdjDev D, Kept kept, con
         own.w += __shfl_xor_sync(0xffffffffu, own.w, o);
     }
     if (lane == 0) atomicAdd(&share_next[n], own);
+    pdl_wait();
 }
 
 // dJ/dq -> dJ/d(control point position, weight) through Eq. (27) and Eq. (4).
@@ -704,7 +715,8 @@ struct lbm_adj {
     char *ws;
     cudaStream_t stream;
     size_t o_state[2], o_ckpt, o_kept, o_lam[2], o_share[2], o_kind, o_nnode, o_nbase, o_nmask, o_lnf, o_ldir, o_lnff,
-        o_lq, o_dqf, o_dqs, o_dJdq, o_cp, o_K, o_J, o_grad, total;
+        o_lq, o_dqf, o_dqs, o_dJdq, o_cp, o_K, o_J, o_grad, o_gate, total;
+    unsigned gate_id;        // steps issued (the gate's numbers)
     bool have_forward;
     char err[256];
 };
@@ -857,6 +869,7 @@ void adj_layout(lbm_adj *a) {
     a->o_K = take((size_t)a->ncp * 8);
     a->o_J = take(8);
     a->o_grad = take((size_t)a->ncp * 32);
+    a->o_gate = take(4);
     a->total = o;
 }
 
@@ -909,6 +922,8 @@ AdjDev adj_dev(lbm_adj *a) {
     D.J_fix = reinterpret_cast<unsigned long long *>(w + a->o_J);
     D.grad = reinterpret_cast<double *>(w + a->o_grad);
     D.inv_W = 1.0f / (float)a->W;
+    D.gate.word = reinterpret_cast<unsigned *>(w + a->o_gate);
+    D.gate.id = 0;  // set per step
     return D;
 }
 
@@ -930,8 +945,8 @@ float *state(lbm_adj *a, size_t off) { return reinterpret_cast<float *>(a->ws + 
 
 unsigned span_grid(const lbm_adj *a) { return (unsigned)((a->N + 255) / 256); }
 
-// The link kernels run with no link node too: the span kernel behind them
-// relies on their wait for the step before.
+// The link kernels run with no link node too: their completion stands for the
+// step's.
 unsigned link_grid(const lbm_adj *a, int per_block) {
     return (unsigned)std::max(1, (a->nnodes + per_block - 1) / per_block);
 }
@@ -939,28 +954,30 @@ unsigned link_grid(const lbm_adj *a, int per_block) {
 // One forward step S -> R on the stream, one adjoint step lamN -> lamT.
 template <bool kForce, bool kWide>
 void forward_step_t(lbm_adj *a, const AdjDev &D, const float *S, float *R, const Kept &kept, int window, int t) {
-    launch_pdl(k_adj_step_links<kForce>, dim3(link_grid(a, 8 * kLinkNodes)), 256, a->stream, D, S, R, kept, window);
     launch_pdl(k_adj_step<kForce, kWide>, dim3(span_grid(a)), 256, a->stream, D, S, R, kept, t & 1);
+    launch_pdl(k_adj_step_links<kForce>, dim3(link_grid(a, 8 * kLinkNodes)), 256, a->stream, D, S, R, kept, window);
 }
 template <bool kForce, bool kWide>
 void adjoint_step_t(lbm_adj *a, const AdjDev &D, const Kept &kept, const float *lamN, float *lamT, float4 *share,
                     float4 *share_next, int window, int t) {
-    launch_pdl(k_adj_back_links, dim3(link_grid(a, 8)), 256, a->stream, D, kept, lamN, lamT, share, share_next, window);
     launch_pdl(k_adj_back<kForce, kWide>, dim3(span_grid(a)), 256, a->stream, D, kept.mom, lamN, lamT, share, t & 1);
+    launch_pdl(k_adj_back_links, dim3(link_grid(a, 8)), 256, a->stream, D, kept, lamN, lamT, share, share_next, window);
 }
 template <typename... X>
-void forward_step(lbm_adj *a, const X &...x) {
+void forward_step(lbm_adj *a, AdjDev D, const X &...x) {
+    D.gate.id = ++a->gate_id;
     const bool force = a->cfg.force[0] != 0.0 || a->cfg.force[1] != 0.0 || a->cfg.force[2] != 0.0;
     const bool wide = a->N >= (1ll << 30);
-    if (wide) force ? forward_step_t<true, true>(a, x...) : forward_step_t<false, true>(a, x...);
-    else force ? forward_step_t<true, false>(a, x...) : forward_step_t<false, false>(a, x...);
+    if (wide) force ? forward_step_t<true, true>(a, D, x...) : forward_step_t<false, true>(a, D, x...);
+    else force ? forward_step_t<true, false>(a, D, x...) : forward_step_t<false, false>(a, D, x...);
 }
 template <typename... X>
-void adjoint_step(lbm_adj *a, const X &...x) {
+void adjoint_step(lbm_adj *a, AdjDev D, const X &...x) {
+    D.gate.id = ++a->gate_id;
     const bool force = a->cfg.force[0] != 0.0 || a->cfg.force[1] != 0.0 || a->cfg.force[2] != 0.0;
     const bool wide = a->N >= (1ll << 30);
-    if (wide) force ? adjoint_step_t<true, true>(a, x...) : adjoint_step_t<false, true>(a, x...);
-    else force ? adjoint_step_t<true, false>(a, x...) : adjoint_step_t<false, false>(a, x...);
+    if (wide) force ? adjoint_step_t<true, true>(a, D, x...) : adjoint_step_t<false, true>(a, D, x...);
+    else force ? adjoint_step_t<true, false>(a, D, x...) : adjoint_step_t<false, false>(a, D, x...);
 }
 
 }  // namespace
@@ -1000,8 +1017,9 @@ int lbm_adj_init(const lbm_config *cfg, const lbm_particle *p, int T, int W, voi
     a->ws = static_cast<char *>(dev_ws);
     a->stream = static_cast<cudaStream_t>(cuda_stream);
     a->have_forward = false;
+    a->gate_id = 0;
     std::snprintf(a->err, sizeof(a->err), "no error");
-    int rc = LBM_OK;
+    int rc = acheck(a, cudaMemsetAsync(a->ws + a->o_gate, 0, 4, a->stream), "cudaMemsetAsync");
     auto up = [&](size_t off, const void *src, size_t bytes) {
         if (rc == LBM_OK && bytes)
             rc = acheck(a, cudaMemcpyAsync(a->ws + off, src, bytes, cudaMemcpyHostToDevice, a->stream), "cudaMemcpyAsync");

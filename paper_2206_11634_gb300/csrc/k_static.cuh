@@ -163,28 +163,38 @@ __device__ __forceinline__ void static_plain_node(const Params &P, int n) {
     plain_pull<S, Q, true>(P, x, y, z, n, fin);
     if (!skip) collide_store<S, Q, kForce, true>(P, fin, (S *)P.fB, P.N, n);
 }
-// Step t's link kernel, then its plain kernel, then step t + 1's, all on one
-// stream as programmatic dependent launches: a kernel's CTAs come up while
-// the one before still runs.  The link kernel waits for the whole of step
-// t - 1 before it lets the plain kernel start, so that one reads nothing
-// unfinished and runs beside it on other nodes; it waits for the link kernel
-// only at its end, so its own completion stands for the whole step.  On two
+// Step t's two kernels, then step t + 1's, all on one stream as programmatic
+// dependent launches: a kernel's CTAs come up while the one before still runs.
+// The first of a step waits for the whole of step t - 1, then lets the second
+// start, which runs beside it on other nodes (ordered by the step's gate,
+// lbm_internal.cuh) and whose completion stands for the whole step.  On two
 // streams with events between them, and a memset a step, a step of the 48^3
-// drag box took 22.6 us, most of it gaps; this way 7.6.
+// drag box took 22.6 us, most of it gaps; this way 7.5, and 11.1 with the
+// kernels one after the other.  While all CTAs of the plain kernel run at once
+// (four per SM) the link kernel, the longer chain of loads, comes first; beyond
+// that the plain kernel, whose CTAs then have no gate to pass.  Plain kernel
+// first and second, us a step: 48^3 FP32 8.5 and 7.5, FP16 10.8 and 10.2; 64^3 12.1
+// and 12.6, 14.1 and 14.5; 96^3 25.6 and 27.0.
 //
 // The last CTA clears the step counters and force totals of the next step's
 // region (the binning, which clears it otherwise, does not run here); they
 // are those of step t - 1, whose kernels are done.
 template <typename S, int Q, bool kForce>
 __global__ void __launch_bounds__(BRICK, 4) k_static_plain(Params P) {
-    pdl_launch_dependents();
+    if (P.links_first) {
+        pdl_launch_dependents();
+        gate_pass(P.gate);
+    } else {
+        pdl_wait();
+        gate_open(P.gate);
+    }
     if (blockIdx.x == gridDim.x - 1) {
         int *tail = static_cast<int *>(P.bin_next) + P.nbricks;
         const int words = (int)(P.bin_next_bytes / 4) - P.nbricks;
         for (int k = threadIdx.x; k < words; k += BRICK) tail[k] = 0;
     }
     static_plain_node<S, Q, kForce>(P, blockIdx.x * BRICK + (int)threadIdx.x);
-    pdl_wait();
+    if (P.links_first) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -201,7 +211,7 @@ struct StaticScratch {
 // One link of node n (direction i, record r): the node's own populations,
 // x_ff's and the record fetched in one round, the unknown and the momentum
 // exchange with the recorded geometry; the force/torque terms in fixed point.
-// Coherent loads: the kernel is up before the step before has written them.
+// Coherent loads: the kernel can be up before the step before has written them.
 template <typename S, int Q>
 __device__ __forceinline__ float static_link(const Params &P, int n, int i, int r, int &j, LinkTerms &lt) {
     using L = Lat<Q>;
@@ -291,8 +301,19 @@ __device__ __forceinline__ void static_add_terms(const Params &P, const LinkTerm
     }
 }
 
-template <typename S, int Q, bool kForce, int kPer>
-__device__ __forceinline__ void static_links_warp(const Params &P, StaticScratch &ss, int wg) {
+// The lane's link node of warp wg (no links past the list's end).
+template <int kPer>
+__device__ __forceinline__ StaticNode static_node(const Params &P, int wg) {
+    const int lane = threadIdx.x & 31, idx = wg * kPer + lane;
+    StaticNode sn;
+    sn.n = 0;
+    sn.mask = 0u;
+    sn.base = 0;
+    if (lane < kPer && idx < P.snodes_n) sn = P.snodes[idx];
+    return sn;
+}
+template <typename S, int Q, bool kForce>
+__device__ __forceinline__ void static_links_warp(const Params &P, StaticScratch &ss, const StaticNode &sn) {
     using L = Lat<Q>;
     using Cd = Codec<S>;
     using C = typename Cd::C;
@@ -301,13 +322,7 @@ __device__ __forceinline__ void static_links_warp(const Params &P, StaticScratch
     S *B = (S *)P.fB;
     const long long N = P.N;
     const C rho0 = Prm<C>::rho0(P);
-    const int idx = wg * kPer + lane;
-    const bool has = lane < kPer && idx < P.snodes_n;
-    StaticNode sn;
-    sn.n = 0;
-    sn.mask = 0u;
-    sn.base = 0;
-    if (has) sn = P.snodes[idx];
+    const bool has = sn.mask != 0u;  // every listed node has links
     __syncwarp();  // the previous round of the warp is done with its queue
     ss.node[warp][lane] = sn.n;
     const uint32_t links = sn.mask;
@@ -381,12 +396,23 @@ template <typename S, int Q, bool kForce, int kPer>
 __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links(Params P) {
     if (sizeof(typename Codec<S>::C) == 8) return;
     __shared__ StaticScratch ss;
-    pdl_wait();
-    pdl_launch_dependents();
-    if (blockIdx.x == gridDim.x - 1) static_constants(P, threadIdx.x, BRICK);
     const int warps = (P.snodes_n + kPer - 1) / kPer;
-    for (int wg = blockIdx.x * (BRICK / 32) + (threadIdx.x >> 5); wg < warps; wg += gridDim.x * (BRICK / 32))
-        static_links_warp<S, Q, kForce, kPer>(P, ss, wg);
+    int wg = blockIdx.x * (BRICK / 32) + (int)(threadIdx.x >> 5);
+    StaticNode sn = static_node<kPer>(P, wg);  // (recorded before any of these steps: read before the wait)
+    if (P.links_first) {
+        pdl_wait();
+        gate_open(P.gate);
+    } else {
+        pdl_launch_dependents();
+        gate_pass(P.gate);
+    }
+    if (blockIdx.x == gridDim.x - 1) static_constants(P, threadIdx.x, BRICK);
+    while (wg < warps) {
+        static_links_warp<S, Q, kForce>(P, ss, sn);
+        wg += gridDim.x * (BRICK / 32);
+        sn = static_node<kPer>(P, wg);
+    }
+    if (!P.links_first) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -407,7 +433,8 @@ __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links(Params P
 // 64-case batch (six spilled 88 bytes and was 2-6 % slower).
 template <typename S, int Q, bool kForce>
 __global__ void __launch_bounds__(BRICK, 5) k_static_plain_batch(BatchArgs B) {
-    pdl_launch_dependents();
+    pdl_wait();
+    gate_open(B.gate);
     const int total = B.span_off[B.ncases];
     const Params *row = B.tab + (size_t)B.parity * B.ncases;
     const int g0 = blockIdx.x * B.plain_chunk;
@@ -435,7 +462,6 @@ __global__ void __launch_bounds__(BRICK, 5) k_static_plain_batch(BatchArgs B) {
         }
         static_plain_node<S, Q, kForce>(P, (g - B.span_off[c]) * BRICK + (int)threadIdx.x);
     }
-    pdl_wait();
 }
 
 // One warp per kStaticNodesPerWarp link nodes of a case (each case at least one
@@ -443,17 +469,19 @@ __global__ void __launch_bounds__(BRICK, 5) k_static_plain_batch(BatchArgs B) {
 template <typename S, int Q, bool kForce>
 __global__ void __launch_bounds__(BRICK, kNearCtasPerSm) k_static_links_batch(BatchArgs B) {
     __shared__ StaticScratch ss;
-    pdl_wait();
     pdl_launch_dependents();
-    const Params *row = B.tab + (size_t)B.parity * B.ncases;
     const int warps = B.swarp_off[B.ncases];
     const int gw = blockIdx.x * (BRICK / 32) + (int)(threadIdx.x >> 5);
-    if (gw >= warps) return;
-    const int c = case_of(B.swarp_off, B.ncases, gw);  // whose warp range holds gw
-    const Params &P = row[c];
+    const int c = case_of(B.swarp_off, B.ncases, min(gw, warps - 1));  // whose warp range holds gw
+    const Params &P = B.tab[(size_t)B.parity * B.ncases + c];
     const int wl = gw - B.swarp_off[c];
-    if (wl == 0) static_constants(P, threadIdx.x & 31, 32);
-    if (wl * kStaticNodesPerWarp < P.snodes_n) static_links_warp<S, Q, kForce, kStaticNodesPerWarp>(P, ss, wl);
+    const StaticNode sn = static_node<kStaticNodesPerWarp>(P, wl);  // (recorded before any of these steps)
+    gate_pass(B.gate);
+    if (gw < warps) {
+        if (wl == 0) static_constants(P, threadIdx.x & 31, 32);
+        if (wl * kStaticNodesPerWarp < P.snodes_n) static_links_warp<S, Q, kForce>(P, ss, sn);
+    }
+    pdl_wait();
 }
 
 }  // namespace lbmmb

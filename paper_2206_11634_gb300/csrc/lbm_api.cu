@@ -307,6 +307,11 @@ Params make_params(lbm_handle *h) {
     P.near_expected = h->near_expected;
     P.idx32 = (long long)c.lattice * (long long)c.nx * c.ny * c.nz <= 0x7fffffffLL;
     P.status = at<int>(h, h->L.status);
+    P.gate.word = reinterpret_cast<unsigned *>(P.status + ST_GATE);
+    P.gate.id = (unsigned)h->steps + 1;
+    // the order of the fixed-geometry step's kernels: the links first while all
+    // spans of the plain kernel run at once (k_static.cuh)
+    P.links_first = (c.nx * (long long)c.ny * c.nz + BRICK - 1) / BRICK <= 4 * h->nsm;
     P.counters = at<int>(h, bin_region(h, h->steps) + (size_t)h->L.nbricks * 4);
     P.force_fixed = h->cfg.storage != LBM_STORE_F64;
     P.Ffix = at<unsigned long long>(h, bin_region(h, h->steps) + h->L.ffix_off);
@@ -905,15 +910,19 @@ int lbm_step(lbm_handle *h, int nsteps) {
             if (e != cudaSuccess) return cuda_check(h, e, "cudaMemsetAsync(bricks)");
         }
         if (fixed_sweep && h->static_state == 1) {
-            // the link nodes, then the plain nodes beside them, in stream
-            // order (k_static.cuh); behind the plain sweep of a brick step
+            // the plain nodes and beside them the link nodes, in stream order
+            // (k_static.cuh); behind the plain sweep of a brick step
             if (plain_pending) {
                 e = cudaStreamWaitEvent(hs, h->ev_plain, 0);
                 if (e != cudaSuccess) return cuda_check(h, e, "stream wait");
                 plain_pending = false;
             }
-            { ProfScope s(h, 3, true, hs); by_storage<DoStaticLinks>(h->cfg.storage, P, hs); }
-            { ProfScope s(h, 2, true, hs); by_storage<DoStaticPlain>(h->cfg.storage, P, hs); }
+            for (int k = 0; k < 2; k++) {
+                const bool links = (P.links_first != 0) == (k == 0);
+                ProfScope s(h, links ? 3 : 2, true, hs);
+                if (links) by_storage<DoStaticLinks>(h->cfg.storage, P, hs);
+                else by_storage<DoStaticPlain>(h->cfg.storage, P, hs);
+            }
             // the plain kernel cleared the next region's counters and force
             // totals (the brick counts are only written by brick steps, which
             // do not follow before the particles are set again)
@@ -1333,7 +1342,7 @@ void batch_layout(const lbm_config *cfgs, int n, BatchLayout *B) {
     B->tab = take(2 * (size_t)n * sizeof(Params));
     B->span_off = take(((size_t)n + 1) * 4);
     B->item_off = take(((size_t)n + 1) * 4);
-    B->ctr = take(4 * 4);
+    B->ctr = take(5 * 4);  // step counters, finished CTAs, the fixed-geometry sweep's gate
     B->swarp_off = take(((size_t)n + 1) * 4);
     size_t spans = 0;
     for (int c = 0; c < n; c++) {
@@ -1454,14 +1463,16 @@ void by_batch_storage(int storage, Fn &&fn) {
 }
 
 // nsteps steps of the fixed-geometry sweep on b->cap, the first of them step
-// number `first`: the link and the plain kernel in stream order (k_static.cuh).
+// number `first`: the plain and the link kernel in stream order (k_static.cuh).
 int batch_issue_fixed(lbm_batch *b, int nsteps, int64_t first) {
     BatchArgs B = batch_args(b);
     const int plain_grid = (b->total_spans + b->plain_chunk - 1) / b->plain_chunk;
     for (int t = 0; t < nsteps; t++) {
         B.parity = (int)((first + t) & 1);
-        by_batch_storage(b->storage, [&](auto D) { D.static_links(B, b->Q, b->force, b->total_swarps, b->cap); });
+        B.gate.word = B.ctr + 4;
+        B.gate.id = (unsigned)(first + t) + 1;
         by_batch_storage(b->storage, [&](auto D) { D.static_plain(B, b->Q, b->force, plain_grid, b->cap); });
+        by_batch_storage(b->storage, [&](auto D) { D.static_links(B, b->Q, b->force, b->total_swarps, b->cap); });
     }
     return bcheck(b, cudaGetLastError(), "batched step launch");
 }

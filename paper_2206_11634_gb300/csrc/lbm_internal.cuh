@@ -30,7 +30,7 @@ constexpr int NWALL = 6;
 constexpr int ROT_ITERS = 2;  // fixed-point sweeps of the implicit rotational half-kick
 
 // Status words in the workspace.
-enum StatusSlot { ST_ERR = 0, ST_SLOTS = 16 };
+enum StatusSlot { ST_ERR = 0, ST_GATE = 1, ST_SLOTS = 16 };  // (ST_GATE: see StepGate)
 // CNT_NEAR_NEXT, CNT_FLAGS_NEXT: the brick queues of the near sweep and of
 // the flag pass (next entry to hand out)
 enum StepCounter { CNT_NREFILL = 0, CNT_NLINKS = 1, CNT_LISTED = 2, CNT_NEAR = 3, CNT_NEAR_NEXT = 4, CNT_FLAGS_NEXT = 5 };
@@ -342,6 +342,13 @@ __host__ __device__ __forceinline__ uint32_t fast_quot(uint32_t n, const FastDiv
 #endif
 }
 
+// What the second kernel of a fixed-geometry step passes (gate_open, gate_pass):
+// a device word that only those kernels write, and the step's number, from 1.
+struct StepGate {
+    unsigned *word;
+    unsigned id;
+};
+
 // Everything a kernel needs, passed by value.
 struct Params {
     int nx, ny, nz, Q;
@@ -421,6 +428,8 @@ struct Params {
     long long bin_next_bytes;
     int *dem_list;     // [8 + 8 np], k_dem64_plan's split of the particles (dem_free() and below)
     int *status;       // [ST_SLOTS], sticky error bits
+    StepGate gate;     // fixed-geometry sweep
+    int links_first;   // ... the order of its two kernels
     int *counters;     // per-step counters, zeroed with the brick lists
     // fixed-geometry sweep (every particle fixed, lattices below FP64): built
     // once by k_static_build, then every step runs k_static_plain over the
@@ -721,6 +730,35 @@ __device__ __forceinline__ void brick_coords(const Params &P, int b, int &bx, in
 // writes visible.  Both do nothing in a kernel launched the ordinary way.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Order for a step of two kernels on disjoint nodes that both read the step
+// before.  The first one waits (above), which makes the step before visible to
+// it, and lets the second start; that one runs beside it, so it cannot wait
+// before it reads (the wait is for the first one's end), and nothing but a
+// wait orders its reads after the step before.  So the first one's block 0
+// stores the step's number (release) before it lets the second start, and
+// every block of the second loads it (acquire): what was visible to the first
+// is then visible to the second.  A block that does not find the number there
+// waits for the first kernel.  The second kernel waits at its end, so that its
+// completion stands for the whole step.
+//
+// Where the larger kernel has several waves of blocks it comes first: passing
+// the gate costs a block 2 to 4 % (64 drag boxes: 1453 us a step, 1484 with the
+// larger kernel second), and the smaller one fills the last wave.
+__device__ __forceinline__ void gate_open(const StepGate &g) {
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(g.word), "r"(g.id) : "memory");
+        __syncthreads();
+    }
+    pdl_launch_dependents();
+}
+__device__ __forceinline__ void gate_pass(const StepGate &g) {
+    if (threadIdx.x == 0) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.word) : "memory");
+        if (v != g.id) pdl_wait();
+    }
+    __syncthreads();
+}
 // Launch that may start before the stream's previous kernel has ended (the
 // kernel itself waits, see above).
 template <typename... K, typename... A>
@@ -768,6 +806,7 @@ struct BatchArgs {
     const int *swarp_off;   // [ncases + 1] prefix sums of the cases' link-node warps (>= 1 each;
                             // fixed-geometry sweep)
     int parity;             // fixed-geometry sweep: parity of the step
+    StepGate gate;          // ... and its gate
 };
 
 // The case's Params for the current step into shared memory (all threads).
