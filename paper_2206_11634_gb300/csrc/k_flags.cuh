@@ -113,8 +113,9 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
         }
         if (tid == 0) sp.n = cnt;
     }
-    __shared__ unsigned s_faces;
-    if (tid == 0) s_faces = 0u;
+    constexpr bool kF64 = sizeof(typename Codec<S>::C) == 8;
+    __shared__ unsigned s_faces, s_far;
+    if (tid == 0) s_faces = s_far = 0u;
     __syncthreads();
     int bxi, byi, bzi;
     brick_coords(P, b, bxi, byi, bzi);
@@ -126,6 +127,19 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
     // the previous flag (the refill below needs it), issued with the
     // particles' loads so that the two latencies overlap
     const uint16_t old = active ? P.flag_old[n] : (uint16_t)0;
+    if (kF64) {
+        // listed particles (a bit each) whose FP32 positions the error band of
+        // metaball32 does not cover: farther than it says, many box lengths
+        // away along a periodic axis
+        for (int t = tid; t < cnt * MAXCP; t += BRICK) {
+            const DevParticle &p = P.parts[sp.id[t / MAXCP]];
+            const int k = t % MAXCP;
+            if (k < p.ncp && (fabsf(p.cpw_hl[k][0][0] - (float)bx0) > kBandReach ||
+                              fabsf(p.cpw_hl[k][1][0] - (float)by0) > kBandReach ||
+                              fabsf(p.cpw_hl[k][2][0] - (float)bz0) > kBandReach))
+                atomicOr(&s_far, 1u << (t / MAXCP));
+        }
+    }
     if (cnt > 0) load_particle_records(P, sp, cnt, bx0, by0, bz0);
 
     // owner: the covering particle with the largest M, ties to the lower
@@ -136,7 +150,7 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
     if (active && cnt > 0) {
         int own_s = -1;
         // FP64 lattices: thresholds at which FP32 has no band left
-        const bool exact = sizeof(typename Codec<S>::C) == 8 && !(P.c0_f > 1e-30f && P.c0_f < 1e30f);
+        const bool exact = kF64 && !(P.c0_f > 1e-30f && P.c0_f < 1e30f);
         double own_M = -1.0;  // FP64 M of the current owner, < 0 until computed
         for (int s = 0; s < cnt; s++) {
             if (!in_bound(P, sp, s, lx, ly, lz)) continue;  // outside s: M < c0 there
@@ -144,7 +158,7 @@ __device__ __forceinline__ void flags_brick(const Params &P, SmemParticles &sp, 
             const float M = metaball32(P, sp, s, (float)lx, (float)ly, (float)lz, unsure);
             bool inside;
             double Md = -1.0;
-            if (unsure || exact) {
+            if (unsure || exact || (kF64 && ((s_far >> s) & 1u))) {
                 Md = metaball64_far(P, P.parts[sp.id[s]], x, y, z);
                 inside = Md >= P.c0;
             } else {

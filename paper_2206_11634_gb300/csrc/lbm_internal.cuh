@@ -623,11 +623,12 @@ __device__ __forceinline__ bool in_bound(const Params &P, const SmemParticles &s
 // Error budget: the control point's brick-relative position is rounded once
 // to FP32 (from the FP32 pair of its FP64 value, see df_minus_int: within a
 // 2^-24 fraction of an ulp of that; |error| <= 2^-24 times its magnitude
-// plus 2^-48 of it, < 2^-16 for magnitudes
-// below 256), each difference along an axis is exact or rounded once, the
-// square sum, the reciprocal and the product add 5 roundings; for distances
-// r >= 1/2 each term K/r^2 is off by at most 2^-13 relative, well inside the
-// band.
+// plus 2^-48 of it, < 2^-16 for magnitudes below kBandReach), each difference
+// along an axis is exact or rounded once, the square sum, the reciprocal and
+// the product add 5 roundings; for distances r >= 1/2 each term K/r^2 is off by
+// at most 2^-13 relative, well inside the band.  (Positions farther than
+// kBandReach along an axis: FP64 lattices evaluate M in FP64 there.)
+constexpr float kBandReach = 256.f;
 __device__ __forceinline__ float metaball32(const Params &P, const SmemParticles &sp, int s, float lx, float ly,
                                             float lz, bool &unsure) {
     float M = 0.f;
