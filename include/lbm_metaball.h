@@ -24,9 +24,9 @@
  *      metaball-metaball and metaball-wall contacts (§2.1.3-2.1.4, Eqs.
  *      (5)-(13)), the contact law of §2.1.1 (Eqs. (2)-(3)), velocity Verlet
  *      and Euler's equations in the body frame (Eq. (1)).  By default the
- *      rigid-body integrator is FP64, and so is the contact geometry on FP64
+ *      rigid-body state is FP64, and so is the contact geometry on FP64
  *      lattices; below FP64 the contact geometry is FP32 (lbm_config.dem_mode
- *      gives the choices).
+ *      gives the choices and says what a particle without contact runs in).
  *
  * Units are lattice units: dx = dt = C = 1, c_s^2 = 1/3.  Node (i,j,k) sits
  * at position (i,j,k); a non-periodic face is a resting no-slip wall halfway
@@ -98,23 +98,26 @@ typedef struct lbm_config {
     int32_t missing_force;     /* 1 = add the missing-force-point terms of §2.3.5 item 2 */
     int32_t max_particles;     /* capacity reserved in the workspace, >= 1 */
     int32_t dem_mode;          /* arithmetic of the DEM (§2.1, §2.3.4), enum lbm_dem_mode.
-                                  0 (LBM_DEM_FP64, the default): the rigid-body state is FP64 and
-                                  every sub-step adds to it in FP64.  On FP64 lattices everything
-                                  is FP64.  On FP32/FP16/BF16 lattices a particle that cannot touch
-                                  a wall or another particle during the step (|v| + |a| + 0.25 lu
-                                  of reach) moves in FP64 arithmetic throughout (translation in
-                                  closed form, rotation sub-stepped); the others compute their
-                                  increments, contact geometry and contact law in FP32 (overlap
-                                  error ~1e-6 lu) and add the increments to the FP64 state; up to
-                                  256 particles with up to 2048 control points in all (else as
-                                  mode 2).
+                                  0 (LBM_DEM_FP64, the default): the rigid-body state is FP64.  A
+                                  particle that cannot touch a wall or another particle during the
+                                  step (|v| + |a| + 0.25 lu of reach; on FP64 lattices: no particle
+                                  can) moves to FP64's accuracy: translation in closed form in
+                                  FP64, rotation sub-stepped in FP64 or, with 8 sub-steps or more
+                                  and small angles, with the change within the step held in pairs
+                                  of FP32 (48 bits of a change of 2^-8 of the state at most; closer
+                                  to 128-bit arithmetic than FP64 sub-steps are).  With contact:
+                                  on FP64 lattices everything is FP64; on FP32/FP16/BF16 lattices
+                                  the increments, contact geometry and contact law are FP32
+                                  (overlap error ~1e-6 lu) and the increments are added to the
+                                  FP64 state; up to 256 particles with up to 2048 control points in
+                                  all (else FP64 contacts, as mode 2).
                                   1 (LBM_DEM_FP32_COMPENSATED): lattices below FP64 only (FP64
                                   lattices ignore it): every particle computes in FP32 and keeps
                                   its state as compensated FP32 pairs (about 48 significant bits),
                                   with the same limits; the fastest, below mode 0's accuracy for
                                   particles without contact.
-                                  2 (LBM_DEM_FP64_ALL): everything in FP64, contact geometry
-                                  included, on any lattice (one CTA; slow for many contacts on
+                                  2 (LBM_DEM_FP64_ALL): everything in FP64, contact geometry and
+                                  every rotation sub-step included, on any lattice (one CTA; slow for many contacts on
                                   this GPU, whose FP64 rate is a small fraction of its FP32 rate). */
     int32_t q_exact;           /* 0 = link fraction q by Eq. (27); 1 = the root of Eq. (26) by Newton's
                                   method from Eq. (27)'s value (§2.3.1: tolerance 1e-7, at most 100

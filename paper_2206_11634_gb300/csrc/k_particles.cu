@@ -1,4 +1,5 @@
-// Particle-side kernels, all FP64:
+// Particle-side kernels, FP64 (but for the rotation sub-steps of a free particle,
+// see rotate_free_quad, and the binning's bound of M):
 //   k_bin          world control points, search boxes, scatter into bricks;
 //   k_force_reduce per-particle totals of the sweep's brick partials;
 //   k_dem          n_sub DEM sub-steps (§2.3.4) with the hydrodynamic load
@@ -632,7 +633,8 @@ __device__ bool contact_possible(const Params &P) {
 // the quaternion's scalar part, lanes 1..3 its vector part and the x,y,z
 // components of every vector (lane 0's vector slot is unused), so the cross
 // products, the quaternion product and Euler's equations run one component
-// per lane with width-4 shuffles.  FP64 throughout.
+// per lane with width-4 shuffles.  In FP64, or (rotate_pairs) with the change
+// within the step in FP32 pairs.
 // ---------------------------------------------------------------------------
 // lanes of the quads that take part (whole quads); set by the caller
 __device__ __forceinline__ double qget(unsigned mask, double v, int lane) { return __shfl_sync(mask, v, lane, 4); }
@@ -836,8 +838,10 @@ __device__ bool rotate_pairs(unsigned mk, const QuadLanes &L, const DevParticle 
 // lanes of every quad of this warp that takes part.  Tw_lane: this lane's
 // component of the world-frame torque (lane 0: not used); the new attitude and
 // world angular velocity go to q_out[4] and w_out[3] (which may be p's own).
+// pairs: the sub-steps run in FP32 pairs where these are no less accurate than
+// FP64 (rot32_applies); else all of them run in FP64 (dem_mode 2 asks for that).
 __device__ void rotate_free_quad(unsigned mk, const DevParticle &p, double Tw_lane, double h, int n_sub,
-                                 double *q_out, double *w_out) {
+                                 bool pairs, double *q_out, double *w_out) {
     const QuadLanes L = quad_lanes();
     const int lane = L.lane;
     const int m = lane == 0 ? 0 : lane - 1;
@@ -850,7 +854,7 @@ __device__ void rotate_free_quad(unsigned mk, const DevParticle &p, double Tw_la
         if (lane > 0) w_out[m] = p.w[m];
         return;
     }
-    const bool done = rotate_pairs(mk, L, p, h, n_sub, q, wb, Tb);
+    const bool done = pairs && rotate_pairs(mk, L, p, h, n_sub, q, wb, Tb);
     const unsigned rest = __ballot_sync(mk, !done);
     if (!done) rotate_sub_steps(rest, L, p, h, n_sub, q, wb, Tb);
     __syncwarp(mk);
@@ -1032,8 +1036,8 @@ __global__ void __launch_bounds__(256) k_dem64_plan(Params P) {
 // runs beside it): the step of a particle that touches nothing, into its
 // record's step results (nx, nv, nq, nw).  Translation in closed form over
 // the unit step (x += v + a/2, v += a: what the n_s kick-drift-kick
-// sub-steps give under the constant force), rotation sub-stepped by
-// rotate_free_quad, all FP64.  The hydrodynamic load comes from the sweep's
+// sub-steps give under the constant force) in FP64, rotation sub-stepped by
+// rotate_free_quad.  The hydrodynamic load comes from the sweep's
 // fixed-point totals by the plan's conversion (the same bits as its Fh, Th).
 __global__ void __launch_bounds__(128) k_dem64_free(Params P) {
     const int np = P.np;
@@ -1052,7 +1056,8 @@ __global__ void __launch_bounds__(128) k_dem64_free(Params P) {
     }
     const unsigned mk = __ballot_sync(0xffffffffu, moving);
     if (moving)
-        rotate_free_quad(mk, p, (double)(long long)P.Ffix[6 * k + 3 + m] * kFix, 1.0 / P.n_sub, P.n_sub, p.nq, p.nw);
+        rotate_free_quad(mk, p, (double)(long long)P.Ffix[6 * k + 3 + m] * kFix, 1.0 / P.n_sub, P.n_sub, P.rot_pairs,
+                         p.nq, p.nw);
 }
 
 // The plan's inactive particles take k_dem64_free's step results; their
@@ -1081,8 +1086,8 @@ __global__ void __launch_bounds__(128) k_dem64_commit(Params P) {
 // frame.  When no contact can occur during the step, the translation of the
 // n_s sub-steps under the constant force is taken in closed form (x += v +
 // a/2, v += a over the unit step: what the sub-steps compute in exact
-// arithmetic) and the rotation is sub-stepped by four FP64 lanes per
-// particle.  (Lattices stored below FP64 use k_dem32 instead.)
+// arithmetic) and the rotation is sub-stepped by four lanes per particle
+// (rotate_free_quad).  (Lattices stored below FP64 use k_dem32 instead.)
 __global__ void __launch_bounds__(256) k_dem(Params P) {
     const double h = 1.0 / P.n_sub;
     if (P.force_fixed) {
@@ -1115,7 +1120,7 @@ __global__ void __launch_bounds__(256) k_dem(Params P) {
             const unsigned mk = __ballot_sync(0xffffffffu, moving);
             const int ql = threadIdx.x & 3;
             if (moving)
-                rotate_free_quad(mk, P.parts[k], ql == 0 ? 0.0 : P.Th[3 * k + ql - 1], h, P.n_sub, P.parts[k].q,
+                rotate_free_quad(mk, P.parts[k], ql == 0 ? 0.0 : P.Th[3 * k + ql - 1], h, P.n_sub, P.rot_pairs, P.parts[k].q,
                                  P.parts[k].w);
         }
         return;

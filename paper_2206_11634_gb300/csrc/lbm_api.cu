@@ -299,6 +299,7 @@ Params make_params(lbm_handle *h) {
     P.wall_xi_f = at<float>(h, h->L.wall_xi_f);
     P.wall_xcw_f = at<float>(h, h->L.wall_xcw_f);
     P.dem_mode = h->dem_mode;
+    P.rot_pairs = c.dem_mode != LBM_DEM_FP64_ALL;
     P.dem_list = at<int>(h, h->L.dem_list);
     P.fc_valid = h->fc_valid;
     P.plain_grid = h->plain_per_sm > 0 ? h->plain_per_sm * h->nsm : 0;

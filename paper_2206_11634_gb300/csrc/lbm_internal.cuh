@@ -364,6 +364,7 @@ struct Params {
     int near_expected;        // near bricks expected (an upper estimate from the particles' extent)
     int idx32;                // Q N < 2^31: population indices fit 32 bits
     int dem_mode;             // enum DemKernel: which DEM kernels run
+    int rot_pairs;            // free rotation may run in FP32 pairs (not with LBM_DEM_FP64_ALL)
     int fc_valid;             // Fc/Tc hold the contact load of the current state (0 after set_particles)
     double tau, rho0, c0;
     double F[3], g[3], u0[3];
