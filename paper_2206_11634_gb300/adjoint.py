@@ -12,6 +12,11 @@ flags frozen, wrapped as a torch.autograd.Function.
 
 Marshalling only: the forward run, the adjoint and the chain rule to the
 control points all run on the GPU.
+
+Memory: keep_steps=True keeps what the backward run needs of every step (16 bytes
+per node and step); False keeps states every sqrt(T) steps and runs the steps
+between them twice (96^3, T = 500: 41 ms instead of 28).  By default every step is kept if that takes
+8 GiB at most and an eighth of the memory that is free on the device.
 """
 from __future__ import annotations
 
@@ -24,7 +29,7 @@ from .lbm import LbmConfig, LbmError, LbmParticle, load_library, make_config
 
 class AdjointDrag:
     def __init__(self, nx: int, ny: int, nz: int, *, particle: LbmParticle, T: int, W: int, device: str = "cuda",
-                 stream=None, **kw):
+                 stream=None, keep_steps: bool | None = None, **kw):
         import torch
 
         if not torch.cuda.is_available():
@@ -38,10 +43,20 @@ class AdjointDrag:
         self.T, self.W = int(T), int(W)
         self.device = torch.device(device)
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
-        size = C.c_size_t()
-        self._ok(self.L.lbm_adj_workspace_size(C.byref(self.cfg), C.byref(particle), self.T, self.W, C.byref(size)),
-                 None)
-        self.ws = torch.empty(size.value, dtype=torch.uint8, device=self.device)
+        least, keep = C.c_size_t(), C.c_size_t()
+        self._ok(self.L.lbm_adj_workspace_sizes(C.byref(self.cfg), C.byref(particle), self.T, self.W, C.byref(least),
+                                                C.byref(keep)), None)
+        choose = keep_steps is None
+        if choose:
+            keep_steps = keep.value <= min(8 << 30, torch.cuda.mem_get_info(self.device)[0] // 8)
+        size = keep if keep_steps else least
+        try:
+            self.ws = torch.empty(size.value, dtype=torch.uint8, device=self.device)
+        except torch.cuda.OutOfMemoryError:  # a limit on this process
+            if not choose:
+                raise
+            size = least
+            self.ws = torch.empty(size.value, dtype=torch.uint8, device=self.device)
         h = C.c_void_p()
         with torch.cuda.device(self.device):
             rc = self.L.lbm_adj_init(C.byref(self.cfg), C.byref(particle), self.T, self.W,

@@ -32,8 +32,9 @@
 // moments of the pulled values (16 bytes, instead of a whole state of 76 and
 // a second gather with its link values) and nine partial derivatives per link
 // (by reverse differentiation of the VIBB value, where the value is formed).
-// Runs whose kept steps would exceed kKeepAllBytes keep a state every
-// ceil(sqrt(T)) steps instead and run each segment forward again from it.
+// A workspace too small for every step's (lbm_adj_workspace_sizes) keeps a
+// state every ceil(sqrt(T)) steps instead, and each segment is run forward again
+// from it.
 //
 // A step, forward or adjoint, is two kernels on disjoint nodes in programmatic
 // dependent launches, ordered as the fixed-geometry sweep's (k_static.cuh): one
@@ -833,13 +834,12 @@ void classify_links(const lbm_config *c, const lbm_particle *p, Links &k) {
         if (f2 >= 0 && k.kind[(size_t)f2] == kPlain) k.kind[(size_t)f2] = kShared;
 }
 
-// Kept data of every step up to this much (a thirty-fifth of the GPU's
-// memory; 96^3 keeps 600 steps): the adjoint then runs no forward step again.
-// Larger runs keep a state every ceil(sqrt(T)) steps and one segment's data.
-constexpr size_t kKeepAllBytes = (size_t)8 << 30;
-
-void adj_layout(lbm_adj *a) {
+// keep_all: room for every step's kept data (96^3: 14.5 MB a step), so that the
+// adjoint runs no forward step again; else a state every ceil(sqrt(T)) steps
+// and one segment's data.
+void adj_layout(lbm_adj *a, bool keep_all) {
     size_t o = 0;
+    a->keep_all = keep_all;
     auto take = [&](size_t bytes) {
         size_t at = o;
         o = align_up(o + bytes);
@@ -886,7 +886,6 @@ void adj_sizes(lbm_adj *a, const lbm_config *c, int T, int W, int ncp, const Lin
     a->S = align_up((size_t)Q * (size_t)a->N * 4);
     const size_t L = (size_t)std::max(1, a->nlinks);
     a->kept = align_up((size_t)a->N * 16) + 2 * align_up(L * 16) + align_up(L * 4);
-    a->keep_all = a->kept <= kKeepAllBytes / (size_t)T;
 }
 
 AdjDev adj_dev(lbm_adj *a) {
@@ -984,16 +983,24 @@ void adjoint_step(lbm_adj *a, AdjDev D, const X &...x) {
 
 extern "C" {
 
-int lbm_adj_workspace_size(const lbm_config *cfg, const lbm_particle *p, int T, int W, size_t *bytes) {
+int lbm_adj_workspace_sizes(const lbm_config *cfg, const lbm_particle *p, int T, int W, size_t *least, size_t *keep) {
     if (const char *m = adj_check(cfg, p, T, W)) return afail(nullptr, LBM_ERR_BAD_ARG, "%s", m);
-    if (!bytes) return afail(nullptr, LBM_ERR_BAD_ARG, "bytes is NULL");
+    if (!least || !keep) return afail(nullptr, LBM_ERR_BAD_ARG, "least or keep is NULL");
     Links k;
     classify_links(cfg, p, k);
     lbm_adj a;
     adj_sizes(&a, cfg, T, W, p->n_cp, k);
-    adj_layout(&a);
-    *bytes = a.total;
+    adj_layout(&a, true);
+    *keep = a.total;
+    adj_layout(&a, false);
+    *least = std::min(a.total, *keep);  // (a short run's steps may take less than its checkpoints)
     return LBM_OK;
+}
+
+int lbm_adj_workspace_size(const lbm_config *cfg, const lbm_particle *p, int T, int W, size_t *bytes) {
+    size_t keep;
+    if (!bytes) return afail(nullptr, LBM_ERR_BAD_ARG, "bytes is NULL");
+    return lbm_adj_workspace_sizes(cfg, p, T, W, bytes, &keep);
 }
 
 int lbm_adj_init(const lbm_config *cfg, const lbm_particle *p, int T, int W, void *dev_ws, size_t ws_bytes,
@@ -1008,9 +1015,12 @@ int lbm_adj_init(const lbm_config *cfg, const lbm_particle *p, int T, int W, voi
     lbm_adj *a = new (std::nothrow) lbm_adj();
     if (!a) return afail(nullptr, LBM_ERR_BAD_ARG, "out of host memory");
     adj_sizes(a, cfg, T, W, p->n_cp, k);
-    adj_layout(a);
+    // every step's kept data if there is room
+    adj_layout(a, true);
+    const size_t keep = a->total;
+    if (ws_bytes < keep) adj_layout(a, false);
     if (ws_bytes < a->total) {
-        const size_t need = a->total;
+        const size_t need = std::min(a->total, keep);
         delete a;
         return afail(nullptr, LBM_ERR_WS_TOO_SMALL, "workspace of %zu bytes, %zu needed", ws_bytes, need);
     }
