@@ -42,7 +42,7 @@ constexpr int kNearCtasPerSm = 2;
 // registers at 4) 420 / 357 / 320 before the lists were culled and 248 after, 128
 // threads at 4 / 6 / 8 CTAs 238 / 246 / 318; 50 settled in 128x128x256 117 and 94;
 // one there 15.9 / 17.8 / 18.1 at 2 / 3 / 4; FP64 at 1 / 2: one sphere in 32x32x48
-// 43 / 60, 25 metaballs in 128^3 451 / 413.
+// 43 / 60, 25 metaballs in 128^3 440 / 262.
 template <typename S, bool kMany>
 constexpr int kNearThreads = sizeof(S) != 8 && kMany ? BRICK / 2 : BRICK;
 template <typename S, bool kMany>

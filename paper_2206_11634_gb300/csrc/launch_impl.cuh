@@ -63,10 +63,13 @@ void launch_sweep_near_n(const Params &P, cudaStream_t st) {
 }
 template <typename S>
 void launch_sweep_near_t(const Params &P, cudaStream_t st) {
-    // FP64 is bound by one brick's FP64 instructions while each SM has at most
-    // one of them; the others' turning point lies between the 2700 bricks
-    // expected for 12 metaballs (two CTAs faster) and the 11600 for 50
-    const int many = sizeof(S) == 8 ? sm_count() + 1 : 40 * sm_count();
+    // The form by the near bricks expected, where a step's time turns (us a
+    // step, few and many): FP32 128x128x256, 3144 bricks 165 and 168, 3848 175
+    // and 174, 4376 186 and 179, 9306 219 and 208; 192^3 4376 237 and 229; 256^3
+    // 4392 514 and 514, 6424 531 and 522; FP16 alike (3144: 140 and 142, 4376: 156
+    // and 150).  FP64, the near sweep by itself: 168 bricks 57 and 72, 504 165 and
+    // 191, 1658 195 and 205, 2090 255 and 205, 4112 440 and 262.
+    const int many = (sizeof(S) == 8 ? 12 : 26) * sm_count();
     if (P.near_expected >= many) launch_sweep_near_n<S, true>(P, st);
     else launch_sweep_near_n<S, false>(P, st);
 }

@@ -82,8 +82,11 @@ constexpr int kDefaultPlainPerSm = 0;
 // Batched lattices: CTAs per case of the flag and near sweeps, bricks per CTA
 // of the plain sweep (lbm_batch_tune chooses them by measurement).
 constexpr int kDefaultBatchChainCtas = 4;
-// 64 boxes of sides 48-128, ms a step with 1 / 2 / 4 / 8 spans a CTA: FP32
-// 1.487 / 1.453 / 1.485 / 1.541, FP16 1.193 / 1.103 / 1.081 / 1.076.
+// us a step with 1 / 2 / 4 / 8 spans a CTA: 64 boxes of sides 48-128, FP32 1572 /
+// 1527 / 1515 / 1530, FP16 1113 / 1081 / 1064 / 1069; 8 boxes of 48-128, FP32 165 /
+// 160 / 162 / 165, FP16 121 / 115 / 112 / 112; 8 of 64-96, FP32 122 / 120 / 121 / 127, FP16
+// 91 / 86 / 84 / 85; one of 64, FP16 15.1 / 13.7 / 12.3 / 15.2; two of 48, FP16 14.9 /
+// 11.0 / 11.3 / 14.4.
 constexpr int kDefaultBatchPlainChunk = 2, kDefaultBatchPlainChunk16 = 4;
 constexpr int kDefaultChainPerSm = 0;
 

@@ -3,8 +3,8 @@ and box sides that are no multiples of the 32x4x2 bricks: the rows of those
 bricks start and end at a wall (and, ragged, inside the brick).  One step
 against the oracle, with the tolerances of tests/test_gpu_parity.py.
 
-"corners" has a few near bricks; "filled" lets 7680 be expected, more than 40 per
-SM, which the near sweep's other form takes."""
+"corners" has a few near bricks; "filled" lets 7680 be expected, some 50 per SM,
+which the near sweep's other form takes."""
 import itertools
 
 import numpy as np
