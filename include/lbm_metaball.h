@@ -188,7 +188,7 @@ int lbm_set_particles(lbm_handle *h, const lbm_particle *host, int n);
  * do not replay one.  When every particle is fixed (fixed = 1) the geometry
  * cannot change, and from the fourth step after lbm_set_particles() on the
  * flag pass (§2.3.1, §2.3.3) is left out: its result would be the same.
- * Lattices below FP64 then run two kernels per step on the high-priority
+ * Lattices below FP64 then run two kernels per step on the low-priority
  * stream alone, each launched while the one before still runs (programmatic
  * dependent launch). */
 int lbm_step(lbm_handle *h, int nsteps);

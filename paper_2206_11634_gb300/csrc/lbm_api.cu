@@ -852,13 +852,18 @@ int lbm_step(lbm_handle *h, int nsteps) {
     if (nsteps < 0) return fail(h, LBM_ERR_BAD_ARG, "nsteps < 0");
     if (nsteps == 0) return LBM_OK;
     // fork: the library streams start after everything issued so far (aux
-    // with the first step that uses it: the fixed-geometry sweep does not)
+    // with the first step that uses it)
     cudaError_t e = cudaEventRecord(h->ev_fork, h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->hi, h->ev_fork, 0);
     if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
     cudaStream_t hs = h->hi;
     bool forked_aux = false;  // aux carries work of this call
-    bool plain_pending = false;  // ... that hs has not waited for
+    bool on_aux = false;      // ... and all of it by now: the fixed-geometry steps
+    const auto fork_aux = [&] {
+        if (forked_aux) return cudaSuccess;
+        forked_aux = true;
+        return cudaStreamWaitEvent(h->aux, h->ev_fork, 0);
+    };
     for (int t = 0; t < nsteps; t++) {
         Params P = make_params(h);
         // with every particle fixed the flags cannot change: once both flag
@@ -872,7 +877,7 @@ int lbm_step(lbm_handle *h, int nsteps) {
         const int rp = (int)(h->steps & 1);
         const size_t region = bin_region(h, h->steps);
         if (!h->bin_clean[rp]) {
-            e = cudaMemsetAsync(h->ws + region, 0, h->L.bin_bytes, hs);
+            e = cudaMemsetAsync(h->ws + region, 0, h->L.bin_bytes, on_aux ? h->aux : hs);
             if (e != cudaSuccess) return cuda_check(h, e, "cudaMemsetAsync(bricks)");
         }
         h->bin_clean[rp] = 0;
@@ -912,28 +917,28 @@ int lbm_step(lbm_handle *h, int nsteps) {
         }
         if (fixed_sweep && h->static_state == 1) {
             // the plain nodes and beside them the link nodes, in stream order
-            // (k_static.cuh); behind the plain sweep of a brick step
-            if (plain_pending) {
-                e = cudaStreamWaitEvent(hs, h->ev_plain, 0);
-                if (e != cudaSuccess) return cuda_check(h, e, "stream wait");
-                plain_pending = false;
+            // (k_static.cuh), on the low-priority stream, as most of a step's
+            // work always is: behind what hs carries
+            if (!on_aux) {
+                e = fork_aux();
+                if (e == cudaSuccess) e = cudaEventRecord(h->ev_near, hs);
+                if (e == cudaSuccess) e = cudaStreamWaitEvent(h->aux, h->ev_near, 0);
+                if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
+                on_aux = true;
             }
             for (int k = 0; k < 2; k++) {
                 const bool links = (P.links_first != 0) == (k == 0);
-                ProfScope s(h, links ? 3 : 2, true, hs);
-                if (links) by_storage<DoStaticLinks>(h->cfg.storage, P, hs);
-                else by_storage<DoStaticPlain>(h->cfg.storage, P, hs);
+                ProfScope s(h, links ? 3 : 2, true, h->aux);
+                if (links) by_storage<DoStaticLinks>(h->cfg.storage, P, h->aux);
+                else by_storage<DoStaticPlain>(h->cfg.storage, P, h->aux);
             }
             // the plain kernel cleared the next region's counters and force
             // totals (the brick counts are only written by brick steps, which
             // do not follow before the particles are set again)
             h->bin_clean[rp ^ 1] = 1;
         } else {
-            if (!forked_aux) {
-                e = cudaStreamWaitEvent(h->aux, h->ev_fork, 0);
-                if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
-                forked_aux = true;
-            }
+            e = fork_aux();
+            if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
             // after fixed-geometry steps, which bin nothing
             if (h->bin_step != h->steps - 1) launch_relist(P, (int)h->flag_step, hs);
             { ProfScope s(h, 0, true, hs); launch_bin(P, hs); }
@@ -978,10 +983,10 @@ int lbm_step(lbm_handle *h, int nsteps) {
                 e = cudaEventRecord(h->ev_plain, h->aux);
                 if (e != cudaSuccess) return cuda_check(h, e, "event record");
             }
-            plain_pending = true;
         }
         if (!P.force_fixed) { ProfScope s(h, 4, P.np > 0, hs); launch_force_reduce(P, hs); }
-        { ProfScope s(h, 5, P.np > 0 && P.n_sub > 0, hs); launch_dem(P, hs, h->dem2, h->ev_dsplit, h->ev_dfree); }
+        cudaStream_t ds = on_aux ? h->aux : hs;
+        { ProfScope s(h, 5, P.np > 0 && P.n_sub > 0, ds); launch_dem(P, ds, h->dem2, h->ev_dsplit, h->ev_dfree); }
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_check(h, e, "kernel launch");
         h->cur ^= 1;
@@ -994,7 +999,8 @@ int lbm_step(lbm_handle *h, int nsteps) {
     // plain sweep
     e = cudaEventRecord(h->ev_join, hs);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->ev_join, 0);
-    if (e == cudaSuccess && forked_aux) e = cudaStreamWaitEvent(h->stream, h->ev_plain, 0);
+    if (e == cudaSuccess && on_aux) e = cudaEventRecord(h->ev_plain, h->aux);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->ev_plain, 0);
     if (e != cudaSuccess) return cuda_check(h, e, "stream join");
     return LBM_OK;
 }

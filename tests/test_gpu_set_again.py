@@ -91,3 +91,25 @@ def test_batch(pkg, storage, held):
                 assert np.array_equal(bt.populations(c).cpu().numpy(), lat.populations().cpu().numpy())
                 for x, y in zip(bt.forces(c), lat.forces()):
                     assert np.array_equal(x, y)
+
+
+def test_held_particles_with_dem_sub_steps(pkg):
+    """The DEM runs behind the fixed-geometry kernels of each step: two held
+    spheres that overlap have the contact load of the first step (brick sweeps) in
+    every later one (FP32 contact geometry, its overlap to 1e-6 of 0.5), and the
+    flow keeps the bits of a run without DEM."""
+    pops = []
+    for n_sub in (0, 10):
+        lat = pkg.Lattice(40, 40, 40, n_sub=n_sub, kn=100.0, kt=50.0, **KW)
+        lat.set_populations(flow(19, 40))
+        lat.set_particles([pkg.make_particle([[0, 0, 0]], [16.0], (14.0 + 9.5 * k, 20.0, 20.0), Rs=1.0, fixed=1,
+                                             mass=100.0, inertia=np.eye(3) * 1e3) for k in range(2)])
+        load = []
+        for steps in (1, 1, 7, 1, 5):
+            lat.step(steps)
+            load.append(lat.contact_forces()[0])
+        pops.append(lat.populations().cpu().numpy())
+        assert (np.abs(load[0][:, 0]).min() > 1.0) == (n_sub > 0)
+        for F in load:
+            assert np.abs(F - load[0]).max() <= 1e-5 * np.abs(load[0]).max()
+    assert np.array_equal(*pops)
