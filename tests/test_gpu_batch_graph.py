@@ -1,0 +1,48 @@
+"""A batch whose recorded geometry does not fit (one box crowded with spheres)
+keeps the brick sweeps: sixteen steps at a time as replays of a captured graph, the
+rest launched directly, with the step numbers in device counters.  Expected, to
+the bit: each box stepped alone with particles not declared fixed, whatever the
+split of the steps into calls, and after new poses."""
+import itertools
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from tests.test_gpu_set_again import pkg  # noqa: E402,F401
+
+KW = dict(periodic=(1, 1, 1), tau=0.7, force=(1e-5, 0.0, -2e-6), n_sub=0)
+
+
+def crowd(pkg, n, per_axis, radius, shift, fixed):  # noqa: F811
+    at = (np.arange(per_axis) + 0.5) * n / per_axis
+    return [pkg.make_particle([[0, 0, 0]], [radius * radius], np.array(c) + shift, v=(0.004, 0.0, -0.002), fixed=fixed,
+                              mass=50.0, inertia=np.eye(3) * 400.0) for c in itertools.product(at, at, at)]
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("calls", [(1, 20, 16, 33), (40, 1, 16), (3, 16, 48), (70,)])
+def test_brick_steps_of_a_crowded_batch(pkg, storage, calls):  # noqa: F811
+    boxes = [(40, 3, 5.2), (45, 1, 6.0)]  # 27 spheres (more than 16 384 links), one sphere
+    batch = pkg.Batch([dict(nx=n, ny=n, nz=n, storage=storage, max_particles=k ** 3, **KW) for n, k, _ in boxes])
+    single = [pkg.Lattice(n, n, n, storage=storage, max_particles=k ** 3, **KW) for n, k, _ in boxes]
+    alone = pkg.Lattice(40, 40, 40, storage=storage, max_particles=27, **KW)
+    alone.set_particles(crowd(pkg, *boxes[0], 0.0, 1))
+    alone.step(5)
+    assert b"brick sweeps kept" in alone.L.lbm_last_error(alone.h)
+    for shift in (0.0, (0.7, 3.1, 2.4)):
+        for c, box in enumerate(boxes):
+            batch.set_particles(c, crowd(pkg, *box, shift, 1))
+            single[c].set_particles(crowd(pkg, *box, shift, 0))
+        for steps in calls:
+            batch.step(steps)
+            for c, lat in enumerate(single):
+                lat.step(steps)
+                assert np.array_equal(batch.populations(c).cpu().numpy(), lat.populations().cpu().numpy())
+                for x, y in zip(batch.forces(c), lat.forces()):
+                    assert np.array_equal(x, y)
