@@ -529,12 +529,12 @@ struct BrickRange {
 
 __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
-__device__ __forceinline__ BrickRange brick_range(const Params &P, const DevParticle &p, int a, double grow = 1.0) {
+__device__ __forceinline__ BrickRange brick_range(const Params &P, const DevParticle &p, int a) {
     const int B = a == 0 ? BX : (a == 1 ? BY : BZ);
     const int nb = a == 0 ? P.nbx : (a == 1 ? P.nby : P.nbz);
     const int L = dim_of(P, a);
-    int nlo = (int)floor(p.lo[a] - grow - 1e-6);
-    int nhi = (int)ceil(p.hi[a] + grow + 1e-6);
+    int nlo = (int)floor(p.lo[a] - 1.0 - 1e-6);
+    int nhi = (int)ceil(p.hi[a] + 1.0 + 1e-6);
     BrickRange r;
     r.all = false;
     if (P.per[a]) {
