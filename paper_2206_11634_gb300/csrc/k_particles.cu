@@ -27,34 +27,29 @@ namespace lbmmb {
 // An upper bound of M over the brick grown by one node, from each control
 // point's distance to that box (periodic: |minimum image of x - c| is at least
 // that of the box's centre less half its extent), with a hundredth of a node,
-// 2^-16 of the distance and a thousandth of M for the FP32 rounding.  A control
-// point many box lengths away is brought back as an FP32 pair before the one
-// rounding (the shift is an exact integer below 2^24; farther ones reach every
-// brick), and 2^-20 of the shift covers the FP32 positions of the sweeps, which
-// are rounded before.
+// 2^-16 of the distance and a thousandth of M for the FP32 rounding.  (A control
+// point more than 2^14 nodes away reaches every brick: its position is rounded
+// before it is brought back into the box, by a thousandth of a node there.)
 __device__ __forceinline__ bool brick_reached(const Params &P, const DevParticle &p, int bxi, int byi, int bzi) {
     const float org[3] = {(float)(bxi * BX), (float)(byi * BY), (float)(bzi * BZ)};
     const float half[3] = {0.5f * (BX - 1), 0.5f * (BY - 1), 0.5f * (BZ - 1)};
     float M = 0.f;
+    bool far = false;
     for (int k = 0; k < p.ncp; k++) {
         float d2 = 0.f;
         for (int a = 0; a < 3; a++) {
-            float m = df_minus_int(p.cpw_hl[k][a], org[a]) - half[a], slack = 1.01f;
+            float m = df_minus_int(p.cpw_hl[k][a], org[a]) - half[a];
             if (P.per[a]) {
-                const float shift = P.dim_f[a] * rintf(m * P.inv_n_f[a]);
-                if (!(fabsf(shift) < 8388608.f)) return true;
-                if (shift != 0.f) {
-                    m = df_minus_int(p.cpw_hl[k][a], org[a] + shift) - half[a];
-                    slack += fabsf(shift) * (1.0f / (1 << 20));
-                }
+                far |= !(fabsf(m) <= 16384.f);
+                m -= P.dim_f[a] * rintf(m * P.inv_n_f[a]);
             }
-            const float d = fmaxf(fabsf(m) * (1.0f - 1.0f / 65536.0f) - (half[a] + slack), 0.f);
+            const float d = fmaxf(fabsf(m) * (1.0f - 1.0f / 65536.0f) - (half[a] + 1.01f), 0.f);
             d2 += d * d;
         }
         M += p.K_f[k] / d2;
     }
     // (NaN: reached; so is everything at thresholds near FP32's range)
-    return !(M * 1.001f < P.c0_f) || !(P.c0_f > 1e-30f && P.c0_f < 1e30f);
+    return far || !(M * 1.001f < P.c0_f) || !(P.c0_f > 1e-30f && P.c0_f < 1e30f);
 }
 __device__ void bin_particle(const Params &P, int j) {
     const int t = threadIdx.x;
