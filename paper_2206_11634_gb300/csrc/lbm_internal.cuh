@@ -367,7 +367,6 @@ struct Params {
     int near_expected;        // near bricks expected (an upper estimate from the particles' extent)
     int idx32;                // Q N < 2^31: population indices fit 32 bits
     int dem_mode;             // enum DemKernel: which DEM kernels run
-    int rot_pairs;            // free rotation may run in FP32 pairs (not with LBM_DEM_FP64_ALL)
     int fc_valid;             // Fc/Tc hold the contact load of the current state (0 after set_particles)
     double tau, rho0, c0;
     double F[3], g[3], u0[3];
@@ -434,6 +433,7 @@ struct Params {
     int *status;       // [ST_SLOTS], sticky error bits
     StepGate gate;     // fixed-geometry sweep
     int links_first;   // ... the order of its two kernels
+    int rot_pairs;     // free rotation may run in FP32 pairs (not with LBM_DEM_FP64_ALL)
     int *counters;     // per-step counters, zeroed with the brick lists
     // fixed-geometry sweep (every particle fixed, lattices below FP64): built
     // once by k_static_build, then every step runs k_static_plain over the
