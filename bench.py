@@ -628,8 +628,8 @@ GRADIENT_MAX = 8
 def run_gradient(args):
     """Workload 4: d(mean drag)/d(control points, weights) of one fixed
     six-control-point metaball in a periodic 96^3 box, T = 500 steps, window
-    W = 100, through the library's hand-written adjoint (flags frozen, sqrt(T)
-    checkpoints).  A "step" here is one gradient evaluation (forward run and
+    W = 100, through the library's hand-written adjoint (flags frozen; every
+    step's data kept, or sqrt(T) checkpoints in little memory).  A "step" here is one gradient evaluation (forward run and
     backward run); value = lattice updates of the objective (N x T per
     gradient) per second of forward plus backward time."""
     import torch
@@ -713,7 +713,7 @@ def run_gradient(args):
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": f"drag_gradient_{ncp}cp_{case['nx']}^3", "lattice": "D3Q19", "storage": "f32",
                        "T": T, "W": case["W"], "tau": case["tau"], "links": info["nlinks"],
-                       "checkpoint_every": info["checkpoint_every"], "step": "one gradient (forward + backward)",
+                       "checkpoint_every": None if eng.keeps_steps else info["checkpoint_every"], "step": "one gradient (forward + backward)",
                        "forward_ms": round(ms_f / grads, 3), "backward_ms": round(ms_b / grads, 3),
                        "l2": "no flush: two FP32 population arrays of 67 MB each, about the 129 MB L2",
                        "parallelism": f"replicas x{world}"},
@@ -724,10 +724,10 @@ def run_gradient(args):
                          "kernel": "forward step (k_adj_step)", "bytes_per_launch": alg,
                          "avg_launch_us": round(step_s * 1e6, 3)},
             "gradient": {"dJ_dK": [float(f"{v:.6e}") for v in g_K]},
-            # per gradient: q and the initial state, T forward steps; T - C
-            # recomputed steps (C checkpoints), three adjoint kernels per step
-            # and the chain rule to the shape
-            "gpu_launches": grads * (2 + T + (T - -(-T // info["checkpoint_every"])) + 3 * T + 1),
+            # per gradient: q and the initial state, two kernels per forward
+            # and per adjoint step (and per step run again from checkpoints),
+            # the chain rule to the shape
+            "gpu_launches": grads * (2 + 2 * T + (0 if eng.keeps_steps else 2 * T) + 2 * T + 1),
             "clocks": clocks.summary(), "cpu_baseline": cpu}
     print(json.dumps(line), flush=True)
     if dist is not None:

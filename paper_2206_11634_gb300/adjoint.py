@@ -57,6 +57,7 @@ class AdjointDrag:
                 raise
             size = least
             self.ws = torch.empty(size.value, dtype=torch.uint8, device=self.device)
+        self.keeps_steps = size.value >= keep.value
         h = C.c_void_p()
         with torch.cuda.device(self.device):
             rc = self.L.lbm_adj_init(C.byref(self.cfg), C.byref(particle), self.T, self.W,
