@@ -238,7 +238,8 @@ int lbm_get_counters(lbm_handle *h, int64_t *steps, int32_t *nrefill, int32_t *n
  * kernels that run beside it; 0 = one CTA per brick).  chain_ctas_per_sm:
  * CTAs per SM of the persistent flag and near-brick sweeps (1..4; 0 = the
  * default).  Takes effect from the next lbm_step(); results do not depend on
- * it.  Defaults: 0 and 0 (one plain CTA per brick, 4 flag/near CTAs per SM). */
+ * it.  Defaults: 0 and 0 (one plain CTA per brick, 4 flag CTAs per SM, near
+ * CTAs by the bricks expected: 2 per SM, or 4 of half the threads for many). */
 int lbm_set_schedule(lbm_handle *h, int plain_ctas_per_sm, int chain_ctas_per_sm);
 
 /* Whether the plain sweep issues a brick's 19 pulls before it has read that
@@ -347,7 +348,10 @@ int lbm_batch_init(const lbm_config *cfgs, int ncases, void *dev_ws, size_t ws_b
  * Synchronises. */
 int lbm_batch_set_particles(lbm_batch *b, int c, const lbm_particle *host, int n);
 
-/* Advance every case by nsteps steps (asynchronous on the batch's stream). */
+/* Advance every case by nsteps steps (asynchronous on the batch's stream).  The
+ * parity of fixed-geometry steps comes from the host: a CUDA graph captured
+ * from the batch's stream may be replayed if it holds an even number of them
+ * (lbm_batch_steps counts captured steps once). */
 int lbm_batch_step(lbm_batch *b, int nsteps);
 
 /* Synchronise and copy out the hydrodynamic force and torque of case c's

@@ -340,18 +340,20 @@ __global__ void k_set_pop(Params P, S *f, const double *in) {
 // a node's memory traffic (FP32 D3Q19: 76 B in, 34 B out) takes 5.2 of those
 // cycles.  The sums as FP64 additions of converted values (about 130 FP64
 // instructions a node) took 3.77 ms at 256^3.  So below FP64 storage the sums
-// run in FP32, exactly, and nine FP64 instructions are left: the density's sum
+// run in FP32, in parts that add up exactly (all but 2^-54), and nine FP64 instructions are left: the density's sum
 // with rho0 and the division.  Measured at 256^3, FP32, the call: 3.77 ->
 // 0.56 ms (one 64-bit integer per value instead of the three FP32 parts
 // below: 0.87).
 //
-// Exact sums: with 2^(E - 126) above the node's largest magnitude, adding and
+// The sums: with 2^(E - 126) above the node's largest magnitude, adding and
 // taking off 1.5 2^23 u rounds a value to a multiple of u, so a value splits
 // exactly into a multiple of u1 = 2^(E - 145) (at most 2^19 of them), one of
 // u2 = 2^-20 u1 (at most 2^19) and a rest of at most u2 / 2 (Rump, Ogita and
 // Oishi's extraction, SIAM J. Sci. Comput. 31, 2008).  Q <= 19 such multiples
-// add up exactly in FP32 in any order; the rests' sum is off by 2^-24 of
-// itself at most, under 2^-60 of the largest value.
+// add up exactly in FP32 in any order.  The rests, up to 2^(E - 166) each, add up
+// with 18 roundings of up to 2^(E - 186), and their sum is rounded to u3 =
+// 2^(E - 182): together under 2^(E - 181), 2^-54 of the largest value, which is
+// 2^(E - 127) at least (a single FP64 sum's roundings are 18 of 2^-53 of it).
 // ---------------------------------------------------------------------------
 constexpr int kFieldEmin = 56, kFieldEmax = 240;  // the exponent fields E that the units stay normal for
 __device__ __forceinline__ float exp2_field(int e) { return __uint_as_float((uint32_t)e << 23); }  // 2^(e - 127)

@@ -46,3 +46,28 @@ def test_brick_steps_of_a_crowded_batch(pkg, storage, calls):  # noqa: F811
                 assert np.array_equal(batch.populations(c).cpu().numpy(), lat.populations().cpu().numpy())
                 for x, y in zip(batch.forces(c), lat.forces()):
                     assert np.array_equal(x, y)
+
+
+def test_captured_fixed_steps_replay(pkg):  # noqa: F811
+    """An even number of fixed-geometry steps in a caller's own graph: five
+    replays are ten steps."""
+    stream = torch.cuda.Stream()
+    runs = []
+    for captured in (True, False):
+        b = pkg.Batch([dict(nx=n, ny=n, nz=n, storage="f32", max_particles=1, **KW) for n in (32, 45)], stream=stream)
+        for c, n in enumerate((32, 45)):
+            b.set_particles(c, crowd(pkg, n, 1, 5.0, 0.3, 1))
+        b.step(6)
+        torch.cuda.synchronize()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                b.step(2)
+            for _ in range(5):
+                graph.replay()
+        else:
+            b.step(10)
+        torch.cuda.synchronize()
+        runs.append([x for c in range(2) for x in (b.populations(c).cpu().numpy(), *b.forces(c))])
+    for x, y in zip(*runs):
+        assert np.array_equal(x, y)
