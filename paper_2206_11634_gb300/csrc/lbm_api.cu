@@ -940,7 +940,7 @@ int lbm_step(lbm_handle *h, int nsteps) {
             e = fork_aux();
             if (e != cudaSuccess) return cuda_check(h, e, "stream fork");
             // after fixed-geometry steps, which bin nothing
-            if (h->bin_step != h->steps - 1) launch_relist(P, (int)h->flag_step, hs);
+            if (h->bin_step < h->steps - 1) launch_relist(P, (int)h->flag_step, hs);
             { ProfScope s(h, 0, true, hs); launch_bin(P, hs); }
             h->bin_step = h->steps;
             h->bin_clean[rp ^ 1] = 1;

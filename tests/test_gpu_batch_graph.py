@@ -71,3 +71,22 @@ def test_captured_fixed_steps_replay(pkg):  # noqa: F811
         runs.append([x for c in range(2) for x in (b.populations(c).cpu().numpy(), *b.forces(c))])
     for x, y in zip(*runs):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("held", [3, 4, 5, 6])  # 4: the step that tries to record the geometry is the last
+def test_crowded_lattice_set_again(pkg, held):  # noqa: F811
+    """A single lattice whose geometry does not fit: new poses right after the
+    step that found so, and around it, against particles not declared fixed."""
+    runs = []
+    for fixed in (1, 0):
+        lat = pkg.Lattice(40, 40, 40, storage="f32", max_particles=27, **KW)
+        out = []
+        for shift in (0.0, (0.7, 4.1, 5.4), (0.2, 1.3, 2.0)):
+            lat.set_particles(crowd(pkg, 40, 3, 5.2, shift, fixed))
+            for steps in (1, held - 1):
+                lat.step(steps)
+                out += [lat.populations().cpu().numpy(), lat.flags().cpu().numpy(), *lat.forces(),
+                        lat.counters()["nrefill"]]
+        runs.append(out)
+    for x, y in zip(*runs):
+        assert np.array_equal(x, y)
